@@ -62,8 +62,7 @@ int launch_fold_partials(float* part, double* acc, int64_t n, cudaStream_t s) {
 }
 
 int64_t adjoint_slot_count(const KParams& p) {
-    Launch l = adjk::grid_of(p);
-    return (int64_t)l.grid.x * l.grid.y * adjk::kSlots;
+    return adjk::strided_blocks(p) * adjk::kSlots;
 }
 
 int launch_adjoint_seed(int vel, int storage, const void* P, const uint32_t* nbr, const float* w_rho,

@@ -42,21 +42,22 @@ using dev::kBlock;
 using dev::warp_sum;
 constexpr int kSlots = 5;         // gB[3], gtau, loss
 
-// Adds the block's sums of acc[kSlots] into slots[block * kSlots + k].
+// Adds the block's sums of acc[FIRST .. kSlots) into slots[block * kSlots + k].
+template <int FIRST = 0>
 __device__ __forceinline__ void block_accumulate(double* acc, double* __restrict__ slots, int64_t block) {
     __shared__ double sh[32][kSlots];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < kSlots; ++k) acc[k] = warp_sum(acc[k]);
+    for (int k = FIRST; k < kSlots; ++k) acc[k] = warp_sum(acc[k]);
     if (lane == 0) {
 #pragma unroll
-        for (int k = 0; k < kSlots; ++k) sh[wid][k] = acc[k];
+        for (int k = FIRST; k < kSlots; ++k) sh[wid][k] = acc[k];
     }
     __syncthreads();
     if (wid == 0) {
         const int nw = (blockDim.x + 31) / 32;
 #pragma unroll
-        for (int k = 0; k < kSlots; ++k) {
+        for (int k = FIRST; k < kSlots; ++k) {
             double v = lane < nw ? sh[lane][k] : 0.0;
             v = warp_sum(v);
             if (lane == 0) slots[block * kSlots + k] += v;
@@ -379,10 +380,12 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_seed(const typename S::T* __
                                                          const uint32_t* __restrict__ nbr,
                                                          const float* __restrict__ w_rho,
                                                          const float* __restrict__ w_j, float* __restrict__ lam,
-                                                         double* __restrict__ slots, int in_window, KParams p) {
-    Cell c;
+                                                         double* __restrict__ slots, int in_window, int chunks, KParams p) {
     double acc[kSlots] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    if (dev::cell_of_thread(p, c)) {
+    const int64_t tiles = (int64_t)p.ny * p.nz * chunks;
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        Cell c;
+        if (!dev::cell_at(p, (int)(t / chunks), (int)(t % chunks) * blockDim.x + threadIdx.x, c)) continue;
         const uint32_t m = nbr[c.cell];
         if (m & kSolidBit) {
 #pragma unroll
@@ -405,7 +408,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_seed(const typename S::T* __
                     jy += L::c(a, 1) * ha;
                     jz += L::c(a, 2) * ha;
                 }
-                acc[4] = (double)wr * (double)(p.rho0 + drho) + (double)wj[0] * jx + (double)wj[1] * jy +
+                acc[4] += (double)wr * (double)(p.rho0 + drho) + (double)wj[0] * jx + (double)wj[1] * jy +
                          (double)wj[2] * jz;
             }
             float lm[L::Q];
@@ -418,11 +421,15 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_seed(const typename S::T* __
             if (o) store_lam_links<L>(link_part(lam, p), o, __ldg(p.lbase + c.cell), lm);
         }
     }
-    block_accumulate(acc, slots, (int64_t)blockIdx.y * gridDim.x + blockIdx.x);
+    if (in_window) block_accumulate<4>(acc, slots, blockIdx.x);  // the loss only
 }
 
 // ---------------------------------------------------------------------------
 // One reverse step, general kernel: one thread per cell, direct global loads.
+// The blocks stride over the tiles (kAdjPerSm of them per SM) and reduce their
+// FP64 sums once at the end.  A reduction per 128 cells took the FP64 pipe
+// (two adds per cycle and SM) longer than the step itself: 0.095 ms on 1024^2
+// cells of D2V9 FP32, 0.112 ms inside the loss window.
 // ---------------------------------------------------------------------------
 template <class L, class S, int FORCE, bool EF, bool WIN>
 __global__ void __launch_bounds__(kBlock) k_adjoint_step(
@@ -430,10 +437,12 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_step(
     const float* __restrict__ lam_in,     // lam_{t+1}
     float* __restrict__ lam_out,          // lam_t
     const uint32_t* __restrict__ nbr, const float* __restrict__ Ef, const float* __restrict__ w_rho,
-    const float* __restrict__ w_j, float* __restrict__ gE, double* __restrict__ slots, KParams p) {
-    Cell c;
+    const float* __restrict__ w_j, float* __restrict__ gE, double* __restrict__ slots, int chunks, KParams p) {
     double acc[kSlots] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    if (dev::cell_of_thread(p, c)) {
+    const int64_t tiles = (int64_t)p.ny * p.nz * chunks;
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        Cell c;
+        if (!dev::cell_at(p, (int)(t / chunks), (int)(t % chunks) * blockDim.x + threadIdx.x, c)) continue;
         const uint32_t m = __ldg(nbr + c.cell);
         if (m & kSolidBit) {
 #pragma unroll
@@ -444,14 +453,16 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_step(
             dev::pull<L, S>(P, p, m, c, h);
             const uint32_t o = outgoing<L::Q>(m);
             const uint32_t lb = m ? __ldg(p.lbase + c.cell) : 0u;
-            const float* lamG_in = link_part(lam_in, p);
+            const float* lg = link_part(lam_in, p) + lb;
 #pragma unroll
             for (int a = 0; a < L::Q; ++a) {
                 h[a] *= p.inv_scale;
-                if (a != 0 && ((o >> a) & 1u))
-                    lt[a] = __ldg(lamG_in + link_slot(lb, o, a));
-                else
-                    lt[a] = __ldg(lam_in + dev::pop_at<L>(p, c, a, +1));
+                // x + e_a solid: the next link slot (address selected, as in pull)
+                const bool bounced = a != 0 && ((o >> a) & 1u);
+                const float* q = lam_in + dev::pop_at<L>(p, c, a, +1);
+                if (bounced) q = lg;
+                lg += bounced;
+                lt[a] = __ldg(q);
             }
             float E[3], wr, wj[3], lam[L::Q], gEc[3];
             load_E<L, EF>(Ef, p, c.cell, E);
@@ -471,7 +482,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_step(
             }
         }
     }
-    block_accumulate(acc, slots, (int64_t)blockIdx.y * gridDim.x + blockIdx.x);
+    block_accumulate(acc, slots, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -737,6 +748,17 @@ inline Launch grid_of(const KParams& p) {
     return l;
 }
 
+// Blocks of the general reverse kernels, and with them the gradient slots.
+constexpr int kAdjPerSm = 8;
+inline int64_t strided_blocks(const KParams& p) {
+    const Launch l = grid_of(p);
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t tiles = (int64_t)l.grid.x * l.grid.y, cap = (int64_t)(sms > 0 ? sms : 1) * kAdjPerSm;
+    return tiles < cap ? tiles : cap;
+}
+
 // GROUP 0: D2V9 and D3V19; GROUP 1: D3V27 and D1V3 (separate translation units)
 template <int GROUP, class F>
 int dispatch_lattice(int vel, F&& f) {
@@ -838,8 +860,8 @@ int seed_storage(int vel, const void* P, const uint32_t* nbr, const float* w_rho
     Launch l = grid_of(p);
     return dispatch_lattice<GROUP>(vel, [&](auto lat) {
         using L = decltype(lat);
-        k_adjoint_seed<L, S><<<l.grid, l.block, 0, s>>>((const typename S::T*)P, nbr, w_rho, w_j, lam, slots,
-                                                       in_window ? 1 : 0, p);
+        k_adjoint_seed<L, S><<<(unsigned)strided_blocks(p), l.block, 0, s>>>(
+            (const typename S::T*)P, nbr, w_rho, w_j, lam, slots, in_window ? 1 : 0, (int)l.grid.y, p);
         return 1;
     });
 }
@@ -849,7 +871,7 @@ int step_storage(int vel, int force, bool efield, bool in_window, const void* P,
                  float* lam_out, const uint32_t* nbr, const float* Ef, const float* w_rho, const float* w_j,
                  float* gE, double* slots, const KParams& p, cudaStream_t s) {
     Launch l = grid_of(p);
-    const int64_t slot_blocks = (int64_t)l.grid.x * l.grid.y;
+    const int64_t slot_blocks = strided_blocks(p);
     return dispatch_lattice<GROUP>(vel, [&](auto lat) {
         using L = decltype(lat);
         const auto* Pt = (const typename S::T*)P;
@@ -866,7 +888,8 @@ int step_storage(int vel, int force, bool efield, bool in_window, const void* P,
                                                   slot_blocks, p, s);                                         \
         if (!staged)                                                                                          \
             k_adjoint_step<L, S, F, EFV, W>                                                                   \
-                <<<l.grid, l.block, 0, s>>>(Pt, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots, p);          \
+                <<<(unsigned)slot_blocks, l.block, 0, s>>>(Pt, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,      \
+                                                           slots, (int)l.grid.y, p);                          \
     } while (0)
         if (force == LBM_FORCE_SHIFT) {
             if (efield) {

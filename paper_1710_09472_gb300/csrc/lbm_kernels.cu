@@ -181,10 +181,10 @@ __global__ void k_row_starts(const uint32_t* __restrict__ nbr, const uint32_t* _
 // partials[block] = {sum rho, sum j_x, sum j_y, sum j_z}.
 // ---------------------------------------------------------------------------
 template <class L, class S>
-__device__ __forceinline__ void cell_moments(const typename S::T* __restrict__ P, const uint32_t* __restrict__ nbr,
-                                             const KParams& p, const Cell& c, float& rho, float* j) {
+__device__ __forceinline__ void cell_moments(const typename S::T* __restrict__ P, uint32_t m, const KParams& p,
+                                             const Cell& c, float& rho, float* j) {
     float h[L::Q];
-    dev::pull<L, S>(P, p, __ldg(nbr + c.cell), c, h);
+    dev::pull<L, S>(P, p, m, c, h);
     float drho = 0.f, jj[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int a = 0; a < L::Q; ++a) {
@@ -202,29 +202,37 @@ __device__ __forceinline__ void cell_moments(const typename S::T* __restrict__ P
     j[2] = (L::D == 3) ? jj[2] * k : 0.f;
 }
 
-template <class L, class S>
+template <class L, class S, bool TOTALS>
 __global__ void __launch_bounds__(kBlock) k_moments(const typename S::T* __restrict__ P, const uint32_t* __restrict__ nbr,
                                                     float* __restrict__ rho_out, float* __restrict__ j_out,
-                                                    double* __restrict__ partials, KParams p) {
-    Cell c;
+                                                    double* __restrict__ partials, int chunks, KParams p) {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    if (dev::cell_of_thread(p, c)) {
-        const uint32_t m = nbr[c.cell];
-        float r = 0.f, j[3] = {0.f, 0.f, 0.f};
-        if (!(m & kSolidBit)) {
-            cell_moments<L, S>(P, nbr, p, c, r, j);
-            acc[0] = (double)r;
-            acc[1] = (double)j[0];
-            acc[2] = (double)j[1];
-            acc[3] = (double)j[2];
-        }
-        if (rho_out) rho_out[c.cell] = r;
-        if (j_out) {
+    // tile t: chunk t % chunks of row t / chunks; the grid has a block for
+    // every tile (fields only) or strides over them (totals)
+    const int64_t tiles = (int64_t)p.ny * p.nz * chunks;
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        Cell c;
+        if (dev::cell_at(p, (int)(t / chunks), (int)(t % chunks) * blockDim.x + threadIdx.x, c)) {
+            const uint32_t m = __ldg(nbr + c.cell);
+            float r = 0.f, j[3] = {0.f, 0.f, 0.f};
+            if (!(m & kSolidBit)) {
+                cell_moments<L, S>(P, m, p, c, r, j);
+                if (TOTALS) {
+                    acc[0] += (double)r;
+                    acc[1] += (double)j[0];
+                    if (L::D >= 2) acc[2] += (double)j[1];
+                    if (L::D == 3) acc[3] += (double)j[2];
+                }
+            }
+            if (rho_out) rho_out[c.cell] = r;
+            if (j_out) {
 #pragma unroll
-            for (int d = 0; d < L::D; ++d) j_out[(int64_t)d * p.N + c.cell] = j[d];
+                for (int d = 0; d < L::D; ++d) j_out[(int64_t)d * p.N + c.cell] = j[d];
+            }
         }
+        if (!TOTALS) return;
     }
-    if (partials) {
+    if (TOTALS) {
         __shared__ double sh[kBlock / 32][4];
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
@@ -240,7 +248,7 @@ __global__ void __launch_bounds__(kBlock) k_moments(const typename S::T* __restr
             for (int k = 0; k < 4; ++k) {
                 double v = lane < nw ? sh[lane][k] : 0.0;
                 v = dev::warp_sum(v);
-                if (lane == 0) partials[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 4 + k] = v;
+                if (lane == 0) partials[(int64_t)blockIdx.x * 4 + k] = v;
             }
         }
     }
@@ -445,15 +453,35 @@ int launch_step(int vel, int storage, int force, bool efield, bool sr, const voi
     return launch_step_f32(vel, force, efield, false, fin, fout, nbr, Ef, p, s);
 }
 
+// With totals the blocks stride over the tiles, kTotalsPerSm of them per SM,
+// and keep their FP64 sums in registers to the end: the chip adds two FP64
+// values per cycle and SM, so a block reduction per 128 cells (160 shuffled
+// FP64 adds) cost several times the reads (52 us on 1024^2 cells of D2V9 FP32),
+// and its 8192 partials another 41 us in the one block that sums them.
+constexpr int kTotalsPerSm = 8;
+
 int launch_moments(int vel, int storage, const void* pop, const uint32_t* nbr, float* rho, float* j,
                    double* partials, int64_t* n_partials, const KParams& p, cudaStream_t s) {
     Launch l = grid_of(p);
-    if (n_partials) *n_partials = (int64_t)l.grid.x * l.grid.y;
+    const int chunks = (int)l.grid.y;
+    const int64_t tiles = (int64_t)l.grid.x * chunks;
+    int64_t blocks = tiles;
+    if (partials) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        blocks = std::min<int64_t>(tiles, (int64_t)std::max(sms, 1) * kTotalsPerSm);
+    }
+    if (n_partials) *n_partials = blocks;
     return dispatch_lattice(vel, [&](auto lat) {
         using L = decltype(lat);
         return dispatch_storage(storage, [&](auto st) {
             using S = decltype(st);
-            k_moments<L, S><<<l.grid, l.block, 0, s>>>((const typename S::T*)pop, nbr, rho, j, partials, p);
+            using T = typename S::T;
+            if (partials)
+                k_moments<L, S, true><<<(unsigned)blocks, l.block, 0, s>>>((const T*)pop, nbr, rho, j, partials, chunks, p);
+            else
+                k_moments<L, S, false><<<(unsigned)blocks, l.block, 0, s>>>((const T*)pop, nbr, rho, j, nullptr, chunks, p);
             return 1;
         });
     });

@@ -445,13 +445,13 @@ __global__ void __launch_bounds__(kBlock) k_step(const typename S::T* __restrict
         collide_any<L, S, FORCE>(h, E, p, out);
     typename S::T t[L::Q];
     round_all<L, S, SR>(out, c.cell, p, t);
-    typename S::T* Gout = reinterpret_cast<typename S::T*>(reinterpret_cast<char*>(Pout) + p.gofs);
-    const uint32_t o = outgoing<L::Q>(m);
-    const uint32_t base = m ? __ldg(p.lbase + c.cell) : 0u;
+    typename S::T* g = reinterpret_cast<typename S::T*>(reinterpret_cast<char*>(Pout) + p.gofs);
+    g += m ? __ldg(p.lbase + c.cell) : 0u;
+    Pout[dev::pop_at<L>(p, c, 0, 0)] = t[0];
 #pragma unroll
-    for (int a = 0; a < L::Q; ++a) {
+    for (int a = 1; a < L::Q; ++a) {
         Pout[dev::pop_at<L>(p, c, a, 0)] = t[a];
-        if (a != 0 && ((o >> a) & 1u)) Gout[link_slot(base, o, a)] = t[a];
+        if ((m >> opposite(a)) & 1u) *g++ = t[a];  // x + e_a is solid: the next link slot
     }
 }
 
