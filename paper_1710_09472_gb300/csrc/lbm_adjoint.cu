@@ -43,21 +43,28 @@ int launch_adjoint_step_bf16_lmu(int, int, bool, bool, const void*, const float*
                                  cudaStream_t);
 
 namespace {
-__global__ void k_fold_partials(float* __restrict__ part, double* __restrict__ acc, int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        acc[i] += (double)part[i];
-        part[i] = 0.f;
+// Blocks stride over chunks of blockDim.x cells of the padded rows.
+__global__ void k_fold_partials(float* __restrict__ part, double* __restrict__ acc, int64_t rows, int nx, int nxp) {
+    const int chunks = (nx + blockDim.x - 1) / blockDim.x;
+    for (int64_t t = blockIdx.x; t < rows * chunks; t += gridDim.x) {
+        const int64_t r = t / chunks;
+        const int x = (int)(t % chunks) * blockDim.x + threadIdx.x;
+        if (x < nx) {
+            acc[r * nx + x] += (double)part[r * nxp + x];
+            part[r * nxp + x] = 0.f;
+        }
     }
 }
 }  // namespace
 
-int launch_fold_partials(float* part, double* acc, int64_t n, cudaStream_t s) {
-    if (n <= 0) return 0;
+int launch_fold_partials(float* part, double* acc, int D, const KParams& p, cudaStream_t s) {
+    const int64_t rows = (int64_t)D * p.ny * p.nz;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t want = (n + 255) / 256, cap = (int64_t)(sms > 0 ? sms : 1) * 8;
-    k_fold_partials<<<(unsigned)(want < cap ? want : cap), 256, 0, s>>>(part, acc, n);
+    const int threads = p.nx >= 256 ? 256 : ((p.nx + 31) / 32) * 32;
+    const int64_t want = rows * ((p.nx + threads - 1) / threads), cap = (int64_t)(sms > 0 ? sms : 1) * 8;
+    k_fold_partials<<<(unsigned)(want < cap ? want : cap), threads, 0, s>>>(part, acc, rows, p.nx, p.nxp);
     return 1;
 }
 

@@ -92,11 +92,11 @@ __device__ __forceinline__ void lmu_table(const KParams& p, float drho, float& d
 }
 
 template <class L, bool EF>
-__device__ __forceinline__ void load_E(const float* __restrict__ Ef, const KParams& p, uint32_t cell, float* E) {
-    if (EF) {
-        E[0] = __ldg(Ef + cell);
-        E[1] = (L::D >= 2) ? __ldg(Ef + p.N + cell) : 0.f;
-        E[2] = (L::D == 3) ? __ldg(Ef + 2 * p.N + cell) : 0.f;
+__device__ __forceinline__ void load_E(const float* __restrict__ Ef, const KParams& p, int64_t pcell, float* E) {
+    if (EF) {  // the padded field, at row * nxp + x
+        E[0] = __ldg(Ef + pcell);
+        E[1] = (L::D >= 2) ? __ldg(Ef + p.NP + pcell) : 0.f;
+        E[2] = (L::D == 3) ? __ldg(Ef + 2 * p.NP + pcell) : 0.f;
     } else {
         E[0] = p.E[0];
         E[1] = p.E[1];
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_step(
                 lt[a] = __ldg(q);
             }
             float E[3], wr, wj[3], lam[L::Q], gEc[3];
-            load_E<L, EF>(Ef, p, c.cell, E);
+            load_E<L, EF>(Ef, p, c.pcell, E);
             load_weights<L, WIN>(w_rho, w_j, p, c.cell, wr, wj);
             // the local-mu model is built for D2V9 and D3V19 (the host refuses others)
             constexpr bool kLmu = L::Q == 9 || L::Q == 19;
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_step(
             if (o) store_lam_links<L>(link_part(lam_out, p), o, lb, lam);
             if (gE) {
 #pragma unroll
-                for (int d = 0; d < L::D; ++d) gE[(int64_t)d * p.N + c.cell] += gEc[d];
+                for (int d = 0; d < L::D; ++d) gE[(int64_t)d * p.NP + c.pcell] += gEc[d];
             }
         }
     }
@@ -486,41 +486,42 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_step(
 }
 
 // ---------------------------------------------------------------------------
-// Row-staged reverse step (persistent; block b takes rows b, b + G, ...).
-// One stage holds, for the row (y, z):
-//   - with dL/dE, the row's D rows of its FP32 partials (accumulated in place
-//     and stored back after the row); with a per-cell field, its D rows of E;
+// Row-staged reverse step (persistent; block b takes units b, b + G, ...: rows,
+// or segments of long rows).  One stage holds, for the unit at row (y, z):
+//   - with dL/dE, the unit's D rows of its FP32 partials (accumulated in place
+//     and stored back after the unit); with a per-cell field, its D rows of E;
 //   - the Q pull rows of the forward state P_t in slot order: direction a
-//     from row (y - e_ay, z - e_az), read at x - e_ax (one copy per
-//     neighbouring row: its block of consecutive slots);
-//   - the row's cell order (fluid cells first, ascending x);
+//     from row (y - e_ay, z - e_az), read at x - e_ax (dev::stage_rows; the
+//     columns beside a segment as in the forward kernel);
+//   - the unit's cell order (fluid cells first, ascending x);
 //   - its window of P_t's link buffer (bounced pulls);
 //   - the Q gather rows of lam_{t+1} in slot order: direction a from row
-//     (y + e_ay, z + e_az), read at x + e_ax (again one copy per row);
+//     (y + e_ay, z + e_az), read at x + e_ax;
 //   - its windows of lam_{t+1}'s link buffer (bounced gathers) and of the
 //     link descriptors;
 // all by bulk asynchronous copies, completing on the stage's mbarrier, armed
 // and issued by lane 0 of the last warp (as in the forward's row-staged
 // kernel; waits are bounded).  One pass over the
-// row's links patches both bounced reads into the staged rows (the solid
+// unit's links patches both bounced reads into the staged rows (the solid
 // neighbour's slot, read by that cell alone), so cells read their rows
 // without link logic.  Thread i takes the i-th cell of the row's order, so
 // each thread's FP64 sums see the same cells in the same order on every run.
 // lam_t goes through shared-memory output rows (zeros for solid cells) that
-// leave by one bulk store (lam has the populations' slot layout), and one
-// pass over the links copies lam_bbar(x) into the row's range of the new
-// link buffer.  dL/dB, dL/dtau and the loss stay
+// leave by one bulk store (lam has the populations' slot layout), and one pass
+// over the links copies lam_bbar(x) into the unit's range of the new link
+// buffer.  dL/dB, dL/dtau and the loss stay
 // in registers until the block's single reduction at the end.
 // ---------------------------------------------------------------------------
 template <class L, class S>
 struct AdjLayout {
-    int nx, rs, lorder, gcapP, gcapL;  // row length, shared-memory row stride (elements), order entries;
-                                       // gcapL also bounds the descriptor window (4-byte elements)
-    int gerow, efrow;                  // bytes of the staged dL/dE rows and E rows (FP32), 0 when absent
+    int rs, lorder, gcapP, gcapL;  // shared-memory row stride (elements), order entries; gcapL also bounds the
+                                   // descriptor window (4-byte elements)
+    int gerow, efrow;              // bytes of the staged dL/dE rows and E rows (FP32), 0 when absent
+    int hP, hL;                    // bytes of the halo arrays of P_t and lam (segments)
     __device__ __host__ int prow() const { return L::Q * rs * S::kBytes; }
     __device__ __host__ int lrow() const { return L::Q * rs * 4; }
     __device__ __host__ int bytes() const {
-        return gerow + prow() + 2 * lorder + gcapP + lrow() + 2 * gcapL + efrow;
+        return gerow + prow() + 2 * lorder + gcapP + lrow() + 2 * gcapL + efrow + hP + hL;
     }
     __device__ unsigned char* gerows(unsigned char* st) const { return st; }
     __device__ unsigned char* prows(unsigned char* st) const { return st + gerow; }
@@ -530,47 +531,33 @@ struct AdjLayout {
     __device__ unsigned char* llinks(unsigned char* st) const { return lrows(st) + lrow(); }
     __device__ unsigned char* descs(unsigned char* st) const { return llinks(st) + gcapL; }
     __device__ unsigned char* efrows(unsigned char* st) const { return descs(st) + gcapL; }
+    __device__ unsigned char* phalo(unsigned char* st) const { return efrows(st) + efrow; }
+    __device__ unsigned char* lhalo(unsigned char* st) const { return phalo(st) + hP; }
 };
 
-// One thread: arms a stage's mbarrier with the byte count of row `row`
+// One thread: arms a stage's mbarrier with the byte count of unit `unit`
 // (links [g0, g1)), records where its windows start (ws[0]: P_t's link
 // window; ws[1]: lam's link window and the descriptor window, which start at
-// the same element), and issues the row's copies into stage st, all
-// completing on bar.  With gE, the row's dL/dE (accumulated in place, stored
-// back after the row); with Ef, its E.
-template <class L, class S>
+// the same element), and issues the unit's copies into stage st, all
+// completing on bar.  With gE, the unit's dL/dE partials (accumulated in
+// place, stored back after the unit); with Ef, its E.
+template <class L, class S, int RS>
 __device__ __forceinline__ void adj_stage(unsigned char* st, const AdjLayout<L, S>& lay, uint64_t* bar,
                                           const typename S::T* P, const float* lam, const float* gE, const float* Ef,
-                                          int row, uint32_t g0, uint32_t g1, uint32_t* ws, const KParams& p) {
-    const uint32_t prb = (uint32_t)p.nx * S::kBytes, lrb = (uint32_t)p.nx * 4u;
-    const int rs = lay.rs;
+                                          int unit, uint32_t g0, uint32_t g1, uint32_t* ws, const KParams& p) {
     uint64_t pb0, pb1, lb0, lb1;
     dev::window_bytes(g0, g1, S::kBytes, pb0, pb1);
     dev::window_bytes(g0, g1, 4, lb0, lb1);
     ws[0] = (uint32_t)(pb0 / S::kBytes);
     ws[1] = (uint32_t)(lb0 / 4);
-    dev::mbar_expect_tx(bar, L::Q * (prb + lrb) + 2u * (uint32_t)lay.lorder + (uint32_t)(pb1 - pb0) +
-                                 2u * (uint32_t)(lb1 - lb0) + (lay.gerow ? L::D * (uint32_t)p.nx * 4u : 0u) +
-                                 (lay.efrow ? L::D * (uint32_t)p.nx * 4u : 0u));
-    const int y = row % p.ny, z = row / p.ny;
-    const int yp = y == p.ny - 1 ? 0 : y + 1, ym = y == 0 ? p.ny - 1 : y - 1;
-    const int zp = z == p.nz - 1 ? 0 : z + 1, zm = z == 0 ? p.nz - 1 : z - 1;
-    unsigned char* pr = lay.prows(st);
-    unsigned char* lr = lay.lrows(st);
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        if (key_count<L>(k) == 0) continue;
-        // the slots key_first(k) .. of the directions with (e_y, e_z): from pull
-        // row (y - e_y, z - e_z) of P_t and gather row (y + e_y, z + e_z) of lam_{t+1}
-        const int ey = k / 3 - 1, ez = k % 3 - 1, s0 = key_first<L>(k), n = key_count<L>(k);
-        const int ysP = ey > 0 ? ym : (ey < 0 ? yp : y), zsP = ez > 0 ? zm : (ez < 0 ? zp : z);
-        const int ysL = ey > 0 ? yp : (ey < 0 ? ym : y), zsL = ez > 0 ? zp : (ez < 0 ? zm : z);
-        dev::bulk_load(pr + s0 * rs * S::kBytes, P + ((int64_t)(zsP * p.ny + ysP) * L::Q + s0) * p.nx,
-                       (uint32_t)n * prb, bar);
-        dev::bulk_load(lr + s0 * rs * 4, lam + ((int64_t)(zsL * p.ny + ysL) * L::Q + s0) * p.nx, (uint32_t)n * lrb,
-                       bar);
-    }
-    dev::bulk_load(lay.order(st), p.rorder + (int64_t)row * lay.lorder, 2u * (uint32_t)lay.lorder, bar);
+    const dev::UnitAt at = dev::unit_at<RS>(p, unit);
+    const uint32_t fb = (uint32_t)lay.rs * 4u;  // bytes of a field row
+    dev::mbar_expect_tx(bar, (uint32_t)(lay.prow() + lay.lrow()) + 2u * (uint32_t)lay.lorder + (uint32_t)(pb1 - pb0) +
+                                 2u * (uint32_t)(lb1 - lb0) + (lay.gerow ? L::D * fb : 0u) +
+                                 (lay.efrow ? L::D * fb : 0u));
+    dev::stage_rows<L, RS, true>(reinterpret_cast<typename S::T*>(lay.prows(st)), P, at, bar, p);
+    dev::stage_rows<L, RS, false>(reinterpret_cast<float*>(lay.lrows(st)), lam, at, bar, p);
+    dev::bulk_load(lay.order(st), p.rorder + (int64_t)unit * lay.lorder, 2u * (uint32_t)lay.lorder, bar);
     if (pb1 > pb0)
         dev::bulk_load(lay.plinks(st), reinterpret_cast<const unsigned char*>(P) + p.gofs + pb0, (uint32_t)(pb1 - pb0),
                        bar);
@@ -580,17 +567,16 @@ __device__ __forceinline__ void adj_stage(unsigned char* st, const AdjLayout<L, 
         dev::bulk_load(lay.descs(st), reinterpret_cast<const unsigned char*>(p.ldesc) + lb0, (uint32_t)(lb1 - lb0),
                        bar);
     }
+    const int64_t f0 = (int64_t)at.row * p.nxp + at.x0;
     if (lay.gerow) {
 #pragma unroll
         for (int d = 0; d < L::D; ++d)
-            dev::bulk_load(lay.gerows(st) + d * rs * 4, gE + (int64_t)d * p.N + (int64_t)row * p.nx,
-                           (uint32_t)p.nx * 4u, bar);
+            dev::bulk_load(lay.gerows(st) + d * lay.rs * 4, gE + (int64_t)d * p.NP + f0, fb, bar);
     }
     if (lay.efrow) {
 #pragma unroll
         for (int d = 0; d < L::D; ++d)
-            dev::bulk_load(lay.efrows(st) + d * rs * 4, Ef + (int64_t)d * p.N + (int64_t)row * p.nx,
-                           (uint32_t)p.nx * 4u, bar);
+            dev::bulk_load(lay.efrows(st) + d * lay.rs * 4, Ef + (int64_t)d * p.NP + f0, fb, bar);
     }
 }
 
@@ -604,24 +590,27 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
                                                          double* __restrict__ slots, int gcapP, int gcapL, KParams p) {
     using T = typename S::T;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int nx = p.nx;
-    const int rs = RS ? RS : nx;  // shared-memory row stride (= nx): a constant for the common row lengths
-    const AdjLayout<L, S> lay{nx, rs, p.lorder, gcapP, gcapL, gE ? L::D * rs * 4 : 0, EF ? L::D * rs * 4 : 0};
+    // RS: whole rows of that many cells, a compile-time stride; 0: a run-time one, whole rows or segments
+    const int rs = RS ? RS : p.seglen;
+    const bool halo = !RS && p.nseg > 1;
+    const AdjLayout<L, S> lay{rs, p.lorder, gcapP, gcapL, gE ? L::D * rs * 4 : 0, EF ? L::D * rs * 4 : 0,
+                              RS ? 0 : dev::halo_bytes(L::Q, p.nseg, S::kBytes),
+                              RS ? 0 : dev::halo_bytes(L::Q, p.nseg, 4)};
     const int sbytes = lay.bytes();
     float* outrow = reinterpret_cast<float*>(smem_raw + STAGES * sbytes);
     __shared__ __align__(8) uint64_t bar[STAGES];
     __shared__ uint32_t wstart[STAGES][2];
     float* lamG_out = link_part(lam_out, p);
-    const int R = p.ny * p.nz;
+    const int U = p.ny * p.nz * (RS ? 1 : p.nseg);
     const int G = gridDim.x;
     const bool leader = threadIdx.x == 0;
     const int warp = (int)(threadIdx.x >> 5), nw = (int)(blockDim.x >> 5), lane = (int)(threadIdx.x & 31);
     const bool issuer = (int)threadIdx.x == (int)blockDim.x - 32;  // lane 0 of the last warp
-    auto range = [&](int row, uint32_t& g0, uint32_t& g1) {
+    auto range = [&](int unit, uint32_t& g0, uint32_t& g1) {
         g0 = g1 = 0u;
-        if (row < R) {
-            g0 = __ldg(p.rowG + row);
-            g1 = __ldg(p.rowG + row + 1);
+        if (unit < U) {
+            g0 = __ldg(p.rowG + unit);
+            g1 = __ldg(p.rowG + unit + 1);
         }
     };
     if (leader) {
@@ -629,27 +618,33 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
         for (int k = 0; k < STAGES; ++k) dev::mbar_init(&bar[k], 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    static_assert(STAGES == 2, "the halo values are fetched one unit ahead");
+    if (halo && dev::halo_thread<L>()) {
+        const dev::UnitAt at = dev::unit_at<RS>(p, blockIdx.x);
+        dev::halo_put<L, true>(reinterpret_cast<T*>(lay.phalo(smem_raw)), dev::halo_fetch<L, true>(P, at, p));
+        dev::halo_put<L, false>(reinterpret_cast<float*>(lay.lhalo(smem_raw)), dev::halo_fetch<L, false>(lam_in, at, p));
+    }
     __syncthreads();
     if (issuer) {
 #pragma unroll
         for (int k = 0; k < STAGES - 1; ++k) {
-            const int rk = blockIdx.x + k * G;
-            if (rk < R) {
+            const int uk = blockIdx.x + k * G;
+            if (uk < U) {
                 uint32_t g0, g1;
-                range(rk, g0, g1);
-                adj_stage<L, S>(smem_raw + k * sbytes, lay, &bar[k], P, lam_in, gE, Ef, rk, g0, g1, wstart[k], p);
+                range(uk, g0, g1);
+                adj_stage<L, S, RS>(smem_raw + k * sbytes, lay, &bar[k], P, lam_in, gE, Ef, uk, g0, g1, wstart[k], p);
             }
         }
     }
     double acc[kSlots] = {0.0, 0.0, 0.0, 0.0, 0.0};
     int it = 0;
     bool ok = true;  // false once a wait has run out (the same in every thread after the first barrier)
-    for (int r = blockIdx.x; r < R; r += G, ++it) {
+    for (int u = blockIdx.x; u < U; u += G, ++it) {
         const int cs = it % STAGES;
-        const int rn = r + (STAGES - 1) * G;       // the row refilled during this one ...
-        const int sn = (it + STAGES - 1) % STAGES;  // ... into the stage of the previous row
+        const int un = u + (STAGES - 1) * G;       // the unit fetched during this one ...
+        const int sn = (it + STAGES - 1) % STAGES;  // ... into the stage of the previous unit
         uint32_t g0, g1;
-        range(r, g0, g1);
+        range(u, g0, g1);
         if (ok && !dev::mbar_wait(&bar[cs], (uint32_t)(it / STAGES) & 1u)) {
             ok = false;
             if (p.status) atomicExch(p.status, 2);
@@ -663,43 +658,69 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
         const uint16_t* ord = reinterpret_cast<const uint16_t*>(lay.order(st));
         const uint32_t* desc = reinterpret_cast<const uint32_t*>(lay.descs(st));
         const uint32_t d0 = wstart[cs][1];
-        dev::patch_links<L, true>(prow, nx, rs, reinterpret_cast<const T*>(lay.plinks(st)), wstart[cs][0], g0, g1,
-                                  desc, d0);
-        dev::patch_links<L, false>(lrow, nx, rs, reinterpret_cast<const float*>(lay.llinks(st)), d0, g0, g1, desc,
-                                   d0);
-        dev::bulk_wait_read();  // this thread's bulk stores of the previous row have read their sources
+        T* phal = reinterpret_cast<T*>(lay.phalo(st));
+        float* lhal = reinterpret_cast<float*>(lay.lhalo(st));
+        dev::patch_links<true, RS == 0>(prow, rs, phal, L::Q, reinterpret_cast<const T*>(lay.plinks(st)),
+                                        wstart[cs][0], g0, g1, desc, d0);
+        dev::patch_links<false, RS == 0>(lrow, rs, lhal, L::Q, reinterpret_cast<const float*>(lay.llinks(st)), d0, g0,
+                                         g1, desc, d0);
+        dev::bulk_wait_read();  // this thread's bulk stores of the previous unit have read their sources
         // bounced values in place, output rows free; a timeout anywhere in
         // the block stops the copies
         ok = __syncthreads_and(ok) != 0;
-        if (issuer && ok && rn < R) {
-            // refill the stage of the previous row (every thread is past its
+        if (issuer && ok && un < U) {
+            // refill the stage of the previous unit (every thread is past its
             // reads of it and its wait on that stage's barrier)
             uint32_t n0, n1;
-            range(rn, n0, n1);
-            adj_stage<L, S>(smem_raw + sn * sbytes, lay, &bar[sn], P, lam_in, gE, Ef, rn, n0, n1, wstart[sn], p);
+            range(un, n0, n1);
+            adj_stage<L, S, RS>(smem_raw + sn * sbytes, lay, &bar[sn], P, lam_in, gE, Ef, un, n0, n1, wstart[sn], p);
+        }
+        const bool fetch = halo && un < U && dev::halo_thread<L>();
+        T hvP{};
+        float hvL = 0.f;
+        if (fetch) {
+            const dev::UnitAt next = dev::unit_at<RS>(p, un);
+            hvP = dev::halo_fetch<L, true>(P, next, p);
+            hvL = dev::halo_fetch<L, false>(lam_in, next, p);
         }
         const int nf = ord[0];
-        const uint32_t rowbase = (uint32_t)r * (uint32_t)nx;
+        const dev::UnitAt at = dev::unit_at<RS>(p, u);
+        const int nx = at.len;  // cells of the unit
+        const uint32_t rowbase = (uint32_t)at.row * (uint32_t)(RS ? RS : p.nx) + (uint32_t)at.x0;  // first cell
         for (int i = threadIdx.x; i < nx; i += blockDim.x) {
             const int x = (int)ord[8 + i];
             if (i < nf) {
                 const uint32_t cell = rowbase + (uint32_t)x;
-                const int xm = x == 0 ? nx - 1 : x - 1;
-                const int xp = x == nx - 1 ? 0 : x + 1;
+                // columns x - 1 and x + 1, as in the forward kernel
+                const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+                const T *pm = prow + xm, *pp = prow + xp;
+                const float *lm = lrow + xm, *lp = lrow + xp;
+                int rm = rs, rp = rs;
+                if (halo && x == 0) {
+                    pm = phal;
+                    lm = lhal;
+                    rm = 1;
+                }
+                if (halo && x == nx - 1) {
+                    pp = phal + L::Q;
+                    lp = lhal + L::Q;
+                    rp = 1;
+                }
                 float h[L::Q], lt[L::Q];
 #pragma unroll
                 for (int a = 0; a < L::Q; ++a) {
-                    const int ex = L::c(a, 0);
-                    h[a] = S::cvt(prow[pop_slot<L>(a) * rs + (ex > 0 ? xm : (ex < 0 ? xp : x))]) * p.inv_scale;
-                    lt[a] = lrow[pop_slot<L>(a) * rs + (ex > 0 ? xp : (ex < 0 ? xm : x))];
+                    const int ex = L::c(a, 0), s = pop_slot<L>(a);
+                    const int sm = s * (RS ? RS : rm), sp = s * (RS ? RS : rp);
+                    h[a] = S::cvt(ex > 0 ? pm[sm] : (ex < 0 ? pp[sp] : prow[s * rs + x])) * p.inv_scale;
+                    lt[a] = ex > 0 ? lp[sp] : (ex < 0 ? lm[sm] : lrow[s * rs + x]);
                 }
                 float E[3], wr, wj[3], lam[L::Q], gEc[3];
                 if (EF) {
                     E[0] = ef_s[x];
-                    E[1] = ef_s[rs + x];
+                    E[1] = (L::D >= 2) ? ef_s[rs + x] : 0.f;
                     E[2] = (L::D == 3) ? ef_s[2 * rs + x] : 0.f;
                 } else {
-                    load_E<L, false>(Ef, p, cell, E);
+                    load_E<L, false>(Ef, p, 0, E);
                 }
                 load_weights<L, WIN>(w_rho, w_j, p, cell, wr, wj);
                 adjoint_cell<L, FORCE, WIN, LMU>(h, lt, E, p, wr, wj, lam, gEc, acc);
@@ -714,26 +735,30 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
                 for (int b = 0; b < L::Q; ++b) outrow[b * rs + x] = 0.f;
             }
         }
+        if (fetch) {
+            dev::halo_put<L, true>(reinterpret_cast<T*>(lay.phalo(smem_raw + sn * sbytes)), hvP);
+            dev::halo_put<L, false>(reinterpret_cast<float*>(lay.lhalo(smem_raw + sn * sbytes)), hvL);
+        }
         dev::fence_proxy_async();
         __syncthreads();  // output rows complete
         {
-            // lane l of warp w takes piece w + l nw: the row's Q output slots
+            // lane l of warp w takes piece w + l nw: the unit's Q output slots
             // (one block), then its D updated dL/dE rows back from the stage
             // (which is refilled only after the issuing threads' reads are done)
             const int k = warp + lane * nw;
             if (k == 0) {
-                dev::bulk_store(lam_out + (int64_t)rowbase * L::Q, outrow, (uint32_t)(L::Q * nx) * 4u);
+                dev::bulk_store(lam_out + (int64_t)u * (L::Q * rs), outrow, (uint32_t)lay.lrow());
                 dev::bulk_commit();
             } else if (gE && k <= L::D) {
                 const int d = k - 1;
-                dev::bulk_store(gE + (int64_t)d * p.N + rowbase, ge_s + d * rs, (uint32_t)nx * 4u);
+                dev::bulk_store(gE + (int64_t)d * p.NP + (int64_t)u * rs, ge_s + d * rs, (uint32_t)rs * 4u);
                 dev::bulk_commit();
             }
         }
         // link copies of lam_t: slot k of (x, b) takes lam_bbar(x)
         for (uint32_t k = g0 + threadIdx.x; k < g1; k += blockDim.x) {
             const uint32_t d = desc[k - d0];
-            lamG_out[k] = outrow[slot_of<L>(opposite((int)(d >> 24))) * rs + (int)(d & 0xFFFFFFu)];
+            lamG_out[k] = outrow[desc_slot_bar(d) * rs + desc_x(d)];
         }
     }
     dev::bulk_wait_all();
@@ -773,9 +798,9 @@ int dispatch_lattice(int vel, F&& f) {
 
 
 // ---------------------------------------------------------------------------
-// Launch policy of the reverse step: the row-staged kernel when a row of one
-// direction of the state is a multiple of 16 bytes, nx >= 32, nx % 4 == 0 and
-// the stages fit the shared-memory budget; otherwise the general kernel.
+// Launch policy of the reverse step: the row-staged kernel when the context has
+// units and their stages fit the shared-memory budget; otherwise the general
+// kernel.
 // ---------------------------------------------------------------------------
 constexpr int kAdjStages = 2;
 constexpr int kAdjThreads = 256;
@@ -785,25 +810,22 @@ template <class L, class S, int FORCE, bool EF, bool WIN, int RS, bool LMU = fal
 bool launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
                  const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
                  const KParams& p, cudaStream_t s) {
-    if (!p.rorder || (p.nx * S::kBytes) % 16 != 0 || p.nx % 4 != 0 || p.nx < 32) return false;
-    if (reinterpret_cast<uintptr_t>(gE) % 16 != 0) return false;  // dL/dE rows move by bulk copies
+    if (!p.rorder || (RS && (RS != p.nx || p.nseg != 1))) return false;
     const int gcapP = dev::window_cap(p.max_row_links, S::kBytes);
     const int gcapL = dev::window_cap(p.max_row_links, 4);
-    if (RS && RS != p.nx) return false;  // the stage rows are exactly nx long
-    const int rs = p.nx;
-    const size_t stage =
-        (size_t)AdjLayout<L, S>{p.nx, rs, p.lorder, gcapP, gcapL, gE ? L::D * rs * 4 : 0, EF ? L::D * rs * 4 : 0}
-            .bytes();
-    const size_t smem = kAdjStages * stage + (size_t)L::Q * rs * 4;
+    const int rs = p.seglen, hP = dev::halo_bytes(L::Q, p.nseg, S::kBytes), hL = dev::halo_bytes(L::Q, p.nseg, 4);
+    const int gerow = L::D * rs * 4, efrow = EF ? L::D * rs * 4 : 0;
+    auto smem_for = [&](int ge) {
+        return kAdjStages * (size_t)AdjLayout<L, S>{rs, p.lorder, gcapP, gcapL, ge, efrow, hP, hL}.bytes() +
+               (size_t)L::Q * rs * 4;
+    };
+    const size_t smem = smem_for(gE ? gerow : 0);
     // the kernel choice and the persistent grid are taken for the layout with
     // dL/dE rows, whether or not this call has them, so that the blocks (and
     // with them the order of the FP64 gradient sums) are the same either way
-    const size_t smem_ref =
-        kAdjStages *
-            (size_t)AdjLayout<L, S>{p.nx, rs, p.lorder, gcapP, gcapL, L::D * rs * 4, EF ? L::D * rs * 4 : 0}.bytes() +
-        (size_t)L::Q * rs * 4;
+    const size_t smem_ref = smem_for(gerow);
     if (smem_ref > kAdjSmemBudget) return false;
-    const int threads = p.nx >= kAdjThreads ? kAdjThreads : ((p.nx + 31) / 32) * 32;
+    const int threads = p.seglen >= kAdjThreads ? kAdjThreads : ((p.seglen + 31) / 32) * 32;
     auto kern = k_adjoint_rows<L, S, FORCE, EF, WIN, kAdjStages, RS, LMU>;
     // persistent grid: co-resident blocks per SM (occupancy API) x SMs,
     // cached per instantiation and shared-memory size
@@ -826,8 +848,8 @@ bool launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const ui
         }
         blocks = last_blocks;
     }
-    const int rows = p.ny * p.nz;
-    if (blocks > rows) blocks = rows;
+    const int units = p.ny * p.nz * p.nseg;
+    if (blocks > units) blocks = units;
     if (blocks <= 0 || blocks > slot_blocks) return false;
     kern<<<blocks, threads, smem, s>>>((const typename S::T*)P, lam_in, lam_out, Ef, w_rho, w_j, gE, slots,
                                        gcapP, gcapL, p);
@@ -845,8 +867,8 @@ bool launch_rows(const void* P, const float* lam_in, float* lam_out, const uint3
     if (kFixed && p.nx == 256)
         return launch_rows_rs<L, S, FORCE, EF, WIN, kFixed ? 256 : 0>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,
                                                                        slots, slot_blocks, p, s);
-    if (kFixed && p.nx == 512)
-        return launch_rows_rs<L, S, FORCE, EF, WIN, kFixed ? 512 : 0>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,
+    if (kFixed && p.nx == 512 && p.nseg == 1)
+        return launch_rows_rs<L, S, FORCE, EF, WIN, kFixed && whole_row<L, S>(512) ? 512 : 0>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,
                                                                        slots, slot_blocks, p, s);
     return launch_rows_rs<L, S, FORCE, EF, WIN, 0>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots, slot_blocks,
                                                     p, s);

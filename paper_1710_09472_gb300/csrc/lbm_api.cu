@@ -173,7 +173,12 @@ lbm::KParams lbm::make_params(const lbm_ctx* c) {
     p.nx = (int)c->nx;
     p.ny = (int)c->ny;
     p.nz = (int)c->nz;
+    p.nseg = c->nseg;
+    p.seglen = c->seglen;
+    p.qm1 = c->Q - 1;
+    p.nxp = (int)c->nxp;
     p.N = c->N;
+    p.NP = c->NP;
     p.omega = (float)(1.0 / c->tau);
     p.tau = (float)c->tau;
     p.rho0 = (float)c->lat.rho0;
@@ -287,6 +292,75 @@ void ws_release(lbm_ctx* c) {
     w = AdjWorkspace();
 }
 
+// Units (see pop_slot).  A row stays whole while its rows of all directions,
+// twice staged and once as outputs, fit kRowSmem: three or more blocks then
+// share an SM.  A longer row is cut into equal segments of at most kMaxSegment
+// columns.  As whole rows, D2V9 FP32 rows of 1024 cells kept one block of eight
+// warps per SM: 27.6 us per step at 1024^2, and no reverse step but the general
+// one (95 us).
+constexpr int kMaxSegment = 256;
+
+void set_units(lbm_ctx* c) {
+    const int nx = (int)c->nx;
+    c->nseg = 1;
+    c->seglen = nx;
+    if (nx >= lbm::kMinStagedRow) {
+        const int up = lbm::kPitch;
+        const int cols = std::min(lbm::kRowSmem / (int)(3 * c->Q * pop_elem_bytes(c->storage)), lbm::kMaxUnit);
+        const int most = std::max(up, std::min(kMaxSegment, cols / up * up));
+        auto padded = [&](int n) { return (n + up - 1) / up * up; };
+        if (padded(nx) > cols) c->nseg = (nx + most - 1) / most;
+        c->seglen = padded((nx + c->nseg - 1) / c->nseg);
+        c->nseg = (nx + c->seglen - 1) / c->seglen;
+    }
+    c->nxp = (int64_t)c->nseg * c->seglen;
+    c->NP = c->nxp * c->ny * c->nz;
+}
+
+// Sizes of a saved state: the populations as whole rows of nx columns (slot
+// order), rounded up to 256 bytes, then the link buffer.  It does not depend on
+// the units.
+struct SavedSize {
+    size_t gofs, payload;
+};
+SavedSize saved_size(const lbm_ctx* c) {
+    SavedSize s;
+    s.gofs = ((size_t)c->Q * (size_t)c->N * pop_elem_bytes(c->storage) + 255) & ~(size_t)255;
+    s.payload = s.gofs + (c->state_bytes - c->gofs);
+    return s;
+}
+
+// Copies a state buffer from or to its saved form in host memory.
+cudaError_t copy_saved(lbm_ctx* c, void* host, bool save) {
+    const SavedSize z = saved_size(c);
+    unsigned char* pop = (unsigned char*)c->pop[c->cur];
+    unsigned char* h = (unsigned char*)host;
+    if (c->nxp == c->nx && c->nseg == 1)
+        return save ? cudaMemcpyAsync(h, pop, z.payload, cudaMemcpyDeviceToHost, c->stream)
+                    : cudaMemcpyAsync(pop, h, z.payload, cudaMemcpyHostToDevice, c->stream);
+    // segment k of every row and slot: host rows of nx, device rows of seglen
+    // in blocks of nseg Q (one block per row)
+    const size_t eb = pop_elem_bytes(c->storage), R = (size_t)(c->ny * c->nz), Q = (size_t)c->Q;
+    const size_t rows = Q * R * (size_t)c->nx * eb, links = c->state_bytes - c->gofs;
+    if (save) std::memset(h + rows, 0, z.gofs - rows);
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < c->nseg && e == cudaSuccess; ++k) {
+        const size_t x0 = (size_t)k * c->seglen, len = std::min<size_t>(c->seglen, (size_t)c->nx - x0);
+        const cudaPitchedPtr hp = make_cudaPitchedPtr(h + x0 * eb, (size_t)c->nx * eb, len * eb, Q);
+        const cudaPitchedPtr dp = make_cudaPitchedPtr(pop + x0 * Q * eb, (size_t)c->seglen * eb, len * eb, Q * c->nseg);
+        cudaMemcpy3DParms m = {};
+        m.srcPtr = save ? dp : hp;
+        m.dstPtr = save ? hp : dp;
+        m.extent = make_cudaExtent(len * eb, Q, R);
+        m.kind = save ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice;
+        e = cudaMemcpy3DAsync(&m, c->stream);
+    }
+    if (e == cudaSuccess)
+        e = save ? cudaMemcpyAsync(h + z.gofs, pop + c->gofs, links, cudaMemcpyDeviceToHost, c->stream)
+                 : cudaMemcpyAsync(pop + c->gofs, h + z.gofs, links, cudaMemcpyHostToDevice, c->stream);
+    return e;
+}
+
 // Link-buffer layout for the current link masks, then state buffers sized
 // for populations + links (contents undefined until lbm_init_equilibrium).
 lbm_status build_links_and_state(lbm_ctx* c) {
@@ -298,7 +372,7 @@ lbm_status build_links_and_state(lbm_ctx* c) {
     LBM_CUDA(c, cudaMalloc(&temp, temp_bytes > 0 ? temp_bytes : 16));
     c->launches += lbm::launch_build_links(c->lat.vel, c->nbr, c->lbase, c->rowG, temp, &temp_bytes, p, c->stream);
     lbm_status st = cuda_check(c, cudaGetLastError(), "link layout kernels");
-    const int64_t R = c->ny * c->nz;
+    const int64_t R = c->ny * c->nz * c->nseg;  // units
     std::vector<uint32_t> rowG((size_t)R + 1);
     if (st == LBM_OK)
         st = cuda_check(c, cudaMemcpyAsync(rowG.data(), c->rowG, sizeof(uint32_t) * (R + 1), cudaMemcpyDeviceToHost,
@@ -310,16 +384,16 @@ lbm_status build_links_and_state(lbm_ctx* c) {
     int mx = 0;
     for (int64_t r = 0; r < R; ++r) mx = std::max(mx, (int)(rowG[r + 1] - rowG[r]));
     c->max_row_links = mx;
-    // link descriptors (x | b << 24), one per slot
+    // link descriptors, one per slot
     cudaFree(c->ldesc);
     c->ldesc = nullptr;
     LBM_CUDA(c, cudaMalloc((void**)&c->ldesc, sizeof(uint32_t) * ((size_t)c->n_links + 4)));
     p.ldesc = c->ldesc;
     c->launches += lbm::launch_build_link_desc(c->lat.vel, c->nbr, c->lbase, c->ldesc, p, c->stream);
     LBM_CUDA(c, cudaGetLastError());
-    // per-row cell order of the row-staged kernels (entries are 16-bit x)
-    if (!c->rorder && c->nx <= 65535) {
-        c->lorder = 8 + (int)((c->nx + 7) / 8) * 8;
+    // per-unit cell order of the row-staged kernels
+    if (!c->rorder && c->nx >= lbm::kMinStagedRow) {
+        c->lorder = 8 + c->seglen;
         LBM_CUDA(c, cudaMalloc((void**)&c->rorder, sizeof(uint16_t) * (size_t)R * (size_t)c->lorder));
         p.lorder = c->lorder;
     }
@@ -329,7 +403,7 @@ lbm_status build_links_and_state(lbm_ctx* c) {
         LBM_CUDA(c, cudaGetLastError());
     }
     const size_t eb = pop_elem_bytes(c->storage);
-    const size_t pbytes = (size_t)c->Q * (size_t)c->N * eb;
+    const size_t pbytes = (size_t)c->Q * (size_t)c->NP * eb;
     c->gofs = (pbytes + 255) & ~(size_t)255;
     const size_t need = c->gofs + ((((size_t)c->n_links * eb) + 16 + 255) & ~(size_t)255);
     if (need != c->state_bytes || c->ws.lam_bytes) ws_release(c);  // sizes follow the links
@@ -401,6 +475,7 @@ lbm_status lbm_create(lbm_ctx** out, const lbm_lattice* lat, const int64_t dims[
     c->N = dims[0] * dims[1] * dims[2];
     c->n_fluid = c->N;
     c->storage = storage;
+    set_units(c);
     c->tau = tau;
     c->stream = (cudaStream_t)cuda_stream;
     for (int d = 0; d < 3; ++d) {
@@ -478,7 +553,7 @@ lbm_status lbm_create(lbm_ctx** out, const lbm_lattice* lat, const int64_t dims[
             LBM_OK ||
         (st = cuda_check(c, cudaMalloc((void**)&c->lbase, sizeof(uint32_t) * c->N), "cudaMalloc link bases")) !=
             LBM_OK ||
-        (st = cuda_check(c, cudaMalloc((void**)&c->rowG, sizeof(uint32_t) * (c->ny * c->nz + 1)),
+        (st = cuda_check(c, cudaMalloc((void**)&c->rowG, sizeof(uint32_t) * (c->ny * c->nz * c->nseg + 1)),
                          "cudaMalloc row links")) != LBM_OK ||
         (st = cuda_check(c, cudaMalloc((void**)&c->mask_dev, c->N), "cudaMalloc mask")) != LBM_OK ||
         (st = cuda_check(c, cudaMalloc((void**)&c->partials, sizeof(double) * 4 * c->partials_cap),
@@ -584,10 +659,13 @@ lbm_status lbm_set_E_field(lbm_ctx* c, const float* E) {
         c->use_Efield = false;
         return LBM_OK;
     }
-    const size_t bytes = sizeof(float) * (size_t)c->D * (size_t)c->N;
-    if (!c->Efield) LBM_CUDA(c, cudaMalloc((void**)&c->Efield, bytes));
+    const size_t row = sizeof(float) * (size_t)c->nx, rows = (size_t)c->D * (size_t)(c->ny * c->nz);
+    if (!c->Efield) LBM_CUDA(c, cudaMalloc((void**)&c->Efield, sizeof(float) * (size_t)c->D * (size_t)c->NP));
     const cudaMemcpyKind kind = is_device_ptr(E) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    LBM_CUDA(c, cudaMemcpyAsync(c->Efield, E, bytes, kind, c->stream));
+    if (c->nxp == c->nx)
+        LBM_CUDA(c, cudaMemcpyAsync(c->Efield, E, row * rows, kind, c->stream));
+    else
+        LBM_CUDA(c, cudaMemcpy2DAsync(c->Efield, sizeof(float) * (size_t)c->nxp, E, row, row, rows, kind, c->stream));
     c->use_Efield = true;
     return LBM_OK;
 }
@@ -774,7 +852,7 @@ lbm_status lbm_get_populations(lbm_ctx* c, float* f, int deviation) {
 
 lbm_status lbm_save_state(lbm_ctx* c, void* host_buf, size_t cap, size_t* used) {
     if (!c || !used) return LBM_ERR_INVALID_ARG;
-    const size_t payload = c->state_bytes;
+    const size_t payload = saved_size(c).payload;
     const size_t total = sizeof(StateHeader) + payload;
     *used = total;
     if (!host_buf) return LBM_OK;
@@ -791,7 +869,7 @@ lbm_status lbm_save_state(lbm_ctx* c, void* host_buf, size_t cap, size_t* used) 
     h.steps = c->steps;
     h.payload = payload;
     unsigned char* dst = (unsigned char*)host_buf + sizeof(StateHeader);
-    LBM_CUDA(c, cudaMemcpyAsync(dst, c->pop[c->cur], payload, cudaMemcpyDeviceToHost, c->stream));
+    LBM_CUDA(c, copy_saved(c, dst, true));
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
     {
         lbm_status _ds = device_status(c);
@@ -807,14 +885,14 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* host_buf, size_t len) {
     if (len < sizeof(StateHeader)) return fail(c, LBM_ERR_INVALID_ARG, "lbm_load_state: short buffer");
     StateHeader h;
     std::memcpy(&h, host_buf, sizeof h);
-    const size_t payload = c->state_bytes;
+    const size_t payload = saved_size(c).payload;
     if (std::memcmp(h.magic, "LBMSTAT", 8) != 0 || h.vel != c->lat.vel || h.storage != c->storage || h.nx != c->nx ||
         h.ny != c->ny || h.nz != c->nz || h.payload != payload)
         return fail(c, LBM_ERR_INVALID_ARG, "lbm_load_state: header does not match this context");
     if (len < sizeof(StateHeader) + payload) return fail(c, LBM_ERR_INVALID_ARG, "lbm_load_state: short buffer");
     const unsigned char* src = (const unsigned char*)host_buf + sizeof(StateHeader);
     if (checksum(src, payload) != h.crc) return fail(c, LBM_ERR_INVALID_ARG, "lbm_load_state: checksum mismatch");
-    LBM_CUDA(c, cudaMemcpyAsync(c->pop[c->cur], src, payload, cudaMemcpyHostToDevice, c->stream));
+    LBM_CUDA(c, copy_saved(c, const_cast<unsigned char*>(src), false));
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
     *(volatile int*)c->status_host = 0;  // the state that a timed-out wait left is replaced
     c->steps = h.steps;
@@ -917,7 +995,7 @@ lbm_status lbm_adjoint(lbm_ctx* c, const float* w_rho, const float* w_j, int64_t
     const size_t pop_bytes = c->state_bytes;  // populations + link buffer
     // adjoint field: lam in population layout, then its link buffer (one FP32
     // per bounce-back link) at a 256-byte aligned offset
-    const size_t lam_bytes = sizeof(float) * (size_t)c->Q * (size_t)c->N;
+    const size_t lam_bytes = sizeof(float) * (size_t)c->Q * (size_t)c->NP;
     const size_t lgofs = (lam_bytes + 255) & ~(size_t)255;
     const size_t lam_alloc = lgofs + ((sizeof(float) * (size_t)c->n_links + 16 + 255) & ~(size_t)255);
     KParams p = make_params(c);
@@ -937,7 +1015,7 @@ lbm_status lbm_adjoint(lbm_ctx* c, const float* w_rho, const float* w_j, int64_t
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
     free_b += ws.held();
-    const size_t gpart_bytes = dL_dE ? sizeof(float) * (size_t)c->D * (size_t)c->N : 0;
+    const size_t gpart_bytes = dL_dE ? sizeof(float) * (size_t)c->D * (size_t)c->NP : 0;
     const size_t fixed =
         2 * lam_alloc + sizeof(double) * (nslot + 8) + sizeof(float) * (size_t)c->N * (1 + c->D) + gpart_bytes;
     // bytes for the kept forward states: the budget, or 95% of what the fixed part leaves free
@@ -1071,7 +1149,7 @@ lbm_status lbm_adjoint(lbm_ctx* c, const float* w_rho, const float* w_j, int64_t
                                                 c->Efield, wr_d, wj_d, gpart, slots, p, c->stream);
         li ^= 1;
         if (gpart && ++rsteps % kFoldEvery == 0)
-            c->launches += lbm::launch_fold_partials(gpart, dL_dE, (int64_t)c->D * c->N, c->stream);
+            c->launches += lbm::launch_fold_partials(gpart, dL_dE, c->D, p, c->stream);
     };
     auto seed = [&](const void* state_T) {
         c->launches += lbm::launch_adjoint_seed(vel, sto, state_T, c->nbr, wr_d, wj_d, lam[li], slots,
@@ -1183,7 +1261,7 @@ lbm_status lbm_adjoint(lbm_ctx* c, const float* w_rho, const float* w_j, int64_t
         c->cur ^= 1;  // the context's current state is the state at T
     }
     if (gpart && rsteps % kFoldEvery != 0)  // the last partials
-        c->launches += lbm::launch_fold_partials(gpart, dL_dE, (int64_t)c->D * c->N, c->stream);
+        c->launches += lbm::launch_fold_partials(gpart, dL_dE, c->D, p, c->stream);
     c->adj_stats[0] = store_all ? 2 : (binomial ? 1 : 0);
     c->adj_stats[1] = store_all ? T + 1 : (binomial ? 2 + nsnap : nseg + K - 1);
     c->adj_stats[2] = fwd_steps;

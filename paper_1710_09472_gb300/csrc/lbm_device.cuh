@@ -16,7 +16,9 @@ struct Cell {
     int x, y, z;
     uint32_t cell;
     int xm, xp;       // x - 1, x + 1 with periodic wrap
-    uint32_t r[3][3]; // row base ((z + dz) * ny + (y + dy)) * nx for dy, dz in {-1, 0, 1}
+    int xo[3];        // offsets of the columns xm, x, xp in a row of units, slot 0
+    uint32_t r[3][3]; // row (z + dz) * ny + (y + dy) for dy, dz in {-1, 0, 1}
+    int64_t pcell;    // row * nxp + x: index into the padded fields (E, dL/dE partials)
 };
 
 __device__ __forceinline__ bool cell_at(const KParams& p, int row, int x, Cell& c) {
@@ -31,7 +33,12 @@ __device__ __forceinline__ bool cell_at(const KParams& p, int row, int x, Cell& 
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) c.r[i][k] = ((uint32_t)zs[k] * (uint32_t)p.ny + (uint32_t)ys[i]) * (uint32_t)p.nx;
+        for (int k = 0; k < 3; ++k) c.r[i][k] = (uint32_t)zs[k] * (uint32_t)p.ny + (uint32_t)ys[i];
+    c.pcell = (int64_t)row * p.nxp + x;
+    const int xs[3] = {c.xm, c.x, c.xp};
+#pragma unroll
+    for (int i = 0; i < 3; ++i)  // whole rows need no division
+        c.xo[i] = p.nseg == 1 ? xs[i] : xs[i] + xs[i] / p.seglen * (p.qm1 * p.seglen);
     return c.x < p.nx;
 }
 __device__ __forceinline__ bool cell_of_thread(const KParams& p, Cell& c) {
@@ -40,10 +47,10 @@ __device__ __forceinline__ bool cell_of_thread(const KParams& p, Cell& c) {
 
 // Index of x + s e_a (s = +1 or -1) with periodic wrap.
 template <class L>
-__device__ __forceinline__ uint32_t shifted(const Cell& c, int a, int s) {
+__device__ __forceinline__ uint32_t shifted(const KParams& p, const Cell& c, int a, int s) {
     const int ex = s * L::c(a, 0), ey = s * L::c(a, 1), ez = s * L::c(a, 2);
     const int xs = ex > 0 ? c.xp : (ex < 0 ? c.xm : c.x);
-    return c.r[ey + 1][ez + 1] + (uint32_t)xs;
+    return c.r[ey + 1][ez + 1] * (uint32_t)p.nx + (uint32_t)xs;
 }
 
 // Storage index of direction a at the cell x + s e_a (s = -1, 0 or +1): slot
@@ -51,8 +58,7 @@ __device__ __forceinline__ uint32_t shifted(const Cell& c, int a, int s) {
 template <class L>
 __device__ __forceinline__ int64_t pop_at(const KParams& p, const Cell& c, int a, int s) {
     const int ex = s * L::c(a, 0), ey = s * L::c(a, 1), ez = s * L::c(a, 2);
-    const int xs = ex > 0 ? c.xp : (ex < 0 ? c.xm : c.x);
-    return (int64_t)L::Q * c.r[ey + 1][ez + 1] + (int64_t)(pop_slot<L>(a) * p.nx + xs);
+    return (int64_t)c.r[ey + 1][ez + 1] * (uint32_t)(L::Q * p.nxp) + (pop_slot<L>(a) * p.seglen + c.xo[ex + 1]);
 }
 
 template <class L>
@@ -117,51 +123,26 @@ __device__ __forceinline__ void pull(const typename S::T* __restrict__ P, const 
     }
 }
 
-// e_ay + 1 and e_az + 1 of every direction, 2 bits each, in two 64-bit words
-// (19 directions need 38 bits per word); the unrolled loops fold to constants.
-template <class L>
-__device__ __forceinline__ unsigned long long packed_y() {
-    unsigned long long v = 0;
-#pragma unroll
-    for (int a = 0; a < L::Q; ++a) v |= (unsigned long long)(L::c(a, 1) + 1) << (2 * a);
-    return v;
-}
-template <class L>
-__device__ __forceinline__ unsigned long long packed_z() {
-    unsigned long long v = 0;
-#pragma unroll
-    for (int a = 0; a < L::Q; ++a) v |= (unsigned long long)(L::c(a, 2) + 1) << (2 * a);
-    return v;
-}
-
-template <class L>
-__device__ __forceinline__ unsigned long long packed_x() {
-    unsigned long long v = 0;
-#pragma unroll
-    for (int a = 0; a < L::Q; ++a) v |= (unsigned long long)(L::c(a, 0) + 1) << (2 * a);
-    return v;
-}
-
-// Bounce-back patch of a staged row set.  Link k of the row is a fluid cell x
-// with an outgoing direction b into a solid cell, descriptor x | b << 24.  The
-// solid neighbour x + e_b is read by exactly one cell of the row for each
-// direction: by x itself, in the pull of direction bbar (which reads
-// x - e_bbar = x + e_b) and in the adjoint gather of direction b (which reads
-// x + e_b).  So the halfway bounce-back value win[k - w0] is written into that
-// staged slot, rows[slot(d) * rs + (x + e_bx mod nx)] (rows in slot order, rs
-// the row stride) with d = bbar (PULL) or b (gather), and the cells then read
-// their rows without any link logic.
-// The descriptors come from the staged window desc (first element d0).
-template <class L, bool PULL, class T>
-__device__ __forceinline__ void patch_links(T* rows, int nx, int rs, const T* win, uint32_t w0, uint32_t g0,
+// Bounce-back patch of a staged row set.  Link k of the unit is a fluid cell x
+// with an outgoing direction b into a solid cell (descriptor link_desc).  The
+// solid neighbour x + e_b is read by exactly one cell for each direction: by x
+// itself, in the pull of direction bbar (which reads x - e_bbar = x + e_b) and
+// in the adjoint gather of direction b (which reads x + e_b).  So the halfway
+// bounce-back value win[k - w0] is written into that staged slot, of direction
+// bbar (PULL) or b (gather), and the cells then read their rows without any
+// link logic.  The descriptors come from the staged window desc (first element
+// d0); they hold the slots and columns worked out once per geometry, which
+// leaves half the instructions of a pass that decodes (x, b) and wraps x.
+// HALO: a neighbour may lie in a halo array (hal: Q left values, Q right ones).
+template <bool PULL, bool HALO, class T>
+__device__ __forceinline__ void patch_links(T* rows, int rs, T* hal, int Q, const T* win, uint32_t w0, uint32_t g0,
                                             uint32_t g1, const uint32_t* desc, uint32_t d0) {
-    const unsigned long long kPx = packed_x<L>();
     for (uint32_t k = g0 + threadIdx.x; k < g1; k += blockDim.x) {
         const uint32_t d = desc[k - d0];
-        const int x = (int)(d & 0xFFFFFFu), b = (int)(d >> 24);
-        int xs = x + (int)((kPx >> (2 * b)) & 3ull) - 1;
-        xs = xs < 0 ? xs + nx : (xs >= nx ? xs - nx : xs);
-        rows[slot_of<L>(PULL ? opposite(b) : b) * rs + xs] = win[k - w0];
+        const int slot = PULL ? desc_slot_bar(d) : desc_slot(d), pos = desc_pos(d);
+        T* q = rows + slot * rs + pos;
+        if (HALO && pos >= kPosLeft) q = hal + (pos == kPosLeft ? 0 : Q) + slot;
+        *q = win[k - w0];
     }
 }
 
@@ -235,6 +216,110 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 // orders this thread's generic-proxy shared-memory accesses before later
 // async-proxy (bulk copy) accesses
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
+
+// A unit of the row-staged kernels: its row, segment, first column x0 and cells.
+// RS: whole rows of that many cells.
+struct UnitAt {
+    int row, seg, x0, len;
+};
+template <int RS>
+__device__ __forceinline__ UnitAt unit_at(const KParams& p, int unit) {
+    UnitAt u{unit, 0, 0, RS ? RS : p.nx};
+    if (!RS && p.nseg > 1) {
+        u.row = unit / p.nseg;
+        u.seg = unit - u.row * p.nseg;
+        u.x0 = u.seg * p.seglen;
+        u.len = min(p.seglen, p.nx - u.x0);
+    }
+    return u;
+}
+
+// One thread: copies the Q source rows of a unit from the field F (unit
+// layout) into rows (slot order, RS or seglen columns each), completing on bar.
+// PULL: the rows (y - e_ay, z - e_az), read at x - e_ax; else the gather rows
+// (y + e_ay, z + e_az), read at x + e_ax.  The slots of the directions with one
+// (e_y, e_z) are consecutive: one copy per neighbouring row.
+template <class L, int RS, bool PULL, class T>
+__device__ __forceinline__ void stage_rows(T* rows, const T* __restrict__ F, const UnitAt& u, uint64_t* bar,
+                                           const KParams& p) {
+    const int y = u.row % p.ny, z = u.row / p.ny;
+    const int yp = y == p.ny - 1 ? 0 : y + 1, ym = y == 0 ? p.ny - 1 : y - 1;
+    const int zp = z == p.nz - 1 ? 0 : z + 1, zm = z == 0 ? p.nz - 1 : z - 1;
+    const int rs = RS ? RS : p.seglen;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        if (key_count<L>(k) == 0) continue;
+        // slots key_first(k) .. of the source row, periodic
+        const int ey = PULL ? k / 3 - 1 : 1 - k / 3, ez = PULL ? k % 3 - 1 : 1 - k % 3, s0 = key_first<L>(k);
+        const int ys = ey > 0 ? ym : (ey < 0 ? yp : y);
+        const int zs = ez > 0 ? zm : (ez < 0 ? zp : z);
+        const int su = RS ? zs * p.ny + ys : (zs * p.ny + ys) * p.nseg + u.seg;
+        bulk_load(rows + s0 * rs, F + ((int64_t)su * L::Q + s0) * rs,
+                  (uint32_t)(key_count<L>(k) * rs) * (uint32_t)sizeof(T), bar);
+    }
+}
+
+// The directions that read column x - 1 (NEG: x + 1) in a pull, by slot, 5 bits
+// each (9 of D3V27 at most), their number, and the velocity components by slot
+// (e + 1, 2 bits each); worked out once per lattice.
+template <class L>
+struct SlotDirs {
+    unsigned long long y, z, pos, neg;
+    int moving_x;
+    constexpr SlotDirs() : y(0), z(0), pos(0), neg(0), moving_x(0) {
+        int np = 0, nn = 0;
+        for (int a = 0; a < L::Q; ++a) {
+            const int s = pop_slot_calc<L>(a);
+            y |= (unsigned long long)(L::c(a, 1) + 1) << (2 * s);
+            z |= (unsigned long long)(L::c(a, 2) + 1) << (2 * s);
+            if (L::c(a, 0) > 0) pos |= (unsigned long long)s << (5 * np++);
+            if (L::c(a, 0) < 0) neg |= (unsigned long long)s << (5 * nn++);
+        }
+        moving_x = np;
+    }
+};
+
+// Halo values of a segment (nseg > 1): thread i < 2 moving_x fetches one value
+// of the field F that a cell at an end of the segment reads beyond it, and
+// halo_put writes it to its place in the halo arrays (left, then right, by
+// slot).  The fetch goes out when the unit's bulk copies do; the put follows a
+// unit later, so the load's latency is covered.
+template <class L, bool PULL, class T>
+__device__ __forceinline__ T halo_fetch(const T* __restrict__ F, const UnitAt& u, const KParams& p) {
+    constexpr SlotDirs<L> dirs{};
+    const int i = threadIdx.x;
+    const bool right = i >= dirs.moving_x;
+    const int k = right ? i - dirs.moving_x : i;
+    // a pull reads the left column along e_x > 0, a gather along e_x < 0
+    const int s = (int)(((right == PULL ? dirs.neg : dirs.pos) >> (5 * k)) & 31ull);
+    const int sy = (int)((dirs.y >> (2 * s)) & 3ull) - 1, sz = (int)((dirs.z >> (2 * s)) & 3ull) - 1;
+    const int y = u.row % p.ny, z = u.row / p.ny;
+    int ys = PULL ? y - sy : y + sy, zs = PULL ? z - sz : z + sz;
+    ys = ys < 0 ? ys + p.ny : (ys >= p.ny ? ys - p.ny : ys);
+    zs = zs < 0 ? zs + p.nz : (zs >= p.nz ? zs - p.nz : zs);
+    int x = right ? u.x0 + u.len : u.x0 - 1;
+    x = x < 0 ? p.nx - 1 : (x >= p.nx ? 0 : x);
+    const int seg = x / p.seglen;
+    return __ldg(F + (((int64_t)(zs * p.ny + ys) * p.nseg + seg) * L::Q + s) * p.seglen + (x - seg * p.seglen));
+}
+template <class L, bool PULL, class T>
+__device__ __forceinline__ void halo_put(T* hal, T v) {
+    constexpr SlotDirs<L> dirs{};
+    const int i = threadIdx.x;
+    const bool right = i >= dirs.moving_x;
+    const int k = right ? i - dirs.moving_x : i;
+    const int s = (int)(((right == PULL ? dirs.neg : dirs.pos) >> (5 * k)) & 31ull);
+    hal[(right ? L::Q : 0) + s] = v;
+}
+template <class L>
+__device__ __forceinline__ bool halo_thread() {
+    constexpr SlotDirs<L> dirs{};
+    return (int)threadIdx.x < 2 * dirs.moving_x;
+}
+// Bytes of the halo arrays of a stage (0 for whole rows).
+__host__ __device__ __forceinline__ int halo_bytes(int Q, int nseg, int esize) {
+    return nseg == 1 ? 0 : (2 * Q * esize + 15) / 16 * 16;
+}
 
 // Bytes [b0, b1) of the 16-byte aligned window covering elements [g0, g1).
 __device__ __forceinline__ void window_bytes(uint32_t g0, uint32_t g1, int esize, uint64_t& b0, uint64_t& b1) {

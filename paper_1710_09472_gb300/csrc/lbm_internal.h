@@ -106,12 +106,16 @@ __host__ __device__ constexpr int shell_first(int s) {
 }
 
 // ---------------------------------------------------------------------------
-// Population storage.  Row r = z ny + y keeps its Q directions one after
-// another, nx values each: direction a of cell (x, r) is element
-// (r Q + slot(a)) nx + x.  The slots order the directions by (e_ay, e_az)
+// Population storage.  A row r = z ny + y is one unit, or is cut into nseg
+// units of seglen columns (set_units, lbm_api.cu); unit u = r nseg + segment
+// keeps its Q directions one after another, seglen values each: direction a of
+// cell (x, r) is element (u Q + slot(a)) seglen + x - x0, with x0 = segment
+// seglen.  seglen is a multiple of kPitch except in short rows, so the units
+// move by 16-byte bulk copies whatever nx is; the columns beyond nx are never
+// read as values.  The slots order the directions by (e_ay, e_az)
 // (key 3 (e_ay + 1) + e_az + 1, ties by a), so the directions that a row
 // pulls from one neighbouring row (y - e_ay, z - e_az) are consecutive slots
-// of that row, and a row's Q directions are one contiguous block.
+// of that row, and a unit's Q directions are one contiguous block.
 // ---------------------------------------------------------------------------
 template <class L>
 __host__ __device__ constexpr int pop_key(int a) {
@@ -261,9 +265,24 @@ struct StoreBF16 {
 // ~1e-15: an FP32-rounded W1 would leak a fixed fraction ~1e-7 of the
 // momentum in every collision, which compounds over thousands of steps.
 // ---------------------------------------------------------------------------
+// Units: rows of kMinStagedRow cells or more are padded to a multiple of kPitch
+// columns (16 bytes of the 16-bit storages).  Shorter rows run on the general
+// kernels and stay as they are.
+constexpr int kPitch = 8, kMinStagedRow = 32;
+// A row is one unit of the staged kernels while three copies of it (all
+// directions) fit kRowSmem bytes; a longer row is cut (set_units, lbm_api.cu).
+constexpr int kRowSmem = 64 * 1024;
+template <class L, class S>
+__host__ __device__ constexpr bool whole_row(int nx) {
+    return 3 * L::Q * nx * S::kBytes <= kRowSmem;
+}
+
 struct KParams {
     int nx, ny, nz;
-    int64_t N;
+    int nseg, seglen;  // units per row and columns of a unit (see pop_slot)
+    int qm1;           // Q - 1
+    int nxp;           // nseg seglen: row pitch of the per-cell fields E and dL/dE in device memory
+    int64_t N, NP;     // cells; cells with the padding, ny nz nxp
     float omega;  // 1 / tau
     float tau;
     float rho0;
@@ -278,19 +297,20 @@ struct KParams {
     uint32_t step;  // global step index of this launch (stochastic rounding stream)
     uint32_t seed;
     // Bounce-back link buffer G (see lbm_kernels.cu): byte offset of G inside
-    // a state buffer, per-cell first link slot, per-row first link slot
-    // (ny * nz + 1 entries) and the largest number of links in one row.
+    // a state buffer, per-cell first link slot, per-unit first link slot
+    // (ny * nz * nseg + 1 entries) and the largest number of links in a unit.
     uint64_t gofs;
     const uint32_t* lbase;
     const uint32_t* rowG;
-    // per link slot k: x | b << 24, the x coordinate of its fluid cell and
-    // its outgoing direction b (the row-staged kernels' link passes)
+    // per link slot of fluid cell x and outgoing direction b, for the link
+    // passes of the row-staged kernels (see link_desc)
     const uint32_t* ldesc;
     int max_row_links;
-    // per row, the cells in the order the row-staged kernels give them to
+    // per unit, the cells in the order the row-staged kernels give them to
     // threads: entry 0 the number of fluid cells nf, entries 1..7 zero, then
-    // the fluid x ascending and the solid x ascending (lorder entries per row,
-    // a multiple of 8; null when nx > 65535)
+    // the fluid x ascending and the solid x ascending, relative to the unit's
+    // first cell (lorder entries per unit, a multiple of 8; null for the rows
+    // that the staged kernels do not take)
     const uint16_t* rorder;
     int lorder;
     // byte offset of the link buffer inside an adjoint field (reverse sweep)
@@ -311,6 +331,25 @@ struct KParams {
     float lmu_K[4];
 };
 
+// A staged unit holds its columns x0 .. x0 + seglen - 1 of every slot, and what
+// its cells read beyond them: nothing for a whole row (the periodic wrap is an
+// index into the row), else the columns left and right of it in two halo
+// arrays of one value per slot.  Their staged positions in a link descriptor:
+constexpr int kPosLeft = 2046, kPosRight = 2047;
+
+// Link descriptor: slot(b), slot(bbar), the unit column xl of the fluid cell
+// and that of its solid neighbour (or kPosLeft, kPosRight), so that a link pass
+// needs two shifts and a multiply-add per staged address.  The columns have 11
+// bits: units have at most kMaxUnit columns.
+constexpr int kMaxUnit = 2040;
+__host__ __device__ __forceinline__ uint32_t link_desc(int slot_b, int slot_bbar, int xl, int pos) {
+    return (uint32_t)slot_b | (uint32_t)slot_bbar << 5 | (uint32_t)xl << 10 | (uint32_t)pos << 21;
+}
+__host__ __device__ __forceinline__ int desc_slot(uint32_t d) { return (int)(d & 31u); }
+__host__ __device__ __forceinline__ int desc_slot_bar(uint32_t d) { return (int)((d >> 5) & 31u); }
+__host__ __device__ __forceinline__ int desc_x(uint32_t d) { return (int)((d >> 10) & 0x7FFu); }
+__host__ __device__ __forceinline__ int desc_pos(uint32_t d) { return (int)(d >> 21); }
+
 struct Launch {
     dim3 grid, block;
 };
@@ -319,14 +358,14 @@ struct Launch {
 int launch_build_neighbors(int vel, const uint8_t* mask, uint32_t* nbr, unsigned long long* fluid_count,
                            const KParams& p, cudaStream_t s);
 // Link buffer layout: lbase[cell] (exclusive prefix of outgoing-link counts),
-// rowG[0..ny*nz]; needs a temporary of *temp_bytes (queried with temp == NULL).
+// rowG[0..ny*nz*nseg]; needs a temporary of *temp_bytes (queried with temp == NULL).
 // Bounded-wait probe (writes code 3 into *status when its wait runs out).
 int launch_wait_probe(int* status, long long limit, cudaStream_t s);
-// Per-link descriptors ldesc[k] = x | b << 24 (needs lbase).
 // FP32 field in the populations' slot layout -> direction-major out[a * N + cell].
 int launch_unslot(int vel, const float* in, float* out, const KParams& p, cudaStream_t s);
-// Per-row cell order (fluid cells first) for the row-staged kernels.
+// Per-unit cell order (fluid cells first) for the row-staged kernels.
 int launch_build_row_order(const uint32_t* nbr, uint16_t* rorder, const KParams& p, cudaStream_t s);
+// Per-link descriptors (link_desc; needs lbase).
 int launch_build_link_desc(int vel, const uint32_t* nbr, const uint32_t* lbase, uint32_t* ldesc, const KParams& p,
                            cudaStream_t s);
 int launch_build_links(int vel, const uint32_t* nbr, uint32_t* lbase, uint32_t* rowG, void* temp,
@@ -365,9 +404,9 @@ int launch_adjoint_step(int vel, int storage, int force, bool efield, bool in_wi
                         const float* w_rho, const float* w_j, float* gE, double* slots, const KParams& p,
                         cudaStream_t s);
 int launch_reduce_slots(const double* slots, int64_t n_blocks, int n_slots, double* out, cudaStream_t s);
-// acc[i] += part[i] (FP64) and part[i] = 0 for i < n: folds the reverse
-// steps' FP32 dL/dE partials into the caller's FP64 gradient.
-int launch_fold_partials(float* part, double* acc, int64_t n, cudaStream_t s);
+// acc += part (FP64) and part = 0, D components: folds the reverse steps' FP32
+// dL/dE partials (rows of nxp) into the caller's FP64 gradient (rows of nx).
+int launch_fold_partials(float* part, double* acc, int D, const KParams& p, cudaStream_t s);
 int launch_accumulate_totals(const double* partials, int64_t n_partials, double* acc4, cudaStream_t s);
 
 // Local chemical-potential table (lbm_fd.cu): for the FD weight of dimension D
@@ -398,7 +437,7 @@ struct AdjWorkspace {
     double* red = nullptr;
     float* wstage = nullptr;  // loss weights staged from the host
     size_t wstage_bytes = 0;
-    float* gpart = nullptr;   // FP32 dL/dE partials of the latest reverse steps (D N)
+    float* gpart = nullptr;   // FP32 dL/dE partials of the latest reverse steps (D NP, padded rows)
     size_t gpart_bytes = 0;
     size_t held() const {
         return states.size() * state_bytes + 2 * lam_bytes + sizeof(double) * (size_t)nslot + wstage_bytes +
@@ -412,6 +451,8 @@ struct lbm_ctx {
     lbm_lattice lat{};
     int D = 0, Q = 0;
     int64_t nx = 1, ny = 1, nz = 1, N = 0;
+    int nseg = 1, seglen = 1;      // units (KParams)
+    int64_t nxp = 1, NP = 0;
     int64_t n_fluid = 0;
     int storage = 0;
     bool stochastic = false;  // stochastic rounding of FP16/BF16 stores
@@ -429,9 +470,9 @@ struct lbm_ctx {
     int cur = 0;
     uint32_t* nbr = nullptr;
     uint32_t* lbase = nullptr;     // per-cell first slot in the link buffer
-    uint32_t* rowG = nullptr;      // per-row first slot (ny * nz + 1)
-    uint32_t* ldesc = nullptr;     // per link slot: x | b << 24
-    uint16_t* rorder = nullptr;    // per row: fluid count, then fluid x, then solid x (lorder entries)
+    uint32_t* rowG = nullptr;      // per-unit first slot (ny * nz * nseg + 1)
+    uint32_t* ldesc = nullptr;     // per link slot: its descriptor (link_desc)
+    uint16_t* rorder = nullptr;    // per unit: fluid count, then fluid x, then solid x (lorder entries)
     int lorder = 0;
     int64_t n_links = 0;           // outgoing links into solid cells
     int max_row_links = 0;

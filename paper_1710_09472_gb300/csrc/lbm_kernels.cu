@@ -3,15 +3,15 @@
 // Lorentz forcing step, moments with FP64 reductions, and the population
 // read-back.
 //
-// Layout: populations are structure-of-arrays, P[a * N + cell] with
-// cell = (z * ny + y) * nx + x.  P holds post-collision values ("pull"
+// Layout: a row (or segment of a long row) keeps its directions one after
+// another (see pop_slot).  P holds post-collision values ("pull"
 // scheme): the state f(x, t) of the method is f_a(x, t) = P_a(x - e_a) when
 // x - e_a is fluid.
 // Halfway bounce-back (Sec. 9.3, 9.4) uses a link buffer G stored after P in
 // the same state buffer: every link from a fluid cell x into a solid cell
 // (x + e_b solid) owns one slot, numbered in cell order (lbase[x] + rank of b
 // among x's outgoing links), so the links of one row form a contiguous range
-// rowG[r] .. rowG[r+1].  The collision stores f*_b(x) there, and the next
+// rowG[u] .. rowG[u+1] (u a row, or a segment of a long row).  The collision stores f*_b(x) there, and the next
 // step reads it back as f_bbar(x).
 #include <algorithm>
 #include <cstdio>
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kBlock) k_neighbors(const uint8_t* __restrict_
             fluid = 1;
 #pragma unroll
             for (int a = 1; a < L::Q; ++a)
-                if (mask[dev::shifted<L>(c, a, -1)]) m |= (1u << a);
+                if (mask[dev::shifted<L>(p, c, a, -1)]) m |= (1u << a);
         }
         nbr[c.cell] = m;
     }
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kBlock) k_init(typename S::T* __restrict__ P, 
                 S::put(G + link_slot(base, o, b), heq_unscaled<L>(p, opposite(b), r0, u0) * p.scale);
             } else {
                 float r1 = r0, u1[3] = {u0[0], u0[1], u0[2]};
-                if (b != 0) fields(dev::shifted<L>(c, b, +1), r1, u1);
+                if (b != 0) fields(dev::shifted<L>(p, c, b, +1), r1, u1);
                 v = heq_unscaled<L>(p, b, r1, u1);
             }
         }
@@ -111,8 +111,9 @@ __global__ void __launch_bounds__(kBlock) k_link_counts(const uint32_t* __restri
     cnt[c.cell] = (m & kSolidBit) ? 0u : (uint32_t)__popc(outgoing<L::Q>(m));
 }
 
-// Descriptor of every link slot: the x coordinate of its fluid cell and its
-// outgoing direction b, ldesc[slot] = x | b << 24.
+// Descriptor of every link slot (link_desc): the slots of its outgoing
+// direction b and of bbar, the unit column of its fluid cell and the staged
+// position of the solid cell behind the link.
 template <class L>
 __global__ void __launch_bounds__(kBlock) k_link_desc(const uint32_t* __restrict__ nbr,
                                                       const uint32_t* __restrict__ lbase,
@@ -123,33 +124,42 @@ __global__ void __launch_bounds__(kBlock) k_link_desc(const uint32_t* __restrict
     if ((m & kSolidBit) || m == 0u) return;
     const uint32_t o = outgoing<L::Q>(m);
     const uint32_t base = lbase[c.cell];
+    const int xl = c.x % p.seglen, last = min(p.seglen, p.nx - (c.x - xl)) - 1;
+    const int left = xl > 0 ? xl - 1 : (p.nseg == 1 ? p.nx - 1 : kPosLeft);
+    const int right = xl < last ? xl + 1 : (p.nseg == 1 ? 0 : kPosRight);
 #pragma unroll
     for (int b = 1; b < L::Q; ++b)
-        if ((o >> b) & 1u) ldesc[link_slot(base, o, b)] = (uint32_t)c.x | ((uint32_t)b << 24);
+        if ((o >> b) & 1u) {
+            const int ex = L::c(b, 0);
+            ldesc[link_slot(base, o, b)] =
+                link_desc(pop_slot<L>(b), pop_slot<L>(opposite(b)), xl, ex < 0 ? left : (ex > 0 ? right : xl));
+        }
 }
 
-// Cell order of each row for the row-staged kernels: entry 0 the number of
+// Cell order of each unit for the row-staged kernels: entry 0 the number of
 // fluid cells nf, entries 1..7 zero, entries 8 .. 8 + nf - 1 the fluid x
-// ascending, then the solid x ascending, then zeros up to lorder.  One warp
-// per row.
+// ascending, then the solid x ascending, then zeros up to lorder; x counts
+// from the unit's first cell.  One warp per unit.
 __global__ void __launch_bounds__(kBlock) k_row_order(const uint32_t* __restrict__ nbr, uint16_t* __restrict__ ord,
                                                       KParams p) {
-    const int64_t R = (int64_t)p.ny * p.nz;
+    const int64_t U = (int64_t)p.ny * p.nz * p.nseg;
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < R; r += nwarps) {
-        const uint32_t* m = nbr + r * p.nx;
+    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < U; r += nwarps) {
+        const int first = (int)(r % p.nseg) * p.seglen;
+        const int len = min(p.seglen, p.nx - first);
+        const uint32_t* m = nbr + (r / p.nseg) * p.nx + first;
         uint16_t* o = ord + r * p.lorder;
         int nf = 0;
-        for (int x0 = 0; x0 < p.nx; x0 += 32) {
+        for (int x0 = 0; x0 < len; x0 += 32) {
             const int x = x0 + lane;
-            nf += __popc(__ballot_sync(0xffffffffu, x < p.nx && !(m[x] & kSolidBit)));
+            nf += __popc(__ballot_sync(0xffffffffu, x < len && !(m[x] & kSolidBit)));
         }
         int nfl = 0, nso = nf;  // entries written so far: fluid, and nf + solid
-        for (int x0 = 0; x0 < p.nx; x0 += 32) {
+        for (int x0 = 0; x0 < len; x0 += 32) {
             const int x = x0 + lane;
-            const bool in = x < p.nx;
+            const bool in = x < len;
             const bool fluid = in && !(m[x] & kSolidBit);
             const unsigned bf = __ballot_sync(0xffffffffu, fluid), bs = __ballot_sync(0xffffffffu, in && !fluid);
             if (fluid) o[8 + nfl + __popc(bf & below)] = (uint16_t)x;
@@ -158,20 +168,20 @@ __global__ void __launch_bounds__(kBlock) k_row_order(const uint32_t* __restrict
             nso += __popc(bs);
         }
         if (lane < 8) o[lane] = lane == 0 ? (uint16_t)nf : (uint16_t)0;
-        for (int k = 8 + p.nx + lane; k < p.lorder; k += 32) o[k] = 0;
+        for (int k = 8 + len + lane; k < p.lorder; k += 32) o[k] = 0;
     }
 }
 
 template <class L>
 __global__ void k_row_starts(const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ lbase,
                              uint32_t* __restrict__ rowG, KParams p) {
-    const int64_t R = (int64_t)p.ny * p.nz;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r <= R; r += (int64_t)gridDim.x * blockDim.x) {
-        if (r < R) {
-            rowG[r] = lbase[r * p.nx];
+    const int64_t U = (int64_t)p.ny * p.nz * p.nseg;
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r <= U; r += (int64_t)gridDim.x * blockDim.x) {
+        if (r < U) {
+            rowG[r] = lbase[(r / p.nseg) * p.nx + (r % p.nseg) * p.seglen];
         } else {
             const uint32_t m = nbr[p.N - 1];
-            rowG[R] = lbase[p.N - 1] + ((m & kSolidBit) ? 0u : (uint32_t)__popc(outgoing<L::Q>(m)));
+            rowG[U] = lbase[p.N - 1] + ((m & kSolidBit) ? 0u : (uint32_t)__popc(outgoing<L::Q>(m)));
         }
     }
 }
@@ -373,8 +383,8 @@ int launch_build_links(int vel, const uint32_t* nbr, uint32_t* lbase, uint32_t* 
         return 1;
     });
     cub::DeviceScan::ExclusiveSum(temp, *temp_bytes, lbase, lbase, n, s);
-    const int64_t R = (int64_t)p.ny * p.nz;
-    const int blocks = (int)((R + 1 + 255) / 256 < 4096 ? (R + 1 + 255) / 256 : 4096);
+    const int64_t U = (int64_t)p.ny * p.nz * p.nseg;
+    const int blocks = (int)((U + 1 + 255) / 256 < 4096 ? (U + 1 + 255) / 256 : 4096);
     dispatch_lattice(vel, [&](auto lat) {
         using L = decltype(lat);
         k_row_starts<L><<<blocks, 256, 0, s>>>(nbr, lbase, rowG, p);
@@ -412,8 +422,8 @@ int launch_unslot(int vel, const float* in, float* out, const KParams& p, cudaSt
 }
 
 int launch_build_row_order(const uint32_t* nbr, uint16_t* rorder, const KParams& p, cudaStream_t s) {
-    const int64_t R = (int64_t)p.ny * p.nz;
-    const int64_t blocks = std::min<int64_t>((R * 32 + kBlock - 1) / kBlock, 65535);
+    const int64_t U = (int64_t)p.ny * p.nz * p.nseg;
+    const int64_t blocks = std::min<int64_t>((U * 32 + kBlock - 1) / kBlock, 65535);
     k_row_order<<<(unsigned)blocks, kBlock, 0, s>>>(nbr, rorder, p);
     return 1;
 }

@@ -395,13 +395,14 @@ __device__ __forceinline__ void round_all(const float* out, uint32_t cell, const
     }
 }
 
+// pcell: row * nxp + x, the cell's place in the padded field
 template <class L>
-__device__ __forceinline__ void load_E(const float* __restrict__ Ef, bool ef, const KParams& p, uint32_t cell,
+__device__ __forceinline__ void load_E(const float* __restrict__ Ef, bool ef, const KParams& p, int64_t pcell,
                                        float* E) {
     if (ef) {
-        E[0] = __ldg(Ef + cell);
-        E[1] = (L::D >= 2) ? __ldg(Ef + p.N + cell) : 0.f;
-        E[2] = (L::D == 3) ? __ldg(Ef + 2 * p.N + cell) : 0.f;
+        E[0] = __ldg(Ef + pcell);
+        E[1] = (L::D >= 2) ? __ldg(Ef + p.NP + pcell) : 0.f;
+        E[2] = (L::D == 3) ? __ldg(Ef + 2 * p.NP + pcell) : 0.f;
     } else {
         E[0] = p.E[0];
         E[1] = p.E[1];
@@ -435,7 +436,7 @@ __global__ void __launch_bounds__(kBlock) k_step(const typename S::T* __restrict
     float h[L::Q];
     dev::pull<L, S>(Pin, p, m, c, h);
     float E[3];
-    load_E<L>(Ef, EF, p, c.cell, E);
+    load_E<L>(Ef, EF, p, c.pcell, E);
     float out[L::Q];
     // the local-mu model is built for D2V9 and D3V19 (the host refuses others)
     constexpr bool kLmu = L::Q == 9 || L::Q == 19;
@@ -456,47 +457,55 @@ __global__ void __launch_bounds__(kBlock) k_step(const typename S::T* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// Row-staged step kernel (used when a whole x-row of one direction is a
-// whole number of 16-byte chunks and the stages fit shared memory).  A
-// persistent block walks rows r = blockIdx.x, blockIdx.x + gridDim.x, ...:
-//  - the Q source rows P_a(y - e_ay, z - e_az, :) of the row (one contiguous
-//    block of consecutive slots per neighbouring row, at most 9 copies), its
-//    cell order and its ranges of the link buffer and of the link
-//    descriptors arrive by bulk asynchronous copies into a ring of STAGES
-//    stages, STAGES - 1 rows ahead of the row being computed.  One thread,
-//    lane 0 of the last warp, arms the stage's mbarrier with the byte count
-//    and issues the copies.  A bulk copy holds its issuing thread for many
-//    cycles, so the issuer is the warp with the least cell work (the order
-//    puts the solid cells, and the cells of a second pass, on the first
-//    warps);
-//  - one pass over the row's links writes each bounced value f*_b(x) into the
+// Row-staged step kernel.  A persistent block walks units u = blockIdx.x,
+// blockIdx.x + gridDim.x, ...; a unit is a whole x-row, or a segment of a long
+// one:
+//  - the Q source rows P_a(y - e_ay, z - e_az, :) of the unit, its cell order
+//    and its ranges of the link buffer and of the link descriptors arrive by
+//    bulk asynchronous copies into a ring of STAGES stages, STAGES - 1 units
+//    ahead of the one being computed (the consecutive slots of one neighbouring
+//    row are one contiguous block: at most 9 copies).  One thread, lane 0 of
+//    the last warp, arms the stage's mbarrier with the byte count and issues
+//    the copies.  A bulk copy holds its issuing thread for many cycles, so the
+//    issuer is the warp with the least cell work (the order puts the solid
+//    cells, and the cells of a second pass, on the first warps).  The columns
+//    beside a segment come by plain loads of a few threads (halo_fetch): as
+//    wider copies, one per direction, they made the issuing thread the
+//    bottleneck (2048 x 1024 cells of D2V9 FP32: 37.8 us against 31.6 for
+//    whole rows of 1024);
+//  - one pass over the unit's links writes each bounced value f*_b(x) into the
 //    staged slot that the pull of direction bbar at x reads (the slot of the
 //    solid neighbour), so the cells pull without link logic;
-//  - thread i takes the i-th cell of the row's order (the fluid cells first,
+//  - thread i takes the i-th cell of the unit's order (the fluid cells first,
 //    fixed by the geometry), so the collision runs on full warps; solid cells
 //    only write zeros;
-//  - f_a(x) is read from the ring at x - e_ax (periodic wrap in x is a
-//    shared-memory index); results go into a shared-memory output row set
-//    that leaves by one bulk store (the row's Q slots are contiguous);
-//  - one pass over the row's links copies the outgoing values f*_b(x) from
-//    the output rows into the row's contiguous range of the link buffer.
-// Two block barriers per row; a stage is refilled after the first barrier of
-// the row that follows its own.  Every wait on an mbarrier is bounded; one that
-// runs out writes a code to p.status, the block stops issuing copies, and the
-// kernel carries on (its results are then invalid, but it ends and no access
-// leaves its buffers).
+//  - f_a(x) is read from the ring at x - e_ax (the periodic wrap in x of a
+//    whole row is a shared-memory index); results go into a shared-memory
+//    output row set that leaves by one bulk store (the unit's Q slots are
+//    contiguous);
+//  - one pass over the unit's links copies the outgoing values f*_b(x) from
+//    the output rows into the unit's contiguous range of the link buffer.
+// Two block barriers per unit; a stage is refilled after the first barrier of
+// the unit that follows its own.  Every wait on an mbarrier is bounded; one
+// that runs out writes a code to p.status, the block stops issuing copies, and
+// the kernel carries on (its results are then invalid, but it ends and no
+// access leaves its buffers).
+//
+// Rows whose length is not a whole number of 16-byte chunks are staged with
+// their padding (kPitch): on the general kernel such a box took 2.7 times as
+// long per cell (250 x 128 x 128 D3V19 FP16: 0.112 ms per 2.36 M cells against
+// 0.042 ms at nx = 256).
 // ---------------------------------------------------------------------------
 
-// Shared-memory layout of one stage: the Q source rows in slot order (row s
-// at s rs, rs = nx, so that consecutive slots of one neighbouring row land
-// with one copy), the row's cell order (lorder 16-bit entries), its range of
-// the link buffer (gcap bytes) and of the link descriptors (dcap bytes), both
-// as 16-byte aligned windows.
+// Shared-memory layout of one stage: the Q source rows in slot order (slot s
+// at s rs), the unit's cell order (lorder 16-bit entries), its range of the
+// link buffer (gcap bytes) and of the link descriptors (dcap bytes), both as
+// 16-byte aligned windows, and the halo arrays of a segment.
 template <class L, class S>
 struct StageLayout {
-    int nx, rs, lorder, gcap, dcap;  // row length, shared-memory row stride (elements), order entries
+    int rs, lorder, gcap, dcap, hb;  // shared-memory row stride (elements), order entries, halo bytes
     __device__ __forceinline__ int rows_bytes() const { return L::Q * rs * S::kBytes; }
-    __device__ __forceinline__ int bytes() const { return rows_bytes() + 2 * lorder + gcap + dcap; }
+    __device__ __forceinline__ int bytes() const { return rows_bytes() + 2 * lorder + gcap + dcap + hb; }
     __device__ __forceinline__ typename S::T* rows(unsigned char* st) const {
         return reinterpret_cast<typename S::T*>(st);
     }
@@ -509,41 +518,30 @@ struct StageLayout {
     __device__ __forceinline__ uint32_t* descs(unsigned char* st) const {
         return reinterpret_cast<uint32_t*>(st + rows_bytes() + 2 * lorder + gcap);
     }
+    __device__ __forceinline__ typename S::T* halo(unsigned char* st) const {
+        return reinterpret_cast<typename S::T*>(st + rows_bytes() + 2 * lorder + gcap + dcap);
+    }
 };
 
-// One thread: arms a stage's mbarrier with the byte count of row `row`
+// One thread: arms a stage's mbarrier with the byte count of unit `unit`
 // (links [g0, g1)), records the first elements of its two windows, and issues
-// the row's copies into stage st, all completing on bar: per neighbouring row
-// (y - e_ay, z - e_az) the block of slots of the directions with that
-// (e_ay, e_az), the cell order, the link window and the descriptor window.  The window
-// starts are written before the barrier is armed, so the arrive releases them
-// to the waiting threads.
-template <class L, class S>
-__device__ __forceinline__ void stage_row(unsigned char* st, const StageLayout<L, S>& lay, uint64_t* bar,
-                                          const typename S::T* __restrict__ Pin, int row, uint32_t g0, uint32_t g1,
-                                          uint32_t* gstart, uint32_t* dstart, const KParams& p) {
-    const uint32_t row_bytes = (uint32_t)p.nx * S::kBytes;
+// the unit's copies into stage st, all completing on bar: the source rows
+// (dev::stage_rows), the cell order, the link window and the descriptor
+// window.  The window starts are written before the barrier is armed, so the
+// arrive releases them to the waiting threads.
+template <class L, class S, int RS>
+__device__ __forceinline__ void stage_unit(unsigned char* st, const StageLayout<L, S>& lay, uint64_t* bar,
+                                           const typename S::T* __restrict__ Pin, int unit, uint32_t g0, uint32_t g1,
+                                           uint32_t* gstart, uint32_t* dstart, const KParams& p) {
     uint64_t gb0, gb1, db0, db1;
     dev::window_bytes(g0, g1, S::kBytes, gb0, gb1);
     dev::window_bytes(g0, g1, 4, db0, db1);
     *gstart = (uint32_t)(gb0 / S::kBytes);
     *dstart = (uint32_t)(db0 / 4);
-    dev::mbar_expect_tx(bar, L::Q * row_bytes + 2u * (uint32_t)lay.lorder + (uint32_t)(gb1 - gb0) +
+    dev::mbar_expect_tx(bar, (uint32_t)lay.rows_bytes() + 2u * (uint32_t)lay.lorder + (uint32_t)(gb1 - gb0) +
                                  (uint32_t)(db1 - db0));
-    const int y = row % p.ny, z = row / p.ny;
-    const int yp = y == p.ny - 1 ? 0 : y + 1, ym = y == 0 ? p.ny - 1 : y - 1;
-    const int zp = z == p.nz - 1 ? 0 : z + 1, zm = z == 0 ? p.nz - 1 : z - 1;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        if (key_count<L>(k) == 0) continue;
-        // slots key_first(k) .. of source row (y - e_y, z - e_z), periodic
-        const int ey = k / 3 - 1, ez = k % 3 - 1, s0 = key_first<L>(k);
-        const int ys = ey > 0 ? ym : (ey < 0 ? yp : y);
-        const int zs = ez > 0 ? zm : (ez < 0 ? zp : z);
-        dev::bulk_load(lay.rows(st) + s0 * lay.rs, Pin + ((int64_t)(zs * p.ny + ys) * L::Q + s0) * p.nx,
-                       (uint32_t)key_count<L>(k) * row_bytes, bar);
-    }
-    dev::bulk_load(lay.order(st), p.rorder + (int64_t)row * lay.lorder, 2u * (uint32_t)lay.lorder, bar);
+    dev::stage_rows<L, RS, true>(lay.rows(st), Pin, dev::unit_at<RS>(p, unit), bar, p);
+    dev::bulk_load(lay.order(st), p.rorder + (int64_t)unit * lay.lorder, 2u * (uint32_t)lay.lorder, bar);
     if (gb1 > gb0)
         dev::bulk_load(lay.links(st), reinterpret_cast<const unsigned char*>(Pin) + p.gofs + gb0,
                        (uint32_t)(gb1 - gb0), bar);
@@ -557,7 +555,7 @@ __device__ __forceinline__ void stage_row(unsigned char* st, const StageLayout<L
 // into separate output rows: 46 instead of 66 KB of shared memory, four
 // blocks per SM instead of three, 0.458 against 0.468 ms per 256^3 step.  The
 // stage is refilled only after the row's bulk store has read it and every
-// thread has passed its link copies (the first barrier of the next row).  For
+// thread has passed its link copies (the first barrier of the next unit).  For
 // FP16 the extra barrier and the 256-thread blocks cost more than the freed
 // memory gains (0.321 against 0.258 ms), so 16-bit storage keeps output rows.
 template <class S, int RS, bool LMU>
@@ -569,27 +567,27 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
                                                    int gcap, int dcap, KParams p) {
     using T = typename S::T;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int nx = p.nx;
-    const int rs = RS ? RS : nx;  // shared-memory row stride (= nx): a constant for the common row lengths
+    // RS: whole rows of that many cells, a compile-time stride; 0: a run-time one, whole rows or segments
+    const int rs = RS ? RS : p.seglen;
+    const bool halo = !RS && p.nseg > 1;
     // FP32 rows of 256 cells write their outputs over the row's own stage
     // (no output rows: four blocks per SM instead of three); see kInPlaceOut
     constexpr bool kInPlace = kInPlaceOut<S, RS, LMU>;
-    const StageLayout<L, S> lay{nx, rs, p.lorder, gcap, dcap};
+    const StageLayout<L, S> lay{rs, p.lorder, gcap, dcap, RS ? 0 : dev::halo_bytes(L::Q, p.nseg, S::kBytes)};
     const int sbytes = lay.bytes();
     T* outrow = reinterpret_cast<T*>(smem_raw + STAGES * sbytes);
     __shared__ __align__(8) uint64_t bar[STAGES];
     __shared__ uint32_t gstart[STAGES], dstart[STAGES];
     T* Gout = reinterpret_cast<T*>(reinterpret_cast<char*>(Pout) + p.gofs);
-    const uint32_t row_bytes = (uint32_t)nx * S::kBytes;
-    const int R = p.ny * p.nz;
+    const int U = p.ny * p.nz * (RS ? 1 : p.nseg);
     const int G = gridDim.x;
     const bool leader = threadIdx.x == 0;
     const bool issuer = (int)threadIdx.x == (int)blockDim.x - 32;  // lane 0 of the last warp
-    auto range = [&](int row, uint32_t& g0, uint32_t& g1) {
+    auto range = [&](int unit, uint32_t& g0, uint32_t& g1) {
         g0 = g1 = 0u;
-        if (row < R) {
-            g0 = __ldg(p.rowG + row);
-            g1 = __ldg(p.rowG + row + 1);
+        if (unit < U) {
+            g0 = __ldg(p.rowG + unit);
+            g1 = __ldg(p.rowG + unit + 1);
         }
     };
     if (leader) {
@@ -597,26 +595,30 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
         for (int k = 0; k < STAGES; ++k) dev::mbar_init(&bar[k], 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    static_assert(STAGES == 2, "the halo values are fetched one unit ahead");
+    if (halo && dev::halo_thread<L>())
+        dev::halo_put<L, true>(lay.halo(smem_raw),
+                               dev::halo_fetch<L, true>(Pin, dev::unit_at<RS>(p, blockIdx.x), p));
     __syncthreads();
     if (issuer) {
 #pragma unroll
         for (int k = 0; k < STAGES - 1; ++k) {
-            const int rk = blockIdx.x + k * G;
-            if (rk < R) {
+            const int uk = blockIdx.x + k * G;
+            if (uk < U) {
                 uint32_t g0, g1;
-                range(rk, g0, g1);
-                stage_row<L, S>(smem_raw + k * sbytes, lay, &bar[k], Pin, rk, g0, g1, &gstart[k], &dstart[k], p);
+                range(uk, g0, g1);
+                stage_unit<L, S, RS>(smem_raw + k * sbytes, lay, &bar[k], Pin, uk, g0, g1, &gstart[k], &dstart[k], p);
             }
         }
     }
     int it = 0;
     bool ok = true;  // false once a wait has run out (the same in every thread after the first barrier)
-    for (int r = blockIdx.x; r < R; r += G, ++it) {
+    for (int u = blockIdx.x; u < U; u += G, ++it) {
         const int cs = it % STAGES;
-        const int rn = r + (STAGES - 1) * G;       // the row refilled during this one ...
-        const int sn = (it + STAGES - 1) % STAGES;  // ... into the stage of the previous row
-        uint32_t g0, g1;  // this row's links
-        range(r, g0, g1);
+        const int un = u + (STAGES - 1) * G;       // the unit fetched during this one ...
+        const int sn = (it + STAGES - 1) % STAGES;  // ... into the stage of the previous unit
+        uint32_t g0, g1;  // this unit's links
+        range(u, g0, g1);
         if (ok && !dev::mbar_wait(&bar[cs], (uint32_t)(it / STAGES) & 1u)) {
             ok = false;
             if (p.status) atomicExch(p.status, 1);
@@ -624,25 +626,30 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
         }
         unsigned char* st = smem_raw + cs * sbytes;
         T* buf = lay.rows(st);
-        T* orow = kInPlace ? buf : outrow;  // where this row's outputs go
+        T* orow = kInPlace ? buf : outrow;  // where this unit's outputs go
         const uint16_t* ord = lay.order(st);
         const uint32_t* desc = lay.descs(st);
         const uint32_t d0 = dstart[cs];
-        dev::patch_links<L, true>(buf, nx, rs, lay.links(st), gstart[cs], g0, g1, desc, d0);
-        dev::bulk_wait_read();  // this thread's bulk stores of the previous row have read the output rows
+        dev::patch_links<true, RS == 0>(buf, rs, lay.halo(st), L::Q, lay.links(st), gstart[cs], g0, g1, desc, d0);
+        dev::bulk_wait_read();  // this thread's bulk stores of the previous unit have read the output rows
         // bounced values in place, output rows free; a timeout anywhere in
         // the block stops the copies
         ok = __syncthreads_and(ok) != 0;
-        if (issuer && ok && rn < R) {
-            // refill the stage of the previous row: every thread is past its
+        if (issuer && ok && un < U) {
+            // refill the stage of the previous unit: every thread is past its
             // last reads of it (the link pass that follows the output) and
             // its wait on that stage's barrier
             uint32_t n0, n1;
-            range(rn, n0, n1);
-            stage_row<L, S>(smem_raw + sn * sbytes, lay, &bar[sn], Pin, rn, n0, n1, &gstart[sn], &dstart[sn], p);
+            range(un, n0, n1);
+            stage_unit<L, S, RS>(smem_raw + sn * sbytes, lay, &bar[sn], Pin, un, n0, n1, &gstart[sn], &dstart[sn], p);
         }
+        const bool fetch = halo && un < U && dev::halo_thread<L>();
+        T hv{};
+        if (fetch) hv = dev::halo_fetch<L, true>(Pin, dev::unit_at<RS>(p, un), p);
         const int nf = ord[0];
-        const uint32_t rowbase = (uint32_t)r * (uint32_t)nx;
+        const dev::UnitAt at = dev::unit_at<RS>(p, u);
+        const int nx = at.len;  // cells of the unit
+        const uint32_t rowbase = (uint32_t)at.row * (uint32_t)(RS ? RS : p.nx) + (uint32_t)at.x0;  // first cell
         if constexpr (kInPlace) {
             // one cell per thread (the launcher sets blockDim.x = nx): every
             // pull first, then a barrier, then the outputs over the stage
@@ -663,7 +670,7 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
             __syncthreads();  // no thread overwrites a slot another has still to pull
             if (fluid) {
                 float E[3];
-                load_E<L>(Ef, EF, p, cell, E);
+                load_E<L>(Ef, EF, p, (int64_t)at.row * (RS ? RS : p.nxp) + (at.x0 + x), E);
                 float out[L::Q];
                 collide_any<L, S, FORCE, LMU>(h, E, p, out);
                 typename S::T t[L::Q];
@@ -679,16 +686,27 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
             const int x = (int)ord[8 + i];
             if (i < nf) {
                 const uint32_t cell = rowbase + (uint32_t)x;
-                const int xm = x == 0 ? nx - 1 : x - 1;
-                const int xp = x == nx - 1 ? 0 : x + 1;
+                // the columns x - 1 and x + 1: in the unit, across the wrap of a
+                // whole row, or in the halo arrays beside a segment (stride 1 by slot)
+                const T* bm = buf + (x == 0 ? nx - 1 : x - 1);
+                const T* bp = buf + (x == nx - 1 ? 0 : x + 1);
+                int rm = rs, rp = rs;
+                if (halo && x == 0) {
+                    bm = lay.halo(st);
+                    rm = 1;
+                }
+                if (halo && x == nx - 1) {
+                    bp = lay.halo(st) + L::Q;
+                    rp = 1;
+                }
                 float h[L::Q];
 #pragma unroll
                 for (int a = 0; a < L::Q; ++a) {
-                    const int ex = L::c(a, 0);
-                    h[a] = S::cvt(buf[pop_slot<L>(a) * rs + (ex > 0 ? xm : (ex < 0 ? xp : x))]);
+                    const int ex = L::c(a, 0), s = pop_slot<L>(a);
+                    h[a] = S::cvt(ex > 0 ? bm[s * (RS ? RS : rm)] : (ex < 0 ? bp[s * (RS ? RS : rp)] : buf[s * rs + x]));
                 }
                 float E[3];
-                load_E<L>(Ef, EF, p, cell, E);
+                load_E<L>(Ef, EF, p, (int64_t)at.row * (RS ? RS : p.nxp) + (at.x0 + x), E);
                 if (S::kBytes == 4) {
                     // FP32 storage: compensated collision
                     float out[L::Q];
@@ -727,28 +745,29 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
                 for (int a = 0; a < L::Q; ++a) S::put(outrow + a * rs + x, 0.f);
             }
         }
+        if (fetch) dev::halo_put<L, true>(lay.halo(smem_raw + sn * sbytes), hv);
         dev::fence_proxy_async();  // this thread's shared-memory writes before the bulk copies
         __syncthreads();           // output rows complete; the stage is free for its refill
         if (threadIdx.x == 0) {
-            // the row's Q slots, one contiguous block
-            dev::bulk_store(Pout + (int64_t)rowbase * L::Q, orow, L::Q * row_bytes);
+            // the unit's Q slots, one contiguous block
+            dev::bulk_store(Pout + (int64_t)u * (L::Q * rs), orow, (uint32_t)lay.rows_bytes());
             dev::bulk_commit();
         }
         // outgoing links: slot k of (x, b) takes f*_b(x)
         for (uint32_t k = g0 + threadIdx.x; k < g1; k += blockDim.x) {
             const uint32_t d = desc[k - d0];
-            Gout[k] = orow[slot_of<L>((int)(d >> 24)) * rs + (int)(d & 0xFFFFFFu)];
+            Gout[k] = orow[desc_slot(d) * rs + desc_x(d)];
         }
     }
     dev::bulk_wait_all();
 }
 
 // ---------------------------------------------------------------------------
-// Launch policy.  The row-staged kernel runs when a row of one direction is a
-// multiple of 16 bytes and STAGES rows of all directions fit the shared-memory
-// budget; otherwise the general kernel runs.  The persistent grid is the
-// number of co-resident blocks (occupancy API) times the SM count, capped by
-// the number of rows.
+// Launch policy.  The row-staged kernel runs when the context has units (rows
+// of kMinStagedRow cells or more) and STAGES units with their outputs fit the
+// shared-memory budget; otherwise the general kernel runs.  The persistent grid
+// is the number of co-resident blocks (occupancy API) times the SM count,
+// capped by the number of units.
 // ---------------------------------------------------------------------------
 constexpr int kStages = 2;
 constexpr int kRowThreads = 256;
@@ -763,7 +782,7 @@ constexpr size_t kSmemBudget = 160 * 1024;
 // 256 threads.  fixed_threads != 0 takes that block size (the in-place FP32
 // rows need one thread per cell).
 struct Shape {
-    int threads, blocks;
+    int threads, blocks, sms;
 };
 template <class K>
 Shape launch_shape(K kernel, int nx, size_t smem, int fixed_threads = 0) {
@@ -771,7 +790,7 @@ Shape launch_shape(K kernel, int nx, size_t smem, int fixed_threads = 0) {
     static const void* last_k = nullptr;
     static size_t last_smem = 0;
     static int last_nx = 0;
-    static Shape last{0, 0};
+    static Shape last{0, 0, 0};
     std::lock_guard<std::mutex> lock(mu);
     if ((const void*)kernel != last_k || smem != last_smem || nx != last_nx) {
         int dev = 0, sms = 0;
@@ -780,7 +799,7 @@ Shape launch_shape(K kernel, int nx, size_t smem, int fixed_threads = 0) {
         if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         const int tmax = fixed_threads ? fixed_threads : (nx >= kRowThreads ? kRowThreads : ((nx + 31) / 32) * 32);
         const int tmin = fixed_threads ? fixed_threads : tmax / 2;
-        Shape best{tmax, 0};
+        Shape best{tmax, 0, sms};
         int best_per_sm = -1;
         for (int t = tmax; t >= 32 && t >= tmin; t -= 32) {
             int per_sm = 0;
@@ -803,22 +822,27 @@ template <class L, class S, int FORCE, bool EF, bool SR, int RS, bool LMU = fals
 bool launch_rows(const S*, const void* fin, void* fout, const uint32_t* nbr, const float* Ef, const KParams& p,
                  cudaStream_t s) {
     using T = typename S::T;
-    if (RS && RS != p.nx) return false;  // the stage rows are exactly nx long
-    const int rs = p.nx;
-    const size_t row_bytes = (size_t)p.nx * S::kBytes, srow = (size_t)rs * S::kBytes;
+    if (!p.rorder || (RS && (RS != p.nx || p.nseg != 1))) return false;
+    const size_t srow = (size_t)p.seglen * S::kBytes;
     const int gcap = dev::window_cap(p.max_row_links, S::kBytes);
     const int dcap = dev::window_cap(p.max_row_links, 4);
-    const size_t stage_bytes = (size_t)L::Q * srow + 2 * (size_t)p.lorder + gcap + dcap;
+    const size_t stage_bytes = (size_t)L::Q * srow + 2 * (size_t)p.lorder + gcap + dcap +
+                               dev::halo_bytes(L::Q, p.nseg, S::kBytes);
     constexpr bool kInPlace = kInPlaceOut<S, RS, LMU>;
     const size_t smem = (size_t)kStages * stage_bytes + (kInPlace ? 0 : (size_t)L::Q * srow);
-    if (!p.rorder || row_bytes % 16 != 0 || smem > kSmemBudget || p.nx < 32 || p.nx % 4 != 0) return false;
+    if (smem > kSmemBudget) return false;
     auto kern = k_step_rows<L, S, FORCE, EF, SR, kStages, RS, LMU>;
     // one cell per thread in place: exactly nx (= 256) threads
-    const Shape sh = launch_shape(kern, p.nx, smem, kInPlace ? p.nx : 0);
+    const Shape sh = launch_shape(kern, p.seglen, smem, kInPlace ? p.nx : 0);
     const int threads = sh.threads, blocks = sh.blocks;
     if (blocks <= 0) return false;
-    const int rows = p.ny * p.nz;
-    kern<<<blocks < rows ? blocks : rows, threads, smem, s>>>((const T*)fin, (T*)fout, Ef, gcap, dcap, p);
+    const int units = p.ny * p.nz * p.nseg;
+    // Fewer units than SMs: most of the chip would idle while each block runs its
+    // chain of copy, wait and two barriers once; the general kernel spreads the
+    // cells over more blocks (4096 x 8 cells of D2V9 BF16, 128 units: 6.2 us a
+    // step staged, below the 4.1 us that a launch takes the host otherwise).
+    if (units < sh.sms) return false;
+    kern<<<blocks < units ? blocks : units, threads, smem, s>>>((const T*)fin, (T*)fout, Ef, gcap, dcap, p);
     return true;
 }
 
@@ -837,8 +861,8 @@ int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef
         done = kFixed && launch_rows<L, S, FORCE, EF, SR, 0, kFixed>(tag, fin, fout, nbr, Ef, p, s);
     else if (kFixed && p.nx == 256)
         done = launch_rows<L, S, FORCE, EF, SR, kFixed ? 256 : 0>(tag, fin, fout, nbr, Ef, p, s);
-    else if (kFixed && p.nx == 512)
-        done = launch_rows<L, S, FORCE, EF, SR, kFixed ? 512 : 0>(tag, fin, fout, nbr, Ef, p, s);
+    else if (kFixed && p.nx == 512 && p.nseg == 1)
+        done = launch_rows<L, S, FORCE, EF, SR, kFixed && whole_row<L, S>(512) ? 512 : 0>(tag, fin, fout, nbr, Ef, p, s);
     else
         done = launch_rows<L, S, FORCE, EF, SR, 0>(tag, fin, fout, nbr, Ef, p, s);
     if (done) return 1;
