@@ -304,6 +304,17 @@ lbm_status lbm_weight_integrals(int D, int stat, double theta, double mu, double
 lbm_status lbm_save_state(lbm_ctx* ctx, void* host_buf, size_t cap, size_t* used);
 lbm_status lbm_load_state(lbm_ctx* ctx, const void* host_buf, size_t len);
 
+/* Copy the current state to / from device memory of the caller, asynchronously
+ * on the context's stream, with no header and no checksum: for programs that
+ * return to a state they have just left (the autograd function does).  The
+ * bytes are the context's own layout, valid for this context and geometry only.
+ * lbm_store_state with dev_buf == NULL only reports the size in *used.  steps
+ * is the step count that the restored state had (lbm_info).
+ * Infrastructure; the paper has no counterpart.  Errors: INVALID_ARG (short
+ * buffer, another size, a host pointer), STATE, CUDA. */
+lbm_status lbm_store_state(lbm_ctx* ctx, void* dev_buf, size_t cap, size_t* used);
+lbm_status lbm_restore_state(lbm_ctx* ctx, const void* dev_buf, size_t len, int64_t steps);
+
 /* FP64 fluid totals of the current state, like the totals of lbm_moments, but
  * without any device allocation; the paper has no counterpart (this is a
  * library service).  It is meant for callers that cannot or must not call

@@ -13,6 +13,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "_build", "liblbm.so")
 
 LBM_OK = 0
+LBM_ERR_OOM = 4
 STATUS = {0: "LBM_OK", 1: "LBM_ERR_INVALID_ARG", 2: "LBM_ERR_UNSTABLE_LATTICE", 3: "LBM_ERR_CUDA", 4: "LBM_ERR_OOM",
           5: "LBM_ERR_NONFINITE", 6: "LBM_ERR_TIMEOUT", 7: "LBM_ERR_STATE"}
 VEL = {"D2V9": 0, "D3V19": 1, "D3V27": 2, "D1V3": 3}
@@ -54,6 +55,8 @@ SIGNATURES = {
     "lbm_get_populations": (_i, [_vp, _vp, _i]),
     "lbm_save_state": (_i, [_vp, _vp, ctypes.c_size_t, ctypes.POINTER(ctypes.c_size_t)]),
     "lbm_load_state": (_i, [_vp, _vp, ctypes.c_size_t]),
+    "lbm_store_state": (_i, [_vp, _vp, ctypes.c_size_t, ctypes.POINTER(ctypes.c_size_t)]),
+    "lbm_restore_state": (_i, [_vp, _vp, ctypes.c_size_t, _i64]),
     "lbm_window_totals": (_i, [_vp, _i64, _i64, _vp]),
     "lbm_adjoint": (_i, [_vp, _vp, _vp, _i64, _i64, _i64, _vp, _vp, _vp, _vp, _vp]),
     "lbm_weight_integrals": (_i, [_i, _i, _d, _d, _vp]),

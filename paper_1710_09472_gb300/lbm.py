@@ -270,6 +270,30 @@ class LBM:
         buf = ctypes.create_string_buffer(blob, len(blob))
         _lib.check(_lib.load().lbm_load_state(self._h, buf, len(blob)), self._h, "lbm_load_state")
 
+    def _torch_stream(self):
+        """The context's stream as a torch stream (its memory then belongs to that stream)."""
+        s = self.stream
+        if s is None or hasattr(s, "cuda_stream"):
+            return s if s is not None else torch.cuda.default_stream()
+        return torch.cuda.ExternalStream(int(s))
+
+    def snapshot(self):
+        """The current state in device memory, for restore(): (bytes tensor,
+        step count).  Valid for this context and geometry only."""
+        used = ctypes.c_size_t(0)
+        lib = _lib.load()
+        _lib.check(lib.lbm_store_state(self._h, None, 0, ctypes.byref(used)), self._h, "lbm_store_state")
+        with torch.cuda.stream(self._torch_stream()):
+            buf = torch.empty(used.value, dtype=torch.uint8, device="cuda")
+            _lib.check(lib.lbm_store_state(self._h, ctypes.c_void_p(buf.data_ptr()), used.value, ctypes.byref(used)),
+                       self._h, "lbm_store_state")
+        return buf, self.info()["steps"]
+
+    def restore(self, snap):
+        buf, steps = snap
+        _lib.check(_lib.load().lbm_restore_state(self._h, ctypes.c_void_p(buf.data_ptr()), buf.numel(), int(steps)),
+                   self._h, "lbm_restore_state")
+
 
 class Thermal:
     """The 1D thermal model with the fourth-order EDF (lbm_thermal_*).
