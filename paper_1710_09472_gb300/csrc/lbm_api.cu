@@ -362,6 +362,32 @@ cudaError_t copy_saved(lbm_ctx* c, void* host, bool save) {
     return e;
 }
 
+// n steps from the current state.  Two or more steps of a box that fits a
+// cluster go out as one launch of up to kMultiSteps (which bounds what one
+// launch holds the GPU for); the others are launched one by one.
+constexpr int64_t kMultiSteps = 4096;
+void advance(lbm_ctx* c, KParams& p, int64_t n) {
+    for (int64_t t = 0; t < n;) {
+        p.step = (uint32_t)(c->steps);
+        const int64_t left = std::min(n - t, kMultiSteps);
+        int64_t done = 1;
+        int k = 0;
+        if (left > 1) {
+            k = lbm::launch_multi(c->lat.vel, c->storage, c->lat.force, c->stochastic, c->pop[c->cur],
+                                  c->pop[c->cur ^ 1], c->nbr, c->use_Efield ? c->Efield : nullptr, (int)left, p,
+                                  c->stream);
+            if (k) done = left;
+        }
+        if (!k)
+            k = lbm::launch_step(c->lat.vel, c->storage, c->lat.force, c->use_Efield, c->stochastic, c->pop[c->cur],
+                                 c->pop[c->cur ^ 1], c->nbr, c->Efield, p, c->stream);
+        c->launches += k;
+        c->cur ^= 1;
+        c->steps += done;
+        t += done;
+    }
+}
+
 // Link-buffer layout for the current link masks, then state buffers sized
 // for populations + links (contents undefined until lbm_init_equilibrium).
 lbm_status build_links_and_state(lbm_ctx* c) {
@@ -769,14 +795,7 @@ lbm_status lbm_step(lbm_ctx* c, int64_t n) {
     if (!c || n < 0) return fail(c, LBM_ERR_INVALID_ARG, "lbm_step: bad argument");
     if (!c->has_state) return fail(c, LBM_ERR_STATE, "lbm_step before lbm_init_equilibrium");
     KParams p = make_params(c);
-    const bool ef = c->use_Efield;
-    for (int64_t t = 0; t < n; ++t) {
-        p.step = (uint32_t)(c->steps + t);
-        c->launches += lbm::launch_step(c->lat.vel, c->storage, c->lat.force, ef, c->stochastic, c->pop[c->cur],
-                                        c->pop[c->cur ^ 1], c->nbr, c->Efield, p, c->stream);
-        c->cur ^= 1;
-    }
-    c->steps += n;
+    advance(c, p, n);
     return cuda_check(c, cudaGetLastError(), "lbm_step launch");
 }
 
@@ -937,18 +956,18 @@ lbm_status lbm_window_totals(lbm_ctx* c, int64_t t_begin, int64_t t_end, double 
                                            c->partials, &np, p, c->stream);
         c->launches += lbm::launch_accumulate_totals(c->partials, np, c->totals_dev, c->stream);
     }
-    for (int64_t t = 1; t <= t_end; ++t) {
-        p.step = (uint32_t)(c->steps + t - 1);
+    const int64_t before = std::max<int64_t>(t_begin, 0);  // steps whose states are not in the window
+    advance(c, p, before);
+    for (int64_t t = before + 1; t <= t_end; ++t) {
+        p.step = (uint32_t)(c->steps);
         c->launches += lbm::launch_step(c->lat.vel, c->storage, c->lat.force, c->use_Efield, c->stochastic,
                                         c->pop[c->cur], c->pop[c->cur ^ 1], c->nbr, c->Efield, p, c->stream);
         c->cur ^= 1;
-        if (t > t_begin) {
-            c->launches += lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, nullptr, nullptr,
-                                               c->partials, &np, p, c->stream);
-            c->launches += lbm::launch_accumulate_totals(c->partials, np, c->totals_dev, c->stream);
-        }
+        c->steps += 1;
+        c->launches += lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, nullptr, nullptr,
+                                           c->partials, &np, p, c->stream);
+        c->launches += lbm::launch_accumulate_totals(c->partials, np, c->totals_dev, c->stream);
     }
-    c->steps += t_end;
     LBM_CUDA(c, cudaGetLastError());
     LBM_CUDA(c, cudaMemcpyAsync(c->totals_host, c->totals_dev, sizeof(double) * 4, cudaMemcpyDeviceToHost, c->stream));
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -350,6 +350,19 @@ __host__ __device__ __forceinline__ int desc_slot_bar(uint32_t d) { return (int)
 __host__ __device__ __forceinline__ int desc_x(uint32_t d) { return (int)((d >> 10) & 0x7FFu); }
 __host__ __device__ __forceinline__ int desc_pos(uint32_t d) { return (int)(d >> 21); }
 
+// The "lowbias32" integer hash of C. Wellons seeds the rounding stream: once
+// per step, and per cell with that key.
+__host__ __device__ __forceinline__ uint32_t hash32(uint32_t x) {
+    x ^= x >> 16;
+    x *= 0x7feb352dU;
+    x ^= x >> 15;
+    x *= 0x846ca68bU;
+    x ^= x >> 16;
+    return x;
+}
+__host__ __device__ __forceinline__ uint32_t step_key(uint32_t step, uint32_t seed) {
+    return hash32(step * 0x9E3779B9u + seed);
+}
 struct Launch {
     dim3 grid, block;
 };
@@ -374,6 +387,11 @@ int launch_init(int vel, int storage, void* pop, const uint32_t* nbr, const floa
                 const KParams& p, cudaStream_t s);
 int launch_step(int vel, int storage, int force, bool efield, bool sr, const void* fin, void* fout,
                 const uint32_t* nbr, const float* Ef, const KParams& p, cudaStream_t s);
+// n steps in one launch where the box fits a cluster (lbm_multi.cuh); 0 where it
+// does not.  p.step is the first step's index; Ef is null for a uniform field;
+// the result is in fout.
+int launch_multi(int vel, int storage, int force, bool sr, const void* fin, void* fout, const uint32_t* nbr,
+                 const float* Ef, int n, const KParams& p, cudaStream_t s);
 int launch_step_f32(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
                     const float* Ef, const KParams& p, cudaStream_t s);
 int launch_step_f16(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,

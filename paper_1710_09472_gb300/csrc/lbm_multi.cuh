@@ -1,0 +1,230 @@
+// Many steps of a small box in one launch (templates; included by one
+// translation unit per storage type).
+//
+// A step of a small box is over before the host has launched the next one: 100
+// steps of 32 x 64 cells of D2V9 FP32 took 4.14 us each, 100 of 4096 x 8 in
+// BF16 the same, whatever the kernel (the host was the limit).  Here one cluster of up to 16 blocks
+// keeps the whole box in its shared memory and steps through all n steps by
+// itself: every thread collides its cells and writes each post-collision value
+// straight into the slot that the destination cell pulls next (distributed
+// shared memory; into its own slot of the opposite direction where a solid cell
+// is behind the link), then the cluster barrier ends the step.  The state
+// comes from global memory before the first step and goes back, in the layout
+// of the other kernels, with the last one.
+//
+// What bounds it: the serial chain of a collision (about 0.6 us) plus the
+// barrier while a block has a warp or two per scheduler, the issue slots of 16
+// SMs beyond that: 0.9 us a step at 32 x 64 (D2V9 FP32), 4.0 us at 4096 x 8
+// (D2V9 BF16).  So boxes up to the shared memory of the cluster qualify.
+// The arithmetic, its order and the rounding stream are those of k_step, so the
+// results have the same bits.
+#pragma once
+
+#include <mutex>
+
+#include "lbm_step.cuh"
+
+namespace lbm {
+namespace multik {
+
+using dev::Cell;
+
+constexpr int kClusterMax = 16;  // the non-portable limit
+constexpr size_t kSmemMax = 220 * 1024;
+constexpr uint32_t kNoCell = 0xFFFFFFFFu;
+
+// Threads per block: the FP32 collision of the larger lattices needs more than 64 registers.
+template <class L>
+constexpr int kThreads = L::Q <= 9 ? 1024 : 512;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+    return r;
+}
+// address of this block's shared address `a` in the block of rank r
+__device__ __forceinline__ uint32_t map_rank(uint32_t a, uint32_t r) {
+    uint32_t d;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(d) : "r"(a), "r"(r));
+    return d;
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, __half v) {
+    asm volatile("st.shared::cluster.u16 [%0], %1;\n" ::"r"(a), "h"(__half_as_ushort(v)) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, __nv_bfloat16 v) {
+    asm volatile("st.shared::cluster.u16 [%0], %1;\n" ::"r"(a), "h"(__bfloat16_as_ushort(v)) : "memory");
+}
+// all blocks' shared-memory writes before it are visible to all after it
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
+}
+
+// Block r of the cluster owns the cells r cpc .. r cpc + cpc - 1.  Shared
+// memory: two states h~_a at [a * cpc + i], and the destination of each value
+// as a cluster address into the second state (direction 0: the cell's place in
+// the padded field, or kNoCell for a solid cell).  Ef: the per-cell field, or null.
+template <class L, class S, int FORCE, bool SR>
+__global__ void __launch_bounds__(kThreads<L>) k_step_multi(const typename S::T* __restrict__ Pin,
+                                                            typename S::T* __restrict__ Pout,
+                                                            const uint32_t* __restrict__ nbr,
+                                                            const float* __restrict__ Ef, int n, int cpc, KParams p) {
+    using T = typename S::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    uint32_t* dst = reinterpret_cast<uint32_t*>(smem_raw);
+    T* state = reinterpret_cast<T*>(smem_raw + (size_t)L::Q * cpc * 4);
+    const int half = L::Q * cpc;  // elements of one state
+    const uint32_t rank = cluster_rank();
+    const int64_t first = (int64_t)rank * cpc;
+    const int mine = (int)(p.N - first < cpc ? (p.N > first ? p.N - first : 0) : cpc);
+    for (int i = threadIdx.x; i < mine; i += blockDim.x) {
+        const uint32_t cell = (uint32_t)first + (uint32_t)i;
+        const int row = (int)(cell / (uint32_t)p.nx);
+        Cell c;
+        dev::cell_at(p, row, (int)(cell - (uint32_t)row * (uint32_t)p.nx), c);
+        const uint32_t m = __ldg(nbr + cell);
+        dst[i] = (m & kSolidBit) ? kNoCell : (uint32_t)c.pcell;
+        if (m & kSolidBit) continue;
+        float h[L::Q];
+        dev::pull<L, S>(Pin, p, m, c, h);
+#pragma unroll
+        for (int a = 0; a < L::Q; ++a) {
+            S::put(state + a * cpc + i, h[a]);  // the stored value itself: it came from this format
+            if (a == 0) continue;
+            const bool wall = (m >> opposite(a)) & 1u;  // x + e_a is solid
+            const uint32_t to = wall ? cell : dev::shifted<L>(p, c, a, +1);
+            const uint32_t r = to / (uint32_t)cpc;
+            const T* at = state + half + (wall ? opposite(a) : a) * cpc + (int)(to - r * (uint32_t)cpc);
+            dst[a * cpc + i] = map_rank(dev::smem_u32(at), r);
+        }
+    }
+    cluster_barrier();
+    const uint32_t back = (uint32_t)(half * (int)sizeof(T));
+    for (int t = 0; t < n; ++t) {
+        const bool last = t == n - 1;
+        const T* in = state + (t & 1) * half;
+        T* own = state + ((t & 1) ^ 1) * half;
+        const uint32_t to = (t & 1) ? back : 0u;  // odd steps write the first state
+        const uint32_t key = step_key(p.step + (uint32_t)t, p.seed);
+        for (int i = threadIdx.x; i < mine; i += blockDim.x) {
+            const uint32_t place = dst[i];
+            const uint32_t cell = (uint32_t)first + (uint32_t)i;
+            T v[L::Q];
+            if (place != kNoCell) {
+                float h[L::Q], E[3], out[L::Q];
+#pragma unroll
+                for (int a = 0; a < L::Q; ++a) h[a] = S::cvt(in[a * cpc + i]);
+                stepk::load_E<L>(Ef, Ef != nullptr, p, place, E);
+                constexpr bool kLmu = L::Q == 9 || L::Q == 19;
+                if (kLmu && p.lmu_tab)
+                    stepk::collide_any<L, S, FORCE, kLmu>(h, E, p, out);
+                else
+                    stepk::collide_any<L, S, FORCE>(h, E, p, out);
+                stepk::round_all<L, S, SR>(out, cell, key, v);
+                if (!last) {
+                    own[i] = v[0];
+#pragma unroll
+                    for (int a = 1; a < L::Q; ++a) cluster_store(dst[a * cpc + i] - to, v[a]);
+                }
+            }
+            if (last) {
+                const int row = (int)(cell / (uint32_t)p.nx);
+                Cell c;
+                dev::cell_at(p, row, (int)(cell - (uint32_t)row * (uint32_t)p.nx), c);
+                if (place == kNoCell) {
+#pragma unroll
+                    for (int a = 0; a < L::Q; ++a) S::put(Pout + dev::pop_at<L>(p, c, a, 0), 0.f);
+                } else {
+                    stepk::store_cell<L, S>(Pout, p, __ldg(nbr + cell), c, v);
+                }
+            }
+        }
+        if (!last) cluster_barrier();
+    }
+}
+
+// Blocks of the cluster and shared memory of a box, or 0 blocks where it does
+// not fit: the smallest power of two of blocks that leaves at most 128 cells
+// each (one warp per scheduler), up to 16.
+struct Plan {
+    int blocks, cpc;
+    size_t smem;
+};
+template <class L, class S>
+Plan plan_of(const KParams& p) {
+    int blocks = 1;
+    while (blocks < kClusterMax && p.N > (int64_t)blocks * 128) blocks *= 2;
+    const int64_t cpc = ((p.N + blocks - 1) / blocks + 31) / 32 * 32;
+    const size_t smem = (size_t)L::Q * (size_t)cpc * (2 * S::kBytes + 4);
+    if (smem > kSmemMax) return {0, 0, 0};
+    return {blocks, (int)cpc, smem};
+}
+
+// Launches n steps, or returns 0: a box that does not fit, or a device on which
+// the cluster cannot be placed.
+template <class L, class S, int FORCE, bool SR>
+int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n, const KParams& p,
+               cudaStream_t s) {
+    using T = typename S::T;
+    const Plan plan = plan_of<L, S>(p);
+    if (plan.blocks == 0) return 0;
+    auto kern = k_step_multi<L, S, FORCE, SR>;
+    int threads = plan.cpc < kThreads<L> ? plan.cpc : kThreads<L>;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {(unsigned)plan.blocks, 1, 1};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)plan.blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = plan.smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    {
+        // whether the device can place this cluster; asked once per shape
+        static std::mutex mu;
+        static int last_blocks = 0, last_threads = 0;
+        static size_t last_smem = 0;
+        static bool fits = false;
+        std::lock_guard<std::mutex> lock(mu);
+        if (last_blocks != plan.blocks || last_smem != plan.smem || last_threads != threads) {
+            int clusters = 0;
+            fits = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) ==
+                       cudaSuccess &&
+                   cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0;
+            if (!fits) cudaGetLastError();
+            last_blocks = plan.blocks;
+            last_smem = plan.smem;
+            last_threads = threads;
+        }
+        if (!fits) return 0;
+    }
+    return cudaLaunchKernelEx(&cfg, kern, (const T*)fin, (T*)fout, nbr, Ef, n, plan.cpc, p) == cudaSuccess ? 1 : 0;
+}
+
+template <class S, bool HAS_SR>
+int launch_storage(int vel, int force, bool sr, const void* fin, void* fout, const uint32_t* nbr, const float* Ef,
+                   int n, const KParams& p, cudaStream_t s) {
+    auto with = [&](auto lat) {
+        using L = decltype(lat);
+        auto go = [&](auto srt) {
+            constexpr bool SR = decltype(srt)::value;
+            return force == LBM_FORCE_SHIFT ? launch_one<L, S, 0, SR>(fin, fout, nbr, Ef, n, p, s)
+                                            : launch_one<L, S, 1, SR>(fin, fout, nbr, Ef, n, p, s);
+        };
+        if constexpr (HAS_SR) {
+            if (sr) return go(std::true_type{});
+        }
+        return go(std::false_type{});
+    };
+    if (vel == LBM_D2V9) return with(LatD2V9{});
+    if (vel == LBM_D3V27) return with(LatD3V27{});
+    if (vel == LBM_D1V3) return with(LatD1V3{});
+    return with(LatD3V19{});
+}
+
+}  // namespace multik
+}  // namespace lbm

@@ -354,16 +354,6 @@ __device__ __forceinline__ void collide_acc(const float* h, const float* E, cons
     out[0] = rest + rest_lo;
 }
 
-// The "lowbias32" integer hash of C. Wellons (seeds the rounding stream).
-__device__ __forceinline__ uint32_t hash32(uint32_t x) {
-    x ^= x >> 16;
-    x *= 0x7feb352dU;
-    x ^= x >> 15;
-    x *= 0x846ca68bU;
-    x ^= x >> 16;
-    return x;
-}
-
 // Random stream for stochastic rounding: one hash of (cell, step) per cell,
 // then per pair of stores one step of a 32-bit LCG (Numerical Recipes
 // constants) folded as x ^ (x >> 16), so that the low bits of each 16-bit half
@@ -371,8 +361,7 @@ __device__ __forceinline__ uint32_t hash32(uint32_t x) {
 // replayed step reproduces its stores bit for bit.
 struct Rng {
     uint32_t x;
-    __device__ __forceinline__ Rng(uint32_t cell, const KParams& p)
-        : x(hash32(cell ^ hash32(p.step * 0x9E3779B9u + p.seed))) {}
+    __device__ __forceinline__ Rng(uint32_t cell, uint32_t key) : x(hash32(cell ^ key)) {}
     __device__ __forceinline__ uint32_t pair() {
         x = x * 1664525u + 1013904223u;
         return x ^ (x >> 16);
@@ -382,9 +371,9 @@ struct Rng {
 // Rounds the Q post-collision values to storage: the opposite pairs (a, a + 1),
 // then out[0] (converted as a pair with itself), stochastically when SR.
 template <class L, class S, bool SR>
-__device__ __forceinline__ void round_all(const float* out, uint32_t cell, const KParams& p, typename S::T* t) {
+__device__ __forceinline__ void round_all(const float* out, uint32_t cell, uint32_t key, typename S::T* t) {
     if (SR) {
-        Rng rng(cell, p);
+        Rng rng(cell, key);
         typename S::T unused;
 #pragma unroll
         for (int a = 1; a < L::Q; a += 2) S::sr2(out[a], out[a + 1], rng.pair(), t[a], t[a + 1]);
@@ -418,6 +407,21 @@ __device__ __forceinline__ void collide_any(const float* h, const float* E, cons
         collide<L, FORCE, LMU>(h, E, p, out);
 }
 
+// Writes a fluid cell's post-collision values to its own slots and, for links
+// into solid cells, to the link slots (ascending direction).
+template <class L, class S>
+__device__ __forceinline__ void store_cell(typename S::T* __restrict__ Pout, const KParams& p, uint32_t m,
+                                           const Cell& c, const typename S::T* t) {
+    typename S::T* g = reinterpret_cast<typename S::T*>(reinterpret_cast<char*>(Pout) + p.gofs);
+    g += m ? __ldg(p.lbase + c.cell) : 0u;
+    Pout[dev::pop_at<L>(p, c, 0, 0)] = t[0];
+#pragma unroll
+    for (int a = 1; a < L::Q; ++a) {
+        Pout[dev::pop_at<L>(p, c, a, 0)] = t[a];
+        if ((m >> opposite(a)) & 1u) *g++ = t[a];  // x + e_a is solid: the next link slot
+    }
+}
+
 // General step kernel: one thread per cell, pulls straight from global memory
 // and writes every own slot (solid cells write zeros, so that every sector is
 // written whole); links into solid cells also store into their link slot.
@@ -445,15 +449,8 @@ __global__ void __launch_bounds__(kBlock) k_step(const typename S::T* __restrict
     else
         collide_any<L, S, FORCE>(h, E, p, out);
     typename S::T t[L::Q];
-    round_all<L, S, SR>(out, c.cell, p, t);
-    typename S::T* g = reinterpret_cast<typename S::T*>(reinterpret_cast<char*>(Pout) + p.gofs);
-    g += m ? __ldg(p.lbase + c.cell) : 0u;
-    Pout[dev::pop_at<L>(p, c, 0, 0)] = t[0];
-#pragma unroll
-    for (int a = 1; a < L::Q; ++a) {
-        Pout[dev::pop_at<L>(p, c, a, 0)] = t[a];
-        if ((m >> opposite(a)) & 1u) *g++ = t[a];  // x + e_a is solid: the next link slot
-    }
+    round_all<L, S, SR>(out, c.cell, step_key(p.step, p.seed), t);
+    store_cell<L, S>(Pout, p, m, c, t);
 }
 
 // ---------------------------------------------------------------------------
@@ -674,7 +671,7 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
                 float out[L::Q];
                 collide_any<L, S, FORCE, LMU>(h, E, p, out);
                 typename S::T t[L::Q];
-                round_all<L, S, SR>(out, cell, p, t);
+                round_all<L, S, SR>(out, cell, step_key(p.step, p.seed), t);
 #pragma unroll
                 for (int a = 0; a < L::Q; ++a) orow[pop_slot<L>(a) * rs + x] = t[a];
             } else {
@@ -712,12 +709,12 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
                     float out[L::Q];
                     collide_any<L, S, FORCE, LMU>(h, E, p, out);
                     typename S::T t[L::Q];
-                    round_all<L, S, SR>(out, cell, p, t);
+                    round_all<L, S, SR>(out, cell, step_key(p.step, p.seed), t);
 #pragma unroll
                     for (int a = 0; a < L::Q; ++a) outrow[pop_slot<L>(a) * rs + x] = t[a];
                 } else {
                     // 16-bit storage: each pair is rounded and stored as soon as it exists
-                    Rng rng(cell, p);
+                    Rng rng(cell, step_key(p.step, p.seed));
                     collide_emit<L, FORCE, LMU>(
                         h, E, p,
                         [&](int a, float ha, float hb) {

@@ -9,7 +9,7 @@ import pytest
 
 import oracle
 from paper_1710_09472_gb300 import workloads as wl
-from tests.helpers import THETA, check_storage_error, gpu_run, oracle_run, rel_linf
+from tests.helpers import THETA, check_storage_error, oracle_run, rel_linf
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -44,17 +44,77 @@ def _case(vel, shape, seed):
     return solid, rho, u, Ef, B
 
 
+def _run(vel, shape, storage, force, case, calls, local_mu=False, seed=0):
+    """A run of the given lbm_step calls; its simulation and the fields after it."""
+    from paper_1710_09472_gb300.lbm import LBM
+
+    solid, rho, u, Ef, B = case
+    sim = LBM(vel, tuple(reversed(shape)), 0.8, B=B, storage=storage, force=force)
+    sim.set_geometry(torch.from_numpy(solid.reshape(-1)).cuda())
+    sim.set_E_field(torch.from_numpy(Ef.reshape(-1)).cuda())
+    if seed:
+        sim.set_rounding_seed(seed)
+    if local_mu:
+        sim.set_local_mu(True)
+    sim.init_equilibrium(torch.from_numpy(rho.reshape(-1)).cuda(), torch.from_numpy(u.reshape(-1)).cuda())
+    for n in calls:
+        sim.step(n)
+    r = torch.empty(sim.N, device="cuda")
+    j = torch.empty(sim.D * sim.N, device="cuda")
+    tot = sim.moments(r, j)
+    return r.cpu().numpy().reshape(shape), j.cpu().numpy().reshape((sim.D,) + tuple(shape)), tot, sim
+
+
 @pytest.mark.parametrize("vel,shape,storage", CASES)
 def test_step_and_totals(vel, shape, storage):
-    solid, rho, u, Ef, B = _case(vel, shape, 81)
-    rg, jg, totg, sim = gpu_run(vel, shape, solid, 0.8, 30, storage, "term", (0, 0, 0), B, rho, u, Ef)
+    """Single steps (the staged or general kernel) against the oracle; the same
+    steps in one call (small boxes: one launch on a cluster) to the last bit."""
+    case = _case(vel, shape, 81)
+    solid, rho, u, Ef, B = case
+    rg, jg, totg, sim = _run(vel, shape, storage, "term", case, [1] * 30)
     ro, jo, toto, _, _ = oracle_run(vel, shape, solid, 0.8, 30, "term", (0, 0, 0), B, rho, u, Ef)
+
+    def rerun(seed):
+        r, j, _, s = _run(vel, shape, storage, "term", case, [1] * 30, seed=seed)
+        s.close()
+        return rel_linf(r, ro), rel_linf(j, jo)
+
     check_storage_error(storage, (rel_linf(rg, ro), rel_linf(jg, jo)),
                         dict(vel=vel, shape=shape, solid=solid, tau=0.8, steps=30, force="term", E=(0, 0, 0), B=B,
-                             rho=rho, u=u, Efield=Ef, reference=(ro, jo)), label=f"units {vel} {shape}")
+                             rho=rho, u=u, Efield=Ef, reference=(ro, jo)), label=f"units {vel} {shape}",
+                        gpu_rerun=rerun)
     # the FP64 total of FP32 (16-bit) cells: rounding of the stored values only
     assert abs(totg[0] / toto[0] - 1) < {"f32": 1e-6, "f16": 1e-5, "bf16": 1e-4}[storage]
+    _, _, _, many = _run(vel, shape, storage, "term", case, [30])
+    np.testing.assert_array_equal(many.populations(deviation=True), sim.populations(deviation=True))
     sim.close()
+    many.close()
+
+
+# boxes on a cluster: one block, a box of one cell, several cells per thread, walls across the wrap, every lattice,
+# odd and even numbers of steps, nearly the largest box that fits and one just beyond
+SMALL = [("D2V9", (1, 1), "f32"), ("D2V9", (3, 5), "f16"), ("D2V9", (64, 32), "f32"), ("D2V9", (8, 4096), "bf16"),
+         ("D2V9", (100, 331), "f32"), ("D3V19", (2, 3, 5), "bf16"), ("D3V19", (24, 25, 26), "f32"),
+         ("D3V27", (12, 13, 14), "f16"), ("D1V3", (33,), "f32"), ("D1V3", (40000,), "f16")]
+
+
+@pytest.mark.parametrize("vel,shape,storage", SMALL)
+@pytest.mark.parametrize("force", ["term", "shift"])
+def test_steps_in_one_launch(vel, shape, storage, force):
+    case = _case(vel, shape, 61)
+    local = vel in ("D2V9", "D3V19") and force == "shift"
+    _, _, _, one = _run(vel, shape, storage, force, case, [1] * 13, local)
+    _, _, _, many = _run(vel, shape, storage, force, case, [2, 11], local)
+    np.testing.assert_array_equal(many.populations(deviation=True), one.populations(deviation=True))
+    before = many.launch_count()
+    many.step(6)
+    # 16 blocks of 32-cell granules with two states and the destinations in 220 KB each
+    N, b = int(np.prod(shape)), 4 if storage == "f32" else 2
+    granule = -(-(-(-N // 16)) // 32) * 32
+    fits = many.Q * granule * (2 * b + 4) <= 220 * 1024
+    assert many.launch_count() == before + (1 if fits else 6)
+    one.close()
+    many.close()
 
 
 @pytest.mark.parametrize("vel,shape,storage", [c for c in CASES if c[2] == "f32" and np.prod(c[1]) < 10000])
