@@ -362,8 +362,8 @@ cudaError_t copy_saved(lbm_ctx* c, void* host, bool save) {
     return e;
 }
 
-// n steps from the current state.  Two or more steps of a box that fits a
-// cluster go out as one launch of up to kMultiSteps (which bounds what one
+// n steps from the current state.  Two or more steps of a small box
+// (lbm_multi.cuh) go out as one launch of up to kMultiSteps (which bounds what one
 // launch holds the GPU for); the others are launched one by one.
 constexpr int64_t kMultiSteps = 4096;
 void advance(lbm_ctx* c, KParams& p, int64_t n) {
@@ -372,17 +372,18 @@ void advance(lbm_ctx* c, KParams& p, int64_t n) {
         const int64_t left = std::min(n - t, kMultiSteps);
         int64_t done = 1;
         int k = 0;
+        bool in_place = false;
         if (left > 1) {
             k = lbm::launch_multi(c->lat.vel, c->storage, c->lat.force, c->stochastic, c->pop[c->cur],
-                                  c->pop[c->cur ^ 1], c->nbr, c->use_Efield ? c->Efield : nullptr, (int)left, p,
-                                  c->stream);
+                                  c->pop[c->cur ^ 1], c->nbr, c->use_Efield ? c->Efield : nullptr, (int)left,
+                                  reinterpret_cast<unsigned*>(c->count_dev + 1), &in_place, p, c->stream);
             if (k) done = left;
         }
         if (!k)
             k = lbm::launch_step(c->lat.vel, c->storage, c->lat.force, c->use_Efield, c->stochastic, c->pop[c->cur],
                                  c->pop[c->cur ^ 1], c->nbr, c->Efield, p, c->stream);
         c->launches += k;
-        c->cur ^= 1;
+        if (!(done > 1 && in_place)) c->cur ^= 1;
         c->steps += done;
         t += done;
     }
@@ -587,7 +588,7 @@ lbm_status lbm_create(lbm_ctx** out, const lbm_lattice* lat, const int64_t dims[
                          "cudaMalloc partials")) != LBM_OK ||
         (st = cuda_check(c, cudaMalloc((void**)&c->totals_dev, sizeof(double) * 4), "cudaMalloc totals")) !=
             LBM_OK ||
-        (st = cuda_check(c, cudaMalloc((void**)&c->count_dev, sizeof(unsigned long long)), "cudaMalloc count")) !=
+        (st = cuda_check(c, cudaMalloc((void**)&c->count_dev, 2 * sizeof(unsigned long long)), "cudaMalloc count")) !=
             LBM_OK ||
         (st = cuda_check(c, cudaMallocHost((void**)&c->totals_host, sizeof(double) * 4), "cudaMallocHost")) !=
             LBM_OK ||

@@ -387,11 +387,12 @@ int launch_init(int vel, int storage, void* pop, const uint32_t* nbr, const floa
                 const KParams& p, cudaStream_t s);
 int launch_step(int vel, int storage, int force, bool efield, bool sr, const void* fin, void* fout,
                 const uint32_t* nbr, const float* Ef, const KParams& p, cudaStream_t s);
-// n steps in one launch where the box fits a cluster (lbm_multi.cuh); 0 where it
-// does not.  p.step is the first step's index; Ef is null for a uniform field;
-// the result is in fout.
-int launch_multi(int vel, int storage, int force, bool sr, const void* fin, void* fout, const uint32_t* nbr,
-                 const float* Ef, int n, const KParams& p, cudaStream_t s);
+// n steps in one launch where the box is small enough (lbm_multi.cuh); 0 where it
+// is not.  p.step is the first step's index; Ef is null for a uniform field;
+// count is a word of device memory for the launch's barrier.  The result is in
+// fout, or in fin where *in_fin says so; the other buffer is overwritten.
+int launch_multi(int vel, int storage, int force, bool sr, void* fin, void* fout, const uint32_t* nbr, const float* Ef,
+                 int n, unsigned* count, bool* in_fin, const KParams& p, cudaStream_t s);
 int launch_step_f32(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
                     const float* Ef, const KParams& p, cudaStream_t s);
 int launch_step_f16(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
@@ -503,7 +504,7 @@ struct lbm_ctx {
     int64_t partials_cap = 0;
     double* totals_dev = nullptr;
     double* totals_host = nullptr;  // pinned, 4 doubles
-    unsigned long long* count_dev = nullptr;
+    unsigned long long* count_dev = nullptr;  // fluid cells; the second word counts blocks at a grid barrier
     AdjWorkspace ws;               // lbm_adjoint buffers kept between calls
     size_t mem_budget = 0;         // device bytes an lbm_adjoint call may allocate (0: free memory)
     int64_t adj_stats[4] = {0, 0, 0, 0};  // last lbm_adjoint: schedule, state buffers, forward steps, reverse steps

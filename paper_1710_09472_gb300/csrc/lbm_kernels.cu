@@ -470,18 +470,20 @@ int launch_step(int vel, int storage, int force, bool efield, bool sr, const voi
 // and its 8192 partials another 41 us in the one block that sums them.
 constexpr int kTotalsPerSm = 8;
 
-int launch_multi_f32(int, int, bool, const void*, void*, const uint32_t*, const float*, int, const KParams&,
-                     cudaStream_t);
-int launch_multi_f16(int, int, bool, const void*, void*, const uint32_t*, const float*, int, const KParams&,
-                     cudaStream_t);
-int launch_multi_bf16(int, int, bool, const void*, void*, const uint32_t*, const float*, int, const KParams&,
-                      cudaStream_t);
+int launch_multi_f32(int, int, bool, void*, void*, const uint32_t*, const float*, int, unsigned*, bool*,
+                     const KParams&, cudaStream_t);
+int launch_multi_f16(int, int, bool, void*, void*, const uint32_t*, const float*, int, unsigned*, bool*,
+                     const KParams&, cudaStream_t);
+int launch_multi_bf16(int, int, bool, void*, void*, const uint32_t*, const float*, int, unsigned*, bool*,
+                      const KParams&, cudaStream_t);
 
-int launch_multi(int vel, int storage, int force, bool sr, const void* fin, void* fout, const uint32_t* nbr,
-                 const float* Ef, int n, const KParams& p, cudaStream_t s) {
-    if (storage == LBM_F16_DEV) return launch_multi_f16(vel, force, sr, fin, fout, nbr, Ef, n, p, s);
-    if (storage == LBM_BF16_DEV) return launch_multi_bf16(vel, force, sr, fin, fout, nbr, Ef, n, p, s);
-    return launch_multi_f32(vel, force, false, fin, fout, nbr, Ef, n, p, s);
+int launch_multi(int vel, int storage, int force, bool sr, void* fin, void* fout, const uint32_t* nbr, const float* Ef,
+                 int n, unsigned* count, bool* in_fin, const KParams& p, cudaStream_t s) {
+    if (storage == LBM_F16_DEV)
+        return launch_multi_f16(vel, force, sr, fin, fout, nbr, Ef, n, count, in_fin, p, s);
+    if (storage == LBM_BF16_DEV)
+        return launch_multi_bf16(vel, force, sr, fin, fout, nbr, Ef, n, count, in_fin, p, s);
+    return launch_multi_f32(vel, force, false, fin, fout, nbr, Ef, n, count, in_fin, p, s);
 }
 
 int launch_moments(int vel, int storage, const void* pop, const uint32_t* nbr, float* rho, float* j,

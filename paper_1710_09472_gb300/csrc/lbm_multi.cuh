@@ -15,7 +15,15 @@
 // What bounds it: the serial chain of a collision (about 0.6 us) plus the
 // barrier while a block has a warp or two per scheduler, the issue slots of 16
 // SMs beyond that: 0.9 us a step at 32 x 64 (D2V9 FP32), 4.0 us at 4096 x 8
-// (D2V9 BF16).  So boxes up to the shared memory of the cluster qualify.
+// (D2V9 BF16).
+//
+// Beyond kClusterWork populations (where 16 SMs take as long as the other
+// kernel's barrier costs) a cooperative grid with a thread for every cell does
+// the same through global memory (k_step_grid): the two state buffers hold the
+// values as they are pulled, [a N + cell], until the last step, and a barrier
+// over the grid ends a step.  Boxes of more cells than threads that are
+// resident at once are stepped one launch at a time: their steps outlast a
+// launch.
 // The arithmetic, its order and the rounding stream are those of k_step, so the
 // results have the same bits.
 #pragma once
@@ -33,9 +41,16 @@ constexpr int kClusterMax = 16;  // the non-portable limit
 constexpr size_t kSmemMax = 220 * 1024;
 constexpr uint32_t kNoCell = 0xFFFFFFFFu;
 
-// Threads per block: the FP32 collision of the larger lattices needs more than 64 registers.
+// Populations up to which the cluster is the faster of the two.  Its step grows
+// with the box (0.87 us at 2048 cells of D2V9, 3.97 us at 32768), the grid's
+// hardly does (2.36 us at 32768): they meet near 16384 cells.
+constexpr int64_t kClusterWork = 16384 * 9;
+// Threads per block: the FP32 collision of the larger lattices needs more than
+// 64 registers.  The grid has one block per SM.
 template <class L>
 constexpr int kThreads = L::Q <= 9 ? 1024 : 512;
+template <class L>
+constexpr int kGridThreads = L::Q <= 9 ? 1024 : 640;
 
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -145,6 +160,103 @@ __global__ void __launch_bounds__(kThreads<L>) k_step_multi(const typename S::T*
     }
 }
 
+// Barrier over a cooperative grid: `count` grows by one per block and step.  A
+// wait that runs out (2^31 clocks, about a second) writes code 4 into the status
+// word; the block then waits no more, and the kernel ends with invalid results.
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, bool ok, int* status) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(count) : "memory");
+        if (ok) {
+            const long long t0 = clock64();
+            for (;;) {
+                unsigned v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(count) : "memory");
+                if (v >= target) break;
+                if (clock64() - t0 > (1ll << 31)) {
+                    ok = false;
+                    if (status) atomicExch(status, 4);
+                    break;
+                }
+            }
+        }
+    }
+    return __syncthreads_and(threadIdx.x != 0 || ok) != 0;
+}
+
+__device__ __forceinline__ float load_l2(const float* q) { return __ldcg(q); }
+__device__ __forceinline__ __half load_l2(const __half* q) {
+    return __ushort_as_half(__ldcg(reinterpret_cast<const unsigned short*>(q)));
+}
+__device__ __forceinline__ __nv_bfloat16 load_l2(const __nv_bfloat16* q) {
+    return __ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(q)));
+}
+
+// n steps with one thread per cell, all blocks resident (cooperative launch).
+// Step t reads buf[t & 1] and writes the other; dst (shared memory, [a][thread])
+// holds the element that each value goes to.  The loads bypass L1, which other
+// blocks' stores do not reach.
+template <class L, class S, int FORCE, bool SR>
+__global__ void __launch_bounds__(kGridThreads<L>) k_step_grid(typename S::T* A, typename S::T* B,
+                                                               const uint32_t* __restrict__ nbr,
+                                                               const float* __restrict__ Ef, int n, unsigned* count,
+                                                               KParams p) {
+    using T = typename S::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    uint32_t* dst = reinterpret_cast<uint32_t*>(smem_raw) + threadIdx.x;
+    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in_box = id < p.N;
+    const uint32_t cell = in_box ? (uint32_t)id : 0u, N = (uint32_t)p.N;
+    const int row = (int)(cell / (uint32_t)p.nx);
+    Cell c;
+    dev::cell_at(p, row, (int)(cell - (uint32_t)row * (uint32_t)p.nx), c);
+    const uint32_t m = __ldg(nbr + cell);
+    const bool fluid = in_box && !(m & kSolidBit);
+#pragma unroll
+    for (int a = 1; a < L::Q; ++a) {
+        const bool wall = (m >> opposite(a)) & 1u;  // x + e_a is solid
+        dst[(a - 1) * (int)blockDim.x] = wall ? (uint32_t)opposite(a) * N + cell
+                                              : (uint32_t)a * N + dev::shifted<L>(p, c, a, +1);
+    }
+    float h[L::Q];
+    if (fluid) dev::pull<L, S>(A, p, m, c, h);  // no block writes A before the first barrier
+    bool ok = true;
+    for (int t = 0; t < n; ++t) {
+        const T* from = (t & 1) ? B : A;
+        T* to = (t & 1) ? A : B;
+        if (t > 0) {
+            ok = grid_barrier(count, (unsigned)t * gridDim.x, ok, p.status);
+            if (fluid) {
+#pragma unroll
+                for (int a = 0; a < L::Q; ++a) h[a] = S::cvt(load_l2(from + ((uint32_t)a * N + cell)));
+            }
+        }
+        const bool last = t == n - 1;
+        if (fluid) {
+            float E[3], out[L::Q];
+            T v[L::Q];
+            stepk::load_E<L>(Ef, Ef != nullptr, p, c.pcell, E);
+            constexpr bool kLmu = L::Q == 9 || L::Q == 19;
+            if (kLmu && p.lmu_tab)
+                stepk::collide_any<L, S, FORCE, kLmu>(h, E, p, out);
+            else
+                stepk::collide_any<L, S, FORCE>(h, E, p, out);
+            stepk::round_all<L, S, SR>(out, cell, step_key(p.step + (uint32_t)t, p.seed), v);
+            if (last) {
+                stepk::store_cell<L, S>(to, p, m, c, v);
+            } else {
+                to[cell] = v[0];
+#pragma unroll
+                for (int a = 1; a < L::Q; ++a) to[dst[(a - 1) * (int)blockDim.x]] = v[a];
+            }
+        } else if (last && in_box) {
+#pragma unroll
+            for (int a = 0; a < L::Q; ++a) S::put(to + dev::pop_at<L>(p, c, a, 0), 0.f);
+        }
+    }
+}
+
 // Blocks of the cluster and shared memory of a box, or 0 blocks where it does
 // not fit: the smallest power of two of blocks that leaves at most 128 cells
 // each (one warp per scheduler), up to 16.
@@ -158,14 +270,14 @@ Plan plan_of(const KParams& p) {
     while (blocks < kClusterMax && p.N > (int64_t)blocks * 128) blocks *= 2;
     const int64_t cpc = ((p.N + blocks - 1) / blocks + 31) / 32 * 32;
     const size_t smem = (size_t)L::Q * (size_t)cpc * (2 * S::kBytes + 4);
-    if (smem > kSmemMax) return {0, 0, 0};
+    if (smem > kSmemMax || p.N * L::Q > kClusterWork) return {0, 0, 0};
     return {blocks, (int)cpc, smem};
 }
 
 // Launches n steps, or returns 0: a box that does not fit, or a device on which
 // the cluster cannot be placed.
 template <class L, class S, int FORCE, bool SR>
-int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n, const KParams& p,
+int launch_cluster(const void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n, const KParams& p,
                cudaStream_t s) {
     using T = typename S::T;
     const Plan plan = plan_of<L, S>(p);
@@ -205,15 +317,70 @@ int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef
     return cudaLaunchKernelEx(&cfg, kern, (const T*)fin, (T*)fout, nbr, Ef, n, plan.cpc, p) == cudaSuccess ? 1 : 0;
 }
 
+// The same for the cooperative grid; the result is in fin when n is even.
+template <class L, class S, int FORCE, bool SR>
+int launch_grid(void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n, unsigned* count, const KParams& p,
+                cudaStream_t s) {
+    using T = typename S::T;
+    auto kern = k_step_grid<L, S, FORCE, SR>;
+    static std::mutex mu;
+    static int sms = 0;  // SMs, 0 where the device has no cooperative launch
+    static int asked_threads = 0;
+    static bool fits = false;
+    int threads;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (sms == 0) {
+            int dev = 0, coop = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+            if (coop) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            if (sms < 1) return 0;
+        }
+        const int64_t per = ((p.N + sms - 1) / sms + 31) / 32 * 32;
+        if (per > kGridThreads<L>) return 0;
+        threads = (int)per;
+        if (asked_threads != threads) {
+            int blocks = 0;
+            const size_t smem = (size_t)(L::Q - 1) * threads * 4;
+            fits = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+                   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, threads, smem) == cudaSuccess &&
+                   blocks > 0;
+            if (!fits) cudaGetLastError();
+            asked_threads = threads;
+        }
+        if (!fits) return 0;
+    }
+    if (cudaMemsetAsync(count, 0, sizeof(unsigned), s) != cudaSuccess) return 0;
+    T *A = (T*)fin, *B = (T*)fout;
+    KParams q = p;
+    void* args[] = {&A, &B, &nbr, &Ef, &n, &count, &q};
+    const unsigned blocks = (unsigned)((p.N + threads - 1) / threads);
+    return cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3((unsigned)threads), args,
+                                       (size_t)(L::Q - 1) * threads * 4, s) == cudaSuccess
+               ? 1
+               : 0;
+}
+
+template <class L, class S, int FORCE, bool SR>
+int launch_one(void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n, unsigned* count, bool* in_fin,
+               const KParams& p, cudaStream_t s) {
+    *in_fin = false;
+    if (int k = launch_cluster<L, S, FORCE, SR>(fin, fout, nbr, Ef, n, p, s)) return k;
+    if (p.N * L::Q <= kClusterWork) return 0;
+    *in_fin = n % 2 == 0;
+    return launch_grid<L, S, FORCE, SR>(fin, fout, nbr, Ef, n, count, p, s);
+}
+
 template <class S, bool HAS_SR>
-int launch_storage(int vel, int force, bool sr, const void* fin, void* fout, const uint32_t* nbr, const float* Ef,
-                   int n, const KParams& p, cudaStream_t s) {
+int launch_storage(int vel, int force, bool sr, void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n,
+                   unsigned* count, bool* in_fin, const KParams& p, cudaStream_t s) {
     auto with = [&](auto lat) {
         using L = decltype(lat);
         auto go = [&](auto srt) {
             constexpr bool SR = decltype(srt)::value;
-            return force == LBM_FORCE_SHIFT ? launch_one<L, S, 0, SR>(fin, fout, nbr, Ef, n, p, s)
-                                            : launch_one<L, S, 1, SR>(fin, fout, nbr, Ef, n, p, s);
+            return force == LBM_FORCE_SHIFT ? launch_one<L, S, 0, SR>(fin, fout, nbr, Ef, n, count, in_fin, p, s)
+                                            : launch_one<L, S, 1, SR>(fin, fout, nbr, Ef, n, count, in_fin, p, s);
         };
         if constexpr (HAS_SR) {
             if (sr) return go(std::true_type{});

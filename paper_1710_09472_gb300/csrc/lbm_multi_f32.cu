@@ -2,8 +2,8 @@
 #include "lbm_multi.cuh"
 
 namespace lbm {
-int launch_multi_f32(int vel, int force, bool sr, const void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n,
-                     const KParams& p, cudaStream_t s) {
-    return multik::launch_storage<StoreF32, false>(vel, force, sr, fin, fout, nbr, Ef, n, p, s);
+int launch_multi_f32(int vel, int force, bool sr, void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n,
+                     unsigned* count, bool* in_fin, const KParams& p, cudaStream_t s) {
+    return multik::launch_storage<StoreF32, false>(vel, force, sr, fin, fout, nbr, Ef, n, count, in_fin, p, s);
 }
 }  // namespace lbm
