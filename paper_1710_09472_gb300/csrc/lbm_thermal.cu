@@ -22,6 +22,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <algorithm>
 #include <cstring>
 #include <string>
 
@@ -81,14 +82,349 @@ __device__ __forceinline__ int t_src(int x, int a, int nx) {
     return s >= nx ? s - nx : s;
 }
 
+// Values of one cell (float) or of two neighbouring cells (F2, the packed FP32
+// arithmetic of sm_100 and later: one instruction for both).  Every operation
+// is written out and rounds once, so a cell has the same bits in either.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pack2(float lo, float hi) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(F2 a, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+template <class V>
+__device__ __forceinline__ V tv(float c);
+template <>
+__device__ __forceinline__ float tv<float>(float c) {
+    return c;
+}
+template <>
+__device__ __forceinline__ F2 tv<F2>(float c) {
+    return pack2(c, c);
+}
+__device__ __forceinline__ float tadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float tsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float tmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float tfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float tneg(float a) { return -a; }
+__device__ __forceinline__ float tdiv(float a, float b) { return __fdiv_rn(a, b); }
+__device__ __forceinline__ F2 tadd(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 tmul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 tfma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 tsub(F2 a, F2 b) { return tfma(b, tv<F2>(-1.f), a); }
+__device__ __forceinline__ F2 tneg(F2 a) { return F2{a.v ^ 0x8000000080000000ull}; }
+__device__ __forceinline__ F2 tdiv(F2 a, F2 b) {
+    float a0, a1, b0, b1;
+    unpack2(a, a0, a1);
+    unpack2(b, b0, b1);
+    return pack2(__fdiv_rn(a0, b0), __fdiv_rn(a1, b1));
+}
+
 // The equilibrium deviations heq~_a (scaled) of one cell (a < Q).  The
 // lattice pairs a, a + 1 have xi_{a+1} = -xi_a, so W_N,a+1 = (-1)^N W_N,a
 // (checked on the host): heq_a = even + odd and heq_{a+1} = even - odd with
 // even = sum over N = 0, 2, 4 and odd = sum over N = 1, 3; the rest
 // population has no odd part.  With kLo the hi + lo weight pairs are used.
+template <int Q, bool kLo, class V>
+__device__ __forceinline__ void t_equilibrium(const TParams& p, V drho, V rho, V us, V dth, V* heq) {
+    auto c = [](float x) { return tv<V>(x); };
+    const V srho = tmul(c(p.scale), rho);
+    const V u2 = tmul(us, us);
+    const V A1 = tmul(tmul(srho, c(p.c1)), us);
+    const V A2 = p.order >= 2 ? tmul(tmul(srho, c(p.c22)), tadd(dth, u2)) : c(0.f);
+    V A3 = c(0.f), A4 = c(0.f);
+    if (p.order >= 3) {
+        const V K3 = tfma(c(p.cb3), u2, tfma(c(fmaf(3.f, p.cb3, p.c3)), dth, c(p.K30)));
+        A3 = tmul(srho, tfma(tmul(c(p.c3), u2), us, tmul(tmul(c(3.f), K3), us)));
+    }
+    if (p.order >= 4) {
+        const V th = tadd(c(p.thw), dth);
+        V S = tfma(tmul(c(p.a4), dth), tadd(c(2.f * p.thw), dth), tmul(c(p.b4), dth));
+        S = tadd(S, c(p.S0));
+        S = tfma(u2, tfma(c(fmaf(2.f, p.cb4, 6.f * p.db4)), th, c(p.dp4)), S);
+        S = tfma(tmul(c(p.db4), u2), u2, S);
+        const V T = tfma(c(p.cb4), u2, tfma(c(p.c45), dth, c(p.T0)));
+        A4 = tmul(srho, tfma(tmul(c(p.c4), u2), u2, tfma(c(3.f), S, tmul(tmul(c(6.f), u2), T))));
+    }
+    const V A[5] = {drho, A1, A2, A3, A4};
+    // sum of W_N,a A_N over N, N + 2, ..
+    auto even_sum = [&](int a) {
+        if (kLo) {
+            auto term = [&](int N) { return tfma(c(p.Wlo[N][a]), A[N], tmul(c(p.W[N][a]), A[N])); };
+            return tadd(tadd(term(0), term(2)), term(4));
+        }
+        return tfma(c(p.W[4][a]), A[4], tfma(c(p.W[0][a]), A[0], tmul(c(p.W[2][a]), A[2])));
+    };
+    auto odd_sum = [&](int a) {
+        if (kLo) {
+            auto term = [&](int N) { return tfma(c(p.Wlo[N][a]), A[N], tmul(c(p.W[N][a]), A[N])); };
+            return tadd(term(1), term(3));
+        }
+        return tfma(c(p.W[1][a]), A[1], tmul(c(p.W[3][a]), A[3]));
+    };
+    heq[0] = even_sum(0);
+#pragma unroll
+    for (int a = 1; a < Q; a += 2) {
+        const V even = even_sum(a), odd = odd_sum(a);
+        heq[a] = tadd(even, odd);
+        heq[a + 1] = tsub(even, odd);
+    }
+}
+
+// Error-free sum and product (Knuth TwoSum, FMA TwoProd) for the moment sums.
+template <class V>
+__device__ __forceinline__ void t_two_sum(V a, V b, V& s, V& e) {
+    const V t = tadd(a, b);
+    const V bb = tsub(t, a);
+    e = tadd(tsub(a, tsub(t, bb)), tsub(b, bb));
+    s = t;
+}
+template <class V>
+__device__ __forceinline__ void t_acc(V& hi, V& lo, V a, V b) {  // hi + lo += a b
+    const V p = tmul(a, b), pe = tfma(a, b, tneg(p));
+    V e;
+    t_two_sum(hi, p, hi, e);
+    lo = tadd(lo, tadd(e, pe));
+}
+
+// One collision: the pulled h~_a become the post-collision values.
+// FP32 storage (kExact): the moments as double-float sums (the first FP32
+// rounding of a moment would otherwise recur in every step) and the hi + lo
+// equilibrium weights; 16-bit storage rounds far coarser, so there plain FP32
+// sums over the pairs a, a + 1 suffice.
+template <int Q, bool kExact, class V>
+__device__ __forceinline__ void t_collide(const TParams& p, V* h) {
+    auto c = [](float x) { return tv<V>(x); };
+    V dh = h[0], dl = c(0.f), j, m2;
+    if (kExact) {
+        V jh = c(0.f), jl = c(0.f), mh = c(0.f), ml = c(0.f);
+        t_acc(mh, ml, h[0], c(p.xim[0]));
+#pragma unroll
+        for (int a = 1; a < Q; ++a) {
+            V e;
+            t_two_sum(dh, h[a], dh, e);
+            dl = tadd(dl, e);
+            t_acc(jh, jl, h[a], c(p.xi[a]));
+            t_acc(mh, ml, h[a], c(p.xim[a]));
+        }
+        j = tadd(jh, jl);
+        m2 = tadd(mh, ml);
+    } else {
+        j = c(0.f);
+        m2 = tmul(c(p.xim[0]), h[0]);
+#pragma unroll
+        for (int a = 1; a < Q; a += 2) {
+            const V sa = tadd(h[a], h[a + 1]), da = tsub(h[a], h[a + 1]);
+            dh = tadd(dh, sa);
+            j = tfma(c(p.xi[a]), da, j);
+            m2 = tfma(c(p.xim[a]), sa, m2);
+        }
+    }
+    const V drho = tadd(dh, dl);
+    const V rho = tfma(drho, c(p.inv_scale), c(p.rho0));
+    V u, dth;
+    if (kExact) {
+        u = tdiv(tmul(j, c(p.inv_scale)), rho);
+        dth = tfma(tneg(u), u, tdiv(tmul(m2, c(p.inv_scale)), rho));
+    } else {
+        const V ir = tdiv(c(p.inv_scale), rho);
+        u = tmul(j, ir);
+        dth = tfma(m2, ir, tneg(tmul(u, u)));
+    }
+    V heq[Q];
+    t_equilibrium<Q, kExact>(p, drho, rho, tadd(u, c(p.tau * p.E)), dth, heq);
+    const V omm = c(1.f - p.omega), om = c(p.omega);
+    V rest = dh;
+#pragma unroll
+    for (int a = 1; a < Q; ++a) h[a] = tfma(omm, h[a], tmul(om, heq[a]));
+#pragma unroll
+    for (int a = 1; a < Q; a += 2) rest = tsub(rest, tadd(h[a], h[a + 1]));
+    h[0] = tadd(rest, dl);
+}
+
+// One cell: pull with the periodic wrap, collide, round, store.
+template <class S, bool SR, int Q>
+__device__ __forceinline__ void t_cell(const typename S::T* __restrict__ Pin, typename S::T* __restrict__ Pout, int x,
+                                       const TParams& p) {
+    float h[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a)
+        h[a] = S::cvt(Pin[(int64_t)a * p.nx + (p.nx >= 3 ? t_src<Q>(x, a, p.nx) : wrapx(x - p.e[a], p.nx))]);
+    t_collide<Q, S::kBytes == 4>(p, h);
+    uint32_t r = 0;
+    if (SR) r = t_hash((uint32_t)x ^ p.skey);
+    typename S::T* py = Pout + x;
+#pragma unroll
+    for (int a = 1; a < Q; a += 2) {
+        typename S::T ta, tb;
+        if (SR) {
+            r = r * 1664525u + 1013904223u;
+            S::sr2(h[a], h[a + 1], r ^ (r >> 16), ta, tb);
+        } else {
+            S::put(&ta, h[a]);
+            S::put(&tb, h[a + 1]);
+        }
+        py[p.plane[a]] = ta;
+        py[p.plane[a + 1]] = tb;
+    }
+    typename S::T t0, unused;
+    if (SR) {
+        r = r * 1664525u + 1013904223u;
+        S::sr2(h[0], h[0], r ^ (r >> 16), t0, unused);
+    } else {
+        S::put(&t0, h[0]);
+    }
+    *py = t0;
+}
+
+// Two neighbouring values of a plane, as they are stored.  WORD: the pair is
+// one aligned word (two words for FP32).
+template <class S, bool WORD>
+__device__ __forceinline__ F2 t_load2(const typename S::T* q) {
+    if constexpr (S::kBytes == 4) {
+        if (WORD) {
+            const float2 v = *reinterpret_cast<const float2*>(q);
+            return pack2(v.x, v.y);
+        }
+        return pack2(q[0], q[1]);
+    } else {
+        union {
+            uint32_t w;
+            typename S::T t[2];
+        } u;
+        if (WORD) {
+            u.w = *reinterpret_cast<const uint32_t*>(q);
+            return pack2(S::cvt(u.t[0]), S::cvt(u.t[1]));
+        }
+        return pack2(S::cvt(q[0]), S::cvt(q[1]));
+    }
+}
+template <class S, bool WORD>
+__device__ __forceinline__ void t_store2(typename S::T* q, typename S::T a, typename S::T b) {
+    if constexpr (WORD && S::kBytes == 4) {
+        *reinterpret_cast<float2*>(q) = make_float2(a, b);
+    } else if constexpr (WORD) {
+        union {
+            uint32_t w;
+            typename S::T t[2];
+        } u;
+        u.t[0] = a;
+        u.t[1] = b;
+        *reinterpret_cast<uint32_t*>(q) = u.w;
+    } else {
+        q[0] = a;
+        q[1] = b;
+    }
+}
+
+// Two cells x, x + 1 (x even) away from the row's ends.  Each pull of a
+// direction goes to a fixed offset, even or odd with e_a; WORD: nx is even, so
+// the stores and the pulls at even offsets are aligned pairs.
+// The random words are those of two single cells: direction a takes the low
+// half of each cell's word, a + 1 the high half, and one conversion rounds one
+// direction of both cells into the word that is stored.
+template <class S, bool SR, int Q, bool WORD>
+__device__ __forceinline__ void t_pair(const typename S::T* __restrict__ Pin, typename S::T* __restrict__ Pout, int x,
+                                       const TParams& p) {
+    F2 h[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+        const typename S::T* q = Pin + p.off[a] + x;
+        if ((t_e<Q>(a) & 1) == 0)
+            h[a] = t_load2<S, WORD>(q);
+        else
+            h[a] = t_load2<S, false>(q);
+    }
+    t_collide<Q, S::kBytes == 4>(p, h);
+    uint32_t r0 = 0, r1 = 0;
+    if (SR) {
+        r0 = t_hash((uint32_t)x ^ p.skey);
+        r1 = t_hash((uint32_t)(x + 1) ^ p.skey);
+    }
+    auto words = [&](uint32_t& wa, uint32_t& wb) {
+        r0 = r0 * 1664525u + 1013904223u;
+        r1 = r1 * 1664525u + 1013904223u;
+        wb = __byte_perm(r0, r1, 0x7632);
+        wa = __byte_perm(r0, r1, 0x5410) ^ wb;
+    };
+    auto put = [&](int a, F2 v, uint32_t w) {
+        float v0, v1;
+        unpack2(v, v0, v1);
+        typename S::T t0, t1;
+        if (SR) {
+            S::sr2(v0, v1, w, t0, t1);
+        } else {
+            S::put(&t0, v0);
+            S::put(&t1, v1);
+        }
+        t_store2<S, WORD>(Pout + p.plane[a] + x, t0, t1);
+    };
+    uint32_t wa = 0, wb = 0;
+#pragma unroll
+    for (int a = 1; a < Q; a += 2) {
+        if (SR) words(wa, wb);
+        put(a, h[a], wa);
+        put(a + 1, h[a + 1], wb);
+    }
+    if (SR) words(wa, wb);
+    put(0, h[0], wa);
+}
+
+// Each thread takes two neighbouring cells.  The step is bound by the
+// instructions it issues (84 to 86 % of the issue slots with one cell per
+// thread: 279 instructions a cell for D1V7 FP16, 455 for FP32, more than half of
+// them FP32 arithmetic), so the arithmetic of both cells goes through packed
+// instructions, and a pair shares its addresses and, in 16 bits, its stores:
+// 20 steps and the moments of 2^24 cells in FP16 3.10 -> 2.12 ms, of 3 000 017
+// in FP32 0.950 -> 0.718 ms.
+// Blocks within 3 cells of an end of the row take the cells one by one with the
+// periodic wrap; so do short rows (PAIRS false, one cell per thread), where the
+// pairs would leave SMs idle and a step lasts as long as its serial chain
+// (33 520 cells of FP32: 5.3 us a step in pairs, 4.3 with one cell).
+template <class S, bool SR, int Q, bool PAIRS>
+__global__ void __launch_bounds__(kTBlock) k_thermal_step(const typename S::T* __restrict__ Pin,
+                                                          typename S::T* __restrict__ Pout, TParams p) {
+    if (!PAIRS) {
+        const int x = (int)(blockIdx.x * kTBlock + threadIdx.x);
+        if (x < p.nx) t_cell<S, SR, Q>(Pin, Pout, x, p);
+        return;
+    }
+    const int first = (int)blockIdx.x * (2 * kTBlock);
+    const int x = first + 2 * (int)threadIdx.x;
+    if (first >= 3 && first + 2 * kTBlock + 3 <= p.nx) {
+        if ((p.nx & 1) == 0)
+            t_pair<S, SR, Q, true>(Pin, Pout, x, p);
+        else
+            t_pair<S, SR, Q, false>(Pin, Pout, x, p);
+    } else {
+        for (int k = 0; k < 2; ++k)
+            if (x + k < p.nx) t_cell<S, SR, Q>(Pin, Pout, x + k, p);
+    }
+}
+
+// The same for the start state, in plain expressions: their contraction is left
+// to the compiler, as it was when t_equilibrium was written so too, and start
+// states keep their bits (t_equilibrium's explicit order is the compiler's own
+// choice in the step kernel, which differs for orders 2 and 3).
 template <int Q, bool kLo>
-__device__ __forceinline__ void t_equilibrium(const TParams& p, float drho, float rho, float us, float dth,
-                                              float* heq) {
+__device__ __forceinline__ void t_start_equilibrium(const TParams& p, float drho, float rho, float us, float dth,
+                                                    float* heq) {
     const float srho = p.scale * rho;
     const float u2 = us * us;
     const float A1 = srho * p.c1 * us;
@@ -117,107 +453,6 @@ __device__ __forceinline__ void t_equilibrium(const TParams& p, float drho, floa
     }
 }
 
-// Error-free sum and product (Knuth TwoSum, FMA TwoProd) for the moment sums.
-__device__ __forceinline__ void t_two_sum(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-__device__ __forceinline__ void t_acc(float& hi, float& lo, float a, float b) {  // hi + lo += a b
-    const float p = a * b, pe = fmaf(a, b, -p);
-    float e;
-    t_two_sum(hi, p, hi, e);
-    lo += e + pe;
-}
-
-template <class S, bool SR, int Q>
-__global__ void __launch_bounds__(kTBlock) k_thermal_step(const typename S::T* __restrict__ Pin,
-                                                          typename S::T* __restrict__ Pout, TParams p) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= p.nx) return;
-    // FP32 storage: the moments as double-float sums (the first FP32
-    // rounding of a moment would otherwise recur in every step) and the
-    // hi + lo equilibrium weights; 16-bit storage rounds far coarser, so
-    // there plain FP32 sums over the pairs a, a + 1 suffice.
-    constexpr bool kExact = sizeof(typename S::T) == 4;
-    float h[Q], heq[Q];
-    float dh = 0.f, dl = 0.f, jh = 0.f, jl = 0.f, mh = 0.f, ml = 0.f;
-    // a block whose cells are all at least 3 cells from both ends of the row
-    // pulls without the periodic wrap, at fixed offsets from its own cell
-    const bool inner = (int)blockIdx.x * kTBlock >= 3 && ((int)blockIdx.x + 1) * kTBlock + 3 <= p.nx;
-    if (inner) {
-        const typename S::T* px = Pin + x;
-#pragma unroll
-        for (int a = 0; a < Q; ++a) h[a] = S::cvt(px[p.off[a]]);
-    } else {
-#pragma unroll
-        for (int a = 0; a < Q; ++a)
-            h[a] = S::cvt(Pin[(int64_t)a * p.nx + (p.nx >= 3 ? t_src<Q>(x, a, p.nx) : wrapx(x - p.e[a], p.nx))]);
-    }
-    if (kExact) {
-#pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            float e;
-            t_two_sum(dh, h[a], dh, e);
-            dl += e;
-            t_acc(jh, jl, h[a], p.xi[a]);
-            t_acc(mh, ml, h[a], p.xim[a]);
-        }
-    } else {
-        dh = h[0];
-        mh = p.xim[0] * h[0];
-#pragma unroll
-        for (int a = 1; a < Q; a += 2) {
-            const float sa = h[a] + h[a + 1], da = h[a] - h[a + 1];
-            dh += sa;
-            jh = fmaf(p.xi[a], da, jh);
-            mh = fmaf(p.xim[a], sa, mh);
-        }
-    }
-    const float drho = dh + dl, j = jh + jl, m2 = mh + ml;
-    const float rho = p.rho0 + drho * p.inv_scale;
-    float u, dth;
-    if (kExact) {
-        u = j * p.inv_scale / rho;
-        dth = m2 * p.inv_scale / rho - u * u;
-    } else {
-        const float ir = p.inv_scale / rho;
-        u = j * ir;
-        dth = m2 * ir - u * u;
-    }
-    t_equilibrium<Q, kExact>(p, drho, rho, u + p.tau * p.E, dth, heq);
-    const float omm = 1.f - p.omega;
-    float rest = dh;
-    uint32_t r = 0;
-    if (SR) r = t_hash((uint32_t)x ^ p.skey);
-    typename S::T* py = Pout + x;
-#pragma unroll
-    for (int a = 1; a < Q; a += 2) {
-        const float ha = fmaf(omm, h[a], p.omega * heq[a]);
-        const float hb = fmaf(omm, h[a + 1], p.omega * heq[a + 1]);
-        rest -= ha + hb;
-        typename S::T ta, tb;
-        if (SR) {
-            r = r * 1664525u + 1013904223u;
-            S::sr2(ha, hb, r ^ (r >> 16), ta, tb);
-        } else {
-            S::put(&ta, ha);
-            S::put(&tb, hb);
-        }
-        py[p.plane[a]] = ta;
-        py[p.plane[a + 1]] = tb;
-    }
-    rest += dl;
-    typename S::T t0, unused;
-    if (SR) {
-        r = r * 1664525u + 1013904223u;
-        S::sr2(rest, rest, r ^ (r >> 16), t0, unused);
-    } else {
-        S::put(&t0, rest);
-    }
-    Pout[x] = t0;
-}
-
 // f(x, 0) = f^eq(rho(x), u(x), thetabar(x)): P_a(y) holds f_a(y + e_a, 0).
 template <class S, int Q>
 __global__ void __launch_bounds__(kTBlock) k_thermal_init(typename S::T* __restrict__ P, const float* __restrict__ rho,
@@ -232,38 +467,50 @@ __global__ void __launch_bounds__(kTBlock) k_thermal_init(typename S::T* __restr
         const float uu = u ? u[x] : 0.f;
         const float dth = th ? th[x] - p.thw : 0.f;
         float heq[Q];
-        t_equilibrium<Q, sizeof(typename S::T) == 4>(p, (r - p.rho0) * p.scale, r, uu, dth, heq);
+        t_start_equilibrium<Q, sizeof(typename S::T) == 4>(p, (r - p.rho0) * p.scale, r, uu, dth, heq);
         S::put(P + (int64_t)a * p.nx + y, heq[a]);
     }
 }
 
-// rho, j = sum f xi, energy = sum f xi^2 per cell; FP64 block partials of the three
-template <class S, int Q>
+// rho, j = sum f xi, energy = sum f xi^2 per cell; FP64 block partials of the
+// three (TOTALS: the blocks stride over the cells and reduce once).  Cells at
+// least 3 from both ends pull at fixed offsets, without the wrap's loops (2^24
+// cells of D1V7 FP16: 0.226 ms with them and a block reduction per 256 cells).
+template <class S, int Q, bool TOTALS>
 __global__ void __launch_bounds__(kTBlock) k_thermal_moments(const typename S::T* __restrict__ P, float* rho_out,
                                                              float* j_out, float* e_out, float* f_out, int deviation,
                                                              double* partials, TParams p) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
     double acc[3] = {0.0, 0.0, 0.0};
-    if (x < p.nx) {
-        float drho = 0.f, j = 0.f, e2 = 0.f;
+    for (int64_t t = blockIdx.x; t * kTBlock < p.nx; t += gridDim.x) {
+        const int64_t xl = t * kTBlock + threadIdx.x;
+        if (xl < p.nx) {
+            const int x = (int)xl;
+            const bool inner = x >= 3 && xl + 3 < p.nx;
+            float h[Q];
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            const float h = S::cvt(P[(int64_t)a * p.nx + wrapx(x - p.e[a], p.nx)]) * p.inv_scale;
-            drho += h;
-            j += h * p.xi[a];
-            e2 += h * p.xi[a] * p.xi[a];
-            if (f_out) f_out[(int64_t)a * p.nx + x] = deviation ? h : p.f0[a] + h;
+            for (int a = 0; a < Q; ++a)
+                h[a] = S::cvt(P[inner ? p.off[a] + x : (int64_t)a * p.nx + wrapx(x - p.e[a], p.nx)]) * p.inv_scale;
+            float drho = 0.f, j = 0.f, e2 = 0.f;
+#pragma unroll
+            for (int a = 0; a < Q; ++a) {
+                drho += h[a];
+                j += h[a] * p.xi[a];
+                e2 += h[a] * p.xi[a] * p.xi[a];
+                if (f_out) f_out[(int64_t)a * p.nx + x] = deviation ? h[a] : p.f0[a] + h[a];
+            }
+            const float rho = p.rho0 + drho;
+            const float en = p.rho0 * p.thw + e2;  // sum_a f0_a xi_a^2 = rho0 thw
+            if (rho_out) rho_out[x] = rho;
+            if (j_out) j_out[x] = j;
+            if (e_out) e_out[x] = en;
+            if (TOTALS) {
+                acc[0] += rho;
+                acc[1] += j;
+                acc[2] += en;
+            }
         }
-        const float rho = p.rho0 + drho;
-        const float en = p.rho0 * p.thw + e2;  // sum_a f0_a xi_a^2 = rho0 thw
-        if (rho_out) rho_out[x] = rho;
-        if (j_out) j_out[x] = j;
-        if (e_out) e_out[x] = en;
-        acc[0] = rho;
-        acc[1] = j;
-        acc[2] = en;
     }
-    if (!partials) return;
+    if (!TOTALS) return;
     __shared__ double sh[kTBlock / 32][3];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int k = 0; k < 3; ++k) acc[k] = lbm::dev::warp_sum(acc[k]);
@@ -474,6 +721,13 @@ bool is_dev(const void* ptr) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(sms, 1);
+}
+
 unsigned tgrid(int64_t nx) { return (unsigned)((nx + kTBlock - 1) / kTBlock); }
 
 }  // namespace
@@ -638,6 +892,7 @@ lbm_status lbm_thermal_init(lbm_thermal* t, const float* rho, const float* u, co
 lbm_status lbm_thermal_step(lbm_thermal* t, int64_t n) {
     if (!t || n < 0) return LBM_ERR_INVALID_ARG;
     if (!t->has_state) return tfail(t, LBM_ERR_STATE, "lbm_thermal_step before lbm_thermal_init");
+    const int sms = sm_count();
     for (int64_t s = 0; s < n; ++s) {
         const TParams p = tparams(t);
         const bool sr = t->stochastic;
@@ -645,12 +900,16 @@ lbm_status lbm_thermal_step(lbm_thermal* t, int64_t n) {
             using S = decltype(st);
             using T = typename S::T;
             constexpr int Q = decltype(q)::value;
+            auto go = [&](auto kern, unsigned blocks) {
+                kern<<<blocks, kTBlock, 0, t->stream>>>((const T*)t->pop[t->cur], (T*)t->pop[t->cur ^ 1], p);
+            };
+            // a block of pairs for every SM at least
+            const bool pairs = t->nx >= (int64_t)2 * kTBlock * sms;
+            const unsigned blocks = pairs ? tgrid((t->nx + 1) / 2) : tgrid(t->nx);
             if (sr && S::kBytes == 2)
-                k_thermal_step<S, true, Q><<<tgrid(t->nx), kTBlock, 0, t->stream>>>((const T*)t->pop[t->cur],
-                                                                                    (T*)t->pop[t->cur ^ 1], p);
+                pairs ? go(k_thermal_step<S, true, Q, true>, blocks) : go(k_thermal_step<S, true, Q, false>, blocks);
             else
-                k_thermal_step<S, false, Q><<<tgrid(t->nx), kTBlock, 0, t->stream>>>((const T*)t->pop[t->cur],
-                                                                                     (T*)t->pop[t->cur ^ 1], p);
+                pairs ? go(k_thermal_step<S, false, Q, true>, blocks) : go(k_thermal_step<S, false, Q, false>, blocks);
             return 1;
         });
         t->cur ^= 1;
@@ -665,14 +924,22 @@ lbm_status lbm_thermal_moments(lbm_thermal* t, float* rho, float* j, float* ener
     for (const float* q : {rho, j, energy})
         if (q && !is_dev(q)) return tfail(t, LBM_ERR_INVALID_ARG, "lbm_thermal_moments: fields must be device memory");
     const TParams p = tparams(t);
+    unsigned blocks = tgrid(t->nx);
+    if (totals) {
+        blocks = std::min(blocks, (unsigned)sm_count() * 8u);
+    }
     t->launches += by_storage_q(t->storage, t->Q, [&](auto st, auto q) {
         using S = decltype(st);
-        k_thermal_moments<S, decltype(q)::value><<<tgrid(t->nx), kTBlock, 0, t->stream>>>(
-            (const typename S::T*)t->pop[t->cur], rho, j, energy, nullptr, 0, totals ? t->partials : nullptr, p);
+        constexpr int Q = decltype(q)::value;
+        const auto* pop = (const typename S::T*)t->pop[t->cur];
+        if (totals)
+            k_thermal_moments<S, Q, true><<<blocks, kTBlock, 0, t->stream>>>(pop, rho, j, energy, nullptr, 0, t->partials, p);
+        else
+            k_thermal_moments<S, Q, false><<<blocks, kTBlock, 0, t->stream>>>(pop, rho, j, energy, nullptr, 0, nullptr, p);
         return 1;
     });
     if (totals) {
-        t->launches += lbm::launch_reduce_slots(t->partials, tgrid(t->nx), 3, t->totals_dev, t->stream);
+        t->launches += lbm::launch_reduce_slots(t->partials, blocks, 3, t->totals_dev, t->stream);
         lbm_status s = tcuda(t, cudaMemcpyAsync(t->totals_host, t->totals_dev, sizeof(double) * 3,
                                                 cudaMemcpyDeviceToHost, t->stream), "lbm_thermal_moments totals");
         if (s != LBM_OK) return s;
@@ -692,7 +959,7 @@ lbm_status lbm_thermal_populations(lbm_thermal* t, float* f, int deviation) {
     const TParams p = tparams(t);
     t->launches += by_storage_q(t->storage, t->Q, [&](auto st, auto q) {
         using S = decltype(st);
-        k_thermal_moments<S, decltype(q)::value><<<tgrid(t->nx), kTBlock, 0, t->stream>>>(
+        k_thermal_moments<S, decltype(q)::value, false><<<tgrid(t->nx), kTBlock, 0, t->stream>>>(
             (const typename S::T*)t->pop[t->cur], nullptr, nullptr, nullptr, f, deviation, nullptr, p);
         return 1;
     });
