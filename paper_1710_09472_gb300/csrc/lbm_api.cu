@@ -308,7 +308,7 @@ void set_units(lbm_ctx* c) {
     if (nx >= lbm::kMinStagedRow) {
         const int up = lbm::kPitch;
         const int cols = std::min(lbm::kRowSmem / (int)(3 * c->Q * pop_elem_bytes(c->storage)), lbm::kMaxUnit);
-        const int most = std::max(up, std::min(kMaxSegment, cols / up * up));
+        const int most = std::max(up, std::min(c->Q <= 9 ? 2 * kMaxSegment : kMaxSegment, cols / up * up));
         auto padded = [&](int n) { return (n + up - 1) / up * up; };
         if (padded(nx) > cols) c->nseg = (nx + most - 1) / most;
         c->seglen = padded((nx + c->nseg - 1) / c->nseg);

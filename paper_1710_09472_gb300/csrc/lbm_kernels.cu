@@ -18,7 +18,7 @@
 
 #include <cub/device/device_scan.cuh>
 
-#include "lbm_device.cuh"
+#include "lbm_step.cuh"
 
 namespace lbm {
 namespace {
@@ -190,11 +190,8 @@ __global__ void k_row_starts(const uint32_t* __restrict__ nbr, const uint32_t* _
 // Moments of f(x, t) and FP64 block partials of the fluid totals
 // partials[block] = {sum rho, sum j_x, sum j_y, sum j_z}.
 // ---------------------------------------------------------------------------
-template <class L, class S>
-__device__ __forceinline__ void cell_moments(const typename S::T* __restrict__ P, uint32_t m, const KParams& p,
-                                             const Cell& c, float& rho, float* j) {
-    float h[L::Q];
-    dev::pull<L, S>(P, p, m, c, h);
+template <class L>
+__device__ __forceinline__ void cell_moments(const float* h, const KParams& p, float& rho, float* j) {
     float drho = 0.f, jj[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int a = 0; a < L::Q; ++a) {
@@ -226,7 +223,9 @@ __global__ void __launch_bounds__(kBlock) k_moments(const typename S::T* __restr
             const uint32_t m = __ldg(nbr + c.cell);
             float r = 0.f, j[3] = {0.f, 0.f, 0.f};
             if (!(m & kSolidBit)) {
-                cell_moments<L, S>(P, m, p, c, r, j);
+                float h[L::Q];
+                dev::pull<L, S>(P, p, m, c, h);
+                cell_moments<L>(h, p, r, j);
                 if (TOTALS) {
                     acc[0] += (double)r;
                     acc[1] += (double)j[0];
@@ -262,6 +261,140 @@ __global__ void __launch_bounds__(kBlock) k_moments(const typename S::T* __restr
             }
         }
     }
+}
+
+// The same over units staged in shared memory (the step kernel's stages, links
+// and cell order; no outputs to stage, so one barrier per unit and twice the
+// blocks per SM).  The general kernel spends 370 instructions a cell on
+// addresses and links: 0.24 ms on 256^3 porous D3V19 FP16, 0.135 of it floor.
+template <class L, class S, bool TOTALS>
+__global__ void __launch_bounds__(256) k_moments_rows(const typename S::T* __restrict__ P, float* __restrict__ rho_out,
+                                                      float* __restrict__ j_out, double* __restrict__ partials,
+                                                      int gcap, int dcap, KParams p) {
+    using T = typename S::T;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int rs = p.seglen, U = p.ny * p.nz * p.nseg, G = gridDim.x;
+    const bool halo = p.nseg > 1;
+    const stepk::StageLayout<L, S> lay{rs, p.lorder, gcap, dcap, dev::halo_bytes(L::Q, p.nseg, S::kBytes)};
+    const int sbytes = lay.bytes();
+    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ uint32_t gstart[2], dstart[2];
+    const bool issuer = (int)threadIdx.x == (int)blockDim.x - 32;
+    auto stage = [&](int k, int unit) {
+        stepk::stage_unit<L, S, 0>(smem_raw + k * sbytes, lay, &bar[k], P, unit, __ldg(p.rowG + unit),
+                                   __ldg(p.rowG + unit + 1), &gstart[k], &dstart[k], p);
+    };
+    if (threadIdx.x == 0) {
+        dev::mbar_init(&bar[0], 1);
+        dev::mbar_init(&bar[1], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (halo && dev::halo_thread<L>())
+        dev::halo_put<L, true>(lay.halo(smem_raw), dev::halo_fetch<L, true>(P, dev::unit_at<0>(p, blockIdx.x), p));
+    __syncthreads();
+    if (issuer && (int)blockIdx.x < U) stage(0, blockIdx.x);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    bool ok = true;
+    int it = 0;
+    for (int u = blockIdx.x; u < U; u += G, ++it) {
+        const int cs = it & 1, un = u + G;
+        unsigned char* st = smem_raw + cs * sbytes;
+        const uint32_t g0 = __ldg(p.rowG + u), g1 = __ldg(p.rowG + u + 1);
+        if (ok && !dev::mbar_wait(&bar[cs], (uint32_t)(it >> 1) & 1u)) {
+            ok = false;
+            if (p.status) atomicExch(p.status, 5);
+            dev::pause_cycles(1ll << 22);  // let this block's copies in flight land
+        }
+        T* buf = lay.rows(st);
+        dev::patch_links<true, true>(buf, rs, lay.halo(st), L::Q, lay.links(st), gstart[cs], g0, g1, lay.descs(st),
+                                     dstart[cs]);
+        dev::fence_proxy_async();  // this stage is overwritten by copies after the next barrier
+        // bounced values in place; every thread is past its reads of the other stage
+        ok = __syncthreads_and(ok) != 0;
+        if (issuer && ok && un < U) stage(cs ^ 1, un);
+        const bool fetch = halo && un < U && dev::halo_thread<L>();
+        T hv{};
+        if (fetch) hv = dev::halo_fetch<L, true>(P, dev::unit_at<0>(p, un), p);
+        const uint16_t* ord = lay.order(st);
+        const int nf = ord[0];
+        const dev::UnitAt at = dev::unit_at<0>(p, u);
+        const int64_t first = (int64_t)at.row * p.nx + at.x0;
+        for (int i = threadIdx.x; i < at.len; i += blockDim.x) {
+            const int x = (int)ord[8 + i];
+            float r = 0.f, j[3] = {0.f, 0.f, 0.f};
+            if (i < nf) {
+                // columns x - 1 and x + 1, as in the step kernel
+                const T* bm = buf + (x == 0 ? at.len - 1 : x - 1);
+                const T* bp = buf + (x == at.len - 1 ? 0 : x + 1);
+                int rm = rs, rp = rs;
+                if (halo && x == 0) {
+                    bm = lay.halo(st);
+                    rm = 1;
+                }
+                if (halo && x == at.len - 1) {
+                    bp = lay.halo(st) + L::Q;
+                    rp = 1;
+                }
+                float h[L::Q];
+#pragma unroll
+                for (int a = 0; a < L::Q; ++a) {
+                    const int ex = L::c(a, 0), s = pop_slot<L>(a);
+                    h[a] = S::cvt(ex > 0 ? bm[s * rm] : (ex < 0 ? bp[s * rp] : buf[s * rs + x]));
+                }
+                cell_moments<L>(h, p, r, j);
+                if (TOTALS) {
+                    acc[0] += (double)r;
+                    acc[1] += (double)j[0];
+                    if (L::D >= 2) acc[2] += (double)j[1];
+                    if (L::D == 3) acc[3] += (double)j[2];
+                }
+            }
+            if (rho_out) rho_out[first + x] = r;
+            if (j_out) {
+#pragma unroll
+                for (int d = 0; d < L::D; ++d) j_out[(int64_t)d * p.N + first + x] = j[d];
+            }
+        }
+        if (halo) {  // the halo values of the next unit, before its link pass
+            if (fetch) dev::halo_put<L, true>(lay.halo(smem_raw + (cs ^ 1) * sbytes), hv);
+            __syncthreads();
+        }
+    }
+    if (TOTALS) {
+        __shared__ double sh[256 / 32][4];
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) / 32;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            acc[k] = dev::warp_sum(acc[k]);
+            if (lane == 0) sh[wid][k] = acc[k];
+        }
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            double v = 0.0;
+            for (int w = 0; w < nw; ++w) v += sh[w][threadIdx.x];
+            partials[(int64_t)blockIdx.x * 4 + threadIdx.x] = v;
+        }
+    }
+}
+
+// Launches it where the context has units, two stages fit the step kernel's
+// budget and there are units for every SM; returns the blocks, 0 where it does
+// not run.
+template <class L, class S, bool TOTALS>
+int64_t launch_moments_rows(const void* pop, float* rho, float* j, double* partials, int64_t most, const KParams& p,
+                            cudaStream_t s) {
+    if (!p.rorder) return 0;
+    const int gcap = dev::window_cap(p.max_row_links, S::kBytes), dcap = dev::window_cap(p.max_row_links, 4);
+    const size_t smem = 2 * ((size_t)L::Q * p.seglen * S::kBytes + 2 * (size_t)p.lorder + gcap + dcap +
+                             dev::halo_bytes(L::Q, p.nseg, S::kBytes));
+    if (smem > stepk::kSmemBudget) return 0;
+    auto kern = k_moments_rows<L, S, TOTALS>;
+    const stepk::Shape sh = stepk::launch_shape(kern, p.seglen, smem);
+    const int units = p.ny * p.nz * p.nseg;
+    if (sh.blocks <= 0 || units < sh.sms) return 0;
+    const int64_t blocks = std::min<int64_t>(std::min(sh.blocks, units), most);
+    kern<<<(unsigned)blocks, sh.threads, smem, s>>>((const typename S::T*)pop, rho, j, partials, gcap, dcap, p);
+    return blocks;
 }
 
 // One block sums interleaved per-block slots in a fixed order (deterministic);
@@ -498,12 +631,16 @@ int launch_moments(int vel, int storage, const void* pop, const uint32_t* nbr, f
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         blocks = std::min<int64_t>(tiles, (int64_t)std::max(sms, 1) * kTotalsPerSm);
     }
-    if (n_partials) *n_partials = blocks;
     return dispatch_lattice(vel, [&](auto lat) {
         using L = decltype(lat);
         return dispatch_storage(storage, [&](auto st) {
             using S = decltype(st);
             using T = typename S::T;
+            // the partials of one launch: as many as the general kernel has tiles at most
+            const int64_t staged = partials ? launch_moments_rows<L, S, true>(pop, rho, j, partials, tiles, p, s)
+                                            : launch_moments_rows<L, S, false>(pop, rho, j, nullptr, tiles, p, s);
+            if (n_partials) *n_partials = staged ? staged : blocks;
+            if (staged) return 1;
             if (partials)
                 k_moments<L, S, true><<<(unsigned)blocks, l.block, 0, s>>>((const T*)pop, nbr, rho, j, partials, chunks, p);
             else

@@ -851,13 +851,17 @@ int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef
     using T = typename S::T;
     const S* tag = nullptr;
     bool done;
-    // the compile-time strides only for the benchmarked lattices (D2V9, D3V19);
-    // the others take the run-time stride (fewer instantiations to compile)
+    // the compile-time strides for the benchmarked lattices (D2V9, D3V19, and 256
+    // for 16-bit D3V27); the others take the run-time stride (fewer
+    // instantiations to compile)
     constexpr bool kFixed = L::Q == 9 || L::Q == 19;
-    if (p.lmu_tab)  // the local-mu model (D2V9, D3V19 only): run-time row stride
-        done = kFixed && launch_rows<L, S, FORCE, EF, SR, 0, kFixed>(tag, fin, fout, nbr, Ef, p, s);
-    else if (kFixed && p.nx == 256)
-        done = launch_rows<L, S, FORCE, EF, SR, kFixed ? 256 : 0>(tag, fin, fout, nbr, Ef, p, s);
+    constexpr bool kFixed256 = kFixed || (L::Q == 27 && whole_row<L, S>(256));
+    if (p.lmu_tab)  // the local-mu model (D2V9, D3V19 only)
+        done = kFixed && (p.nx == 256 && p.nseg == 1
+                              ? launch_rows<L, S, FORCE, EF, SR, kFixed ? 256 : 0, kFixed>(tag, fin, fout, nbr, Ef, p, s)
+                              : launch_rows<L, S, FORCE, EF, SR, 0, kFixed>(tag, fin, fout, nbr, Ef, p, s));
+    else if (kFixed256 && p.nx == 256 && p.nseg == 1)
+        done = launch_rows<L, S, FORCE, EF, SR, kFixed256 ? 256 : 0>(tag, fin, fout, nbr, Ef, p, s);
     else if (kFixed && p.nx == 512 && p.nseg == 1)
         done = launch_rows<L, S, FORCE, EF, SR, kFixed && whole_row<L, S>(512) ? 512 : 0>(tag, fin, fout, nbr, Ef, p, s);
     else

@@ -485,11 +485,15 @@ __global__ void __launch_bounds__(kTBlock) k_thermal_moments(const typename S::T
         const int64_t xl = t * kTBlock + threadIdx.x;
         if (xl < p.nx) {
             const int x = (int)xl;
-            const bool inner = x >= 3 && xl + 3 < p.nx;
             float h[Q];
+            if (x >= 3 && xl + 3 < p.nx) {
 #pragma unroll
-            for (int a = 0; a < Q; ++a)
-                h[a] = S::cvt(P[inner ? p.off[a] + x : (int64_t)a * p.nx + wrapx(x - p.e[a], p.nx)]) * p.inv_scale;
+                for (int a = 0; a < Q; ++a) h[a] = S::cvt(P[p.off[a] + x]) * p.inv_scale;
+            } else {
+#pragma unroll
+                for (int a = 0; a < Q; ++a)
+                    h[a] = S::cvt(P[(int64_t)a * p.nx + wrapx(x - p.e[a], p.nx)]) * p.inv_scale;
+            }
             float drho = 0.f, j = 0.f, e2 = 0.f;
 #pragma unroll
             for (int a = 0; a < Q; ++a) {
