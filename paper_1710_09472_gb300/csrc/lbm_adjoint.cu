@@ -59,11 +59,8 @@ __global__ void k_fold_partials(float* __restrict__ part, double* __restrict__ a
 
 int launch_fold_partials(float* part, double* acc, int D, const KParams& p, cudaStream_t s) {
     const int64_t rows = (int64_t)D * p.ny * p.nz;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int threads = p.nx >= 256 ? 256 : ((p.nx + 31) / 32) * 32;
-    const int64_t want = rows * ((p.nx + threads - 1) / threads), cap = (int64_t)(sms > 0 ? sms : 1) * 8;
+    const int64_t want = rows * ((p.nx + threads - 1) / threads), cap = (int64_t)sm_count() * 8;
     k_fold_partials<<<(unsigned)(want < cap ? want : cap), threads, 0, s>>>(part, acc, rows, p.nx, p.nxp);
     return 1;
 }

@@ -499,9 +499,9 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_step(
 //     (y + e_ay, z + e_az), read at x + e_ax;
 //   - its windows of lam_{t+1}'s link buffer (bounced gathers) and of the
 //     link descriptors;
-// all by bulk asynchronous copies, completing on the stage's mbarrier, armed
-// and issued by lane 0 of the last warp (as in the forward's row-staged
-// kernel; waits are bounded).  One pass over the
+// all by bulk asynchronous copies, completing on the stage's mbarrier, issued by
+// lane 0 of the last two warps (waits are bounded, as in the forward's
+// row-staged kernel).  One pass over the
 // unit's links patches both bounced reads into the staged rows (the solid
 // neighbour's slot, read by that cell alone), so cells read their rows
 // without link logic.  Thread i takes the i-th cell of the row's order, so
@@ -535,39 +535,50 @@ struct AdjLayout {
     __device__ unsigned char* lhalo(unsigned char* st) const { return phalo(st) + hP; }
 };
 
-// One thread: arms a stage's mbarrier with the byte count of unit `unit`
-// (links [g0, g1)), records where its windows start (ws[0]: P_t's link
-// window; ws[1]: lam's link window and the descriptor window, which start at
-// the same element), and issues the unit's copies into stage st, all
-// completing on bar.  With gE, the unit's dL/dE partials (accumulated in
-// place, stored back after the unit); with Ef, its E.
-template <class L, class S, int RS>
-__device__ __forceinline__ void adj_stage(unsigned char* st, const AdjLayout<L, S>& lay, uint64_t* bar,
-                                          const typename S::T* P, const float* lam, const float* gE, const float* Ef,
-                                          int unit, uint32_t g0, uint32_t g1, uint32_t* ws, const KParams& p) {
+// Two threads fill a stage with unit `unit` (links [g0, g1)), all copies
+// completing on bar.  The first (adj_stage_state) arms the mbarrier with the
+// byte count of all, records where the windows start (ws[0]: P_t's link window;
+// ws[1]: lam's link window and the descriptor window, which start at the same
+// element) and copies P_t's rows, the cell order, P_t's links and the
+// descriptors; the other (adj_stage_lam) lam's rows and links and, where they
+// exist, the unit's dL/dE partials (accumulated in place, stored back after the
+// unit) and its E.  A copy holds its issuing thread for a hundred cycles or
+// more and there are up to 28; the phase cannot complete before the first
+// thread has armed it, so the order of the two does not matter.
+template <class L, class S, int RS, int MODE>
+__device__ __forceinline__ void adj_stage_state(unsigned char* st, const AdjLayout<L, S>& lay, uint64_t* bar,
+                                                const typename S::T* P, int unit, uint32_t g0, uint32_t g1,
+                                                uint32_t* ws, const KParams& p) {
     uint64_t pb0, pb1, lb0, lb1;
     dev::window_bytes(g0, g1, S::kBytes, pb0, pb1);
     dev::window_bytes(g0, g1, 4, lb0, lb1);
     ws[0] = (uint32_t)(pb0 / S::kBytes);
     ws[1] = (uint32_t)(lb0 / 4);
-    const dev::UnitAt at = dev::unit_at<RS>(p, unit);
-    const uint32_t fb = (uint32_t)lay.rs * 4u;  // bytes of a field row
-    dev::mbar_expect_tx(bar, (uint32_t)(lay.prow() + lay.lrow()) + 2u * (uint32_t)lay.lorder + (uint32_t)(pb1 - pb0) +
-                                 2u * (uint32_t)(lb1 - lb0) + (lay.gerow ? L::D * fb : 0u) +
-                                 (lay.efrow ? L::D * fb : 0u));
-    dev::stage_rows<L, RS, true>(reinterpret_cast<typename S::T*>(lay.prows(st)), P, at, bar, p);
-    dev::stage_rows<L, RS, false>(reinterpret_cast<float*>(lay.lrows(st)), lam, at, bar, p);
+    dev::mbar_expect_tx(bar, (uint32_t)(lay.prow() + lay.lrow() + lay.gerow + lay.efrow) +
+                                 2u * (uint32_t)lay.lorder + (uint32_t)(pb1 - pb0) + 2u * (uint32_t)(lb1 - lb0));
+    dev::stage_rows<L, RS, MODE, true>(reinterpret_cast<typename S::T*>(lay.prows(st)), P,
+                                      dev::unit_at<RS, MODE>(p, unit), bar, p);
     dev::bulk_load(lay.order(st), p.rorder + (int64_t)unit * lay.lorder, 2u * (uint32_t)lay.lorder, bar);
     if (pb1 > pb0)
         dev::bulk_load(lay.plinks(st), reinterpret_cast<const unsigned char*>(P) + p.gofs + pb0, (uint32_t)(pb1 - pb0),
                        bar);
-    if (lb1 > lb0) {
-        dev::bulk_load(lay.llinks(st), reinterpret_cast<const unsigned char*>(lam) + p.lgofs + lb0,
-                       (uint32_t)(lb1 - lb0), bar);
+    if (lb1 > lb0)
         dev::bulk_load(lay.descs(st), reinterpret_cast<const unsigned char*>(p.ldesc) + lb0, (uint32_t)(lb1 - lb0),
                        bar);
-    }
-    const int64_t f0 = (int64_t)at.row * p.nxp + at.x0;
+}
+template <class L, class S, int RS, int MODE>
+__device__ __forceinline__ void adj_stage_lam(unsigned char* st, const AdjLayout<L, S>& lay, uint64_t* bar,
+                                              const float* lam, const float* gE, const float* Ef, int unit,
+                                              uint32_t g0, uint32_t g1, const KParams& p) {
+    uint64_t lb0, lb1;
+    dev::window_bytes(g0, g1, 4, lb0, lb1);
+    dev::stage_rows<L, RS, MODE, false>(reinterpret_cast<float*>(lay.lrows(st)), lam,
+                                       dev::unit_at<RS, MODE>(p, unit), bar, p);
+    if (lb1 > lb0)
+        dev::bulk_load(lay.llinks(st), reinterpret_cast<const unsigned char*>(lam) + p.lgofs + lb0,
+                       (uint32_t)(lb1 - lb0), bar);
+    const uint32_t fb = (uint32_t)lay.rs * 4u;  // bytes of a field row
+    const int64_t f0 = (int64_t)unit * lay.rs;
     if (lay.gerow) {
 #pragma unroll
         for (int d = 0; d < L::D; ++d)
@@ -580,7 +591,7 @@ __device__ __forceinline__ void adj_stage(unsigned char* st, const AdjLayout<L, 
     }
 }
 
-template <class L, class S, int FORCE, bool EF, bool WIN, int STAGES, int RS, bool LMU = false>
+template <class L, class S, int FORCE, bool EF, bool WIN, int STAGES, int RS, int MODE, bool LMU = false>
 __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __restrict__ P,
                                                          const float* __restrict__ lam_in,
                                                          float* __restrict__ lam_out,
@@ -590,22 +601,26 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
                                                          double* __restrict__ slots, int gcapP, int gcapL, KParams p) {
     using T = typename S::T;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    // RS: whole rows of that many cells, a compile-time stride; 0: a run-time one, whole rows or segments
+    // RS: units of that many columns (a compile-time stride; 0: a run-time one).
+    // MODE: rows of exactly RS cells (kExactRow), rows (kWholeRow) or segments
+    constexpr bool kOne = MODE != kSegment, kExact = RS && MODE == kExactRow;
     const int rs = RS ? RS : p.seglen;
-    const bool halo = !RS && p.nseg > 1;
+    const bool halo = !kOne;
     const AdjLayout<L, S> lay{rs, p.lorder, gcapP, gcapL, gE ? L::D * rs * 4 : 0, EF ? L::D * rs * 4 : 0,
-                              RS ? 0 : dev::halo_bytes(L::Q, p.nseg, S::kBytes),
-                              RS ? 0 : dev::halo_bytes(L::Q, p.nseg, 4)};
+                              kOne ? 0 : dev::halo_bytes(L::Q, p.nseg, S::kBytes),
+                              kOne ? 0 : dev::halo_bytes(L::Q, p.nseg, 4)};
     const int sbytes = lay.bytes();
     float* outrow = reinterpret_cast<float*>(smem_raw + STAGES * sbytes);
     __shared__ __align__(8) uint64_t bar[STAGES];
     __shared__ uint32_t wstart[STAGES][2];
     float* lamG_out = link_part(lam_out, p);
-    const int U = p.ny * p.nz * (RS ? 1 : p.nseg);
+    const int U = p.ny * p.nz * (kOne ? 1 : p.nseg);
     const int G = gridDim.x;
     const bool leader = threadIdx.x == 0;
     const int warp = (int)(threadIdx.x >> 5), nw = (int)(blockDim.x >> 5), lane = (int)(threadIdx.x & 31);
-    const bool issuer = (int)threadIdx.x == (int)blockDim.x - 32;  // lane 0 of the last warp
+    // lane 0 of the last warp and of the one before it (the same in a block of one warp)
+    const bool issuer = (int)threadIdx.x == (int)blockDim.x - 32;
+    const bool lam_issuer = nw > 1 ? (int)threadIdx.x == (int)blockDim.x - 64 : issuer;
     auto range = [&](int unit, uint32_t& g0, uint32_t& g1) {
         g0 = g1 = 0u;
         if (unit < U) {
@@ -620,19 +635,21 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
     }
     static_assert(STAGES == 2, "the halo values are fetched one unit ahead");
     if (halo && dev::halo_thread<L>()) {
-        const dev::UnitAt at = dev::unit_at<RS>(p, blockIdx.x);
+        const dev::UnitAt at = dev::unit_at<RS, MODE>(p, blockIdx.x);
         dev::halo_put<L, true>(reinterpret_cast<T*>(lay.phalo(smem_raw)), dev::halo_fetch<L, true>(P, at, p));
         dev::halo_put<L, false>(reinterpret_cast<float*>(lay.lhalo(smem_raw)), dev::halo_fetch<L, false>(lam_in, at, p));
     }
     __syncthreads();
-    if (issuer) {
+    if (issuer || lam_issuer) {
 #pragma unroll
         for (int k = 0; k < STAGES - 1; ++k) {
             const int uk = blockIdx.x + k * G;
             if (uk < U) {
                 uint32_t g0, g1;
                 range(uk, g0, g1);
-                adj_stage<L, S, RS>(smem_raw + k * sbytes, lay, &bar[k], P, lam_in, gE, Ef, uk, g0, g1, wstart[k], p);
+                unsigned char* st = smem_raw + k * sbytes;
+                if (issuer) adj_stage_state<L, S, RS, MODE>(st, lay, &bar[k], P, uk, g0, g1, wstart[k], p);
+                if (lam_issuer) adj_stage_lam<L, S, RS, MODE>(st, lay, &bar[k], lam_in, gE, Ef, uk, g0, g1, p);
             }
         }
     }
@@ -660,33 +677,35 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
         const uint32_t d0 = wstart[cs][1];
         T* phal = reinterpret_cast<T*>(lay.phalo(st));
         float* lhal = reinterpret_cast<float*>(lay.lhalo(st));
-        dev::patch_links<true, RS == 0>(prow, rs, phal, L::Q, reinterpret_cast<const T*>(lay.plinks(st)),
+        dev::patch_links<true, !kOne>(prow, rs, phal, L::Q, reinterpret_cast<const T*>(lay.plinks(st)),
                                         wstart[cs][0], g0, g1, desc, d0);
-        dev::patch_links<false, RS == 0>(lrow, rs, lhal, L::Q, reinterpret_cast<const float*>(lay.llinks(st)), d0, g0,
+        dev::patch_links<false, !kOne>(lrow, rs, lhal, L::Q, reinterpret_cast<const float*>(lay.llinks(st)), d0, g0,
                                          g1, desc, d0);
         dev::bulk_wait_read();  // this thread's bulk stores of the previous unit have read their sources
         // bounced values in place, output rows free; a timeout anywhere in
         // the block stops the copies
         ok = __syncthreads_and(ok) != 0;
-        if (issuer && ok && un < U) {
+        if ((issuer || lam_issuer) && ok && un < U) {
             // refill the stage of the previous unit (every thread is past its
             // reads of it and its wait on that stage's barrier)
             uint32_t n0, n1;
             range(un, n0, n1);
-            adj_stage<L, S, RS>(smem_raw + sn * sbytes, lay, &bar[sn], P, lam_in, gE, Ef, un, n0, n1, wstart[sn], p);
+            unsigned char* sst = smem_raw + sn * sbytes;
+            if (issuer) adj_stage_state<L, S, RS, MODE>(sst, lay, &bar[sn], P, un, n0, n1, wstart[sn], p);
+            if (lam_issuer) adj_stage_lam<L, S, RS, MODE>(sst, lay, &bar[sn], lam_in, gE, Ef, un, n0, n1, p);
         }
         const bool fetch = halo && un < U && dev::halo_thread<L>();
         T hvP{};
         float hvL = 0.f;
         if (fetch) {
-            const dev::UnitAt next = dev::unit_at<RS>(p, un);
+            const dev::UnitAt next = dev::unit_at<RS, MODE>(p, un);
             hvP = dev::halo_fetch<L, true>(P, next, p);
             hvL = dev::halo_fetch<L, false>(lam_in, next, p);
         }
         const int nf = ord[0];
-        const dev::UnitAt at = dev::unit_at<RS>(p, u);
+        const dev::UnitAt at = dev::unit_at<RS, MODE>(p, u);
         const int nx = at.len;  // cells of the unit
-        const uint32_t rowbase = (uint32_t)at.row * (uint32_t)(RS ? RS : p.nx) + (uint32_t)at.x0;  // first cell
+        const uint32_t rowbase = (uint32_t)at.row * (uint32_t)(kExact ? RS : p.nx) + (uint32_t)at.x0;  // first cell
         for (int i = threadIdx.x; i < nx; i += blockDim.x) {
             const int x = (int)ord[8 + i];
             if (i < nf) {
@@ -710,7 +729,7 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
 #pragma unroll
                 for (int a = 0; a < L::Q; ++a) {
                     const int ex = L::c(a, 0), s = pop_slot<L>(a);
-                    const int sm = s * (RS ? RS : rm), sp = s * (RS ? RS : rp);
+                    const int sm = s * (kOne ? rs : rm), sp = s * (kOne ? rs : rp);
                     h[a] = S::cvt(ex > 0 ? pm[sm] : (ex < 0 ? pp[sp] : prow[s * rs + x])) * p.inv_scale;
                     lt[a] = ex > 0 ? lp[sp] : (ex < 0 ? lm[sm] : lrow[s * rs + x]);
                 }
@@ -777,10 +796,7 @@ inline Launch grid_of(const KParams& p) {
 constexpr int kAdjPerSm = 8;
 inline int64_t strided_blocks(const KParams& p) {
     const Launch l = grid_of(p);
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t tiles = (int64_t)l.grid.x * l.grid.y, cap = (int64_t)(sms > 0 ? sms : 1) * kAdjPerSm;
+    const int64_t tiles = (int64_t)l.grid.x * l.grid.y, cap = (int64_t)sm_count() * kAdjPerSm;
     return tiles < cap ? tiles : cap;
 }
 
@@ -806,11 +822,12 @@ constexpr int kAdjStages = 2;
 constexpr int kAdjThreads = 256;
 constexpr size_t kAdjSmemBudget = 200 * 1024;
 
-template <class L, class S, int FORCE, bool EF, bool WIN, int RS, bool LMU = false>
+template <class L, class S, int FORCE, bool EF, bool WIN, int RS, int MODE, bool LMU = false>
 bool launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
                  const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
                  const KParams& p, cudaStream_t s) {
-    if (!p.rorder || (RS && (RS != p.nx || p.nseg != 1))) return false;
+    if (!p.rorder || (RS && RS != p.seglen) || (MODE == kExactRow && RS != p.nx) || (MODE == kSegment) != (p.nseg > 1))
+        return false;
     const int gcapP = dev::window_cap(p.max_row_links, S::kBytes);
     const int gcapL = dev::window_cap(p.max_row_links, 4);
     const int rs = p.seglen, hP = dev::halo_bytes(L::Q, p.nseg, S::kBytes), hL = dev::halo_bytes(L::Q, p.nseg, 4);
@@ -826,7 +843,7 @@ bool launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const ui
     const size_t smem_ref = smem_for(gerow);
     if (smem_ref > kAdjSmemBudget) return false;
     const int threads = p.seglen >= kAdjThreads ? kAdjThreads : ((p.seglen + 31) / 32) * 32;
-    auto kern = k_adjoint_rows<L, S, FORCE, EF, WIN, kAdjStages, RS, LMU>;
+    auto kern = k_adjoint_rows<L, S, FORCE, EF, WIN, kAdjStages, RS, MODE, LMU>;
     // persistent grid: co-resident blocks per SM (occupancy API) x SMs,
     // cached per instantiation and shared-memory size
     static std::mutex mu;
@@ -856,22 +873,41 @@ bool launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const ui
     return true;
 }
 
-// The shared-memory row stride (the row length) is a compile-time constant
-// for rows of 256 or 512 cells (as in the step kernel).
+// Rows or segments at a run-time stride.
+template <class L, class S, int FORCE, bool EF, bool WIN, bool LMU = false>
+bool launch_rows_any(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
+                     const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
+                     const KParams& p, cudaStream_t s) {
+    return p.nseg > 1 ? launch_rows_rs<L, S, FORCE, EF, WIN, 0, kSegment, LMU>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j,
+                                                                               gE, slots, slot_blocks, p, s)
+                      : launch_rows_rs<L, S, FORCE, EF, WIN, 0, kWholeRow, LMU>(P, lam_in, lam_out, nbr, Ef, w_rho,
+                                                                                w_j, gE, slots, slot_blocks, p, s);
+}
+
+// The shared-memory row stride is a compile-time constant for the usual units,
+// as in the step kernel.
 template <class L, class S, int FORCE, bool EF, bool WIN>
 bool launch_rows(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
                  const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
                  const KParams& p, cudaStream_t s) {
     // the compile-time strides only for the benchmarked lattices (D2V9, D3V19)
     constexpr bool kFixed = L::Q == 9 || L::Q == 19;
-    if (kFixed && p.nx == 256)
-        return launch_rows_rs<L, S, FORCE, EF, WIN, kFixed ? 256 : 0>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,
-                                                                       slots, slot_blocks, p, s);
-    if (kFixed && p.nx == 512 && p.nseg == 1)
-        return launch_rows_rs<L, S, FORCE, EF, WIN, kFixed && whole_row<L, S>(512) ? 512 : 0>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,
-                                                                       slots, slot_blocks, p, s);
-    return launch_rows_rs<L, S, FORCE, EF, WIN, 0>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots, slot_blocks,
-                                                    p, s);
+    if constexpr (kFixed) {
+        constexpr int kSeg = segment_columns<L>();
+        if (p.nseg > 1 && p.seglen == kSeg)
+            return launch_rows_rs<L, S, FORCE, EF, WIN, kSeg, kSegment>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,
+                                                                        slots, slot_blocks, p, s);
+        if (p.nseg == 1 && p.nx == 256)
+            return launch_rows_rs<L, S, FORCE, EF, WIN, 256, kExactRow>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,
+                                                                        slots, slot_blocks, p, s);
+        if constexpr (whole_row<L, S>(512)) {
+            if (p.nseg == 1 && p.nx == 512)
+                return launch_rows_rs<L, S, FORCE, EF, WIN, 512, kExactRow>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j,
+                                                                            gE, slots, slot_blocks, p, s);
+        }
+    }
+    return launch_rows_any<L, S, FORCE, EF, WIN>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots, slot_blocks, p,
+                                                 s);
 }
 
 // Launchers for one storage type (instantiated in one translation unit per
@@ -903,8 +939,8 @@ int step_storage(int vel, int force, bool efield, bool in_window, const void* P,
     do {                                                                                                      \
         bool staged;                                                                                          \
         if constexpr (GROUP == 2)                                                                             \
-            staged = launch_rows_rs<L, S, F, EFV, W, 0, true>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,    \
-                                                              slots, slot_blocks, p, s);                      \
+            staged = launch_rows_any<L, S, F, EFV, W, true>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,      \
+                                                            slots, slot_blocks, p, s);                        \
         else                                                                                                  \
             staged = launch_rows<L, S, F, EFV, W>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots,         \
                                                   slot_blocks, p, s);                                         \

@@ -295,23 +295,24 @@ void ws_release(lbm_ctx* c) {
 
 // Units (see pop_slot).  A row stays whole while its rows of all directions,
 // twice staged and once as outputs, fit kRowSmem: three or more blocks then
-// share an SM.  A longer row is cut into equal segments of at most kMaxSegment
-// columns.  As whole rows, D2V9 FP32 rows of 1024 cells kept one block of eight
+// share an SM.  A longer row is cut into segments: the usual ones
+// (usual_segment) where they fit and pad the row by no more than an eighth,
+// what a compile-time stride gains; else equal ones of that many columns at
+// most.  As whole rows, D2V9 FP32 rows of 1024 cells kept one block of eight
 // warps per SM: 27.6 us per step at 1024^2, and no reverse step but the general
 // one (95 us).
-constexpr int kMaxSegment = 256;
-
 void set_units(lbm_ctx* c) {
     const int nx = (int)c->nx;
     c->nseg = 1;
     c->seglen = nx;
     if (nx >= lbm::kMinStagedRow) {
-        const int up = lbm::kPitch;
+        const int up = lbm::kPitch, usual = lbm::usual_segment(c->Q);
         const int cols = std::min(lbm::kRowSmem / (int)(3 * c->Q * pop_elem_bytes(c->storage)), lbm::kMaxUnit);
-        const int most = std::max(up, std::min(c->Q <= 9 ? 2 * kMaxSegment : kMaxSegment, cols / up * up));
+        const int most = std::max(up, std::min(usual, cols / up * up));
         auto padded = [&](int n) { return (n + up - 1) / up * up; };
         if (padded(nx) > cols) c->nseg = (nx + most - 1) / most;
         c->seglen = padded((nx + c->nseg - 1) / c->nseg);
+        if (c->nseg > 1 && most == usual && 8 * (int64_t)c->nseg * usual <= 9 * (int64_t)nx) c->seglen = usual;
         c->nseg = (nx + c->seglen - 1) / c->seglen;
     }
     c->nxp = (int64_t)c->nseg * c->seglen;

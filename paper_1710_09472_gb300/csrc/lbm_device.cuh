@@ -218,14 +218,13 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 // A unit of the row-staged kernels: its row, segment, first column x0 and cells.
-// RS: whole rows of that many cells.
 struct UnitAt {
     int row, seg, x0, len;
 };
-template <int RS>
+template <int RS, int MODE>
 __device__ __forceinline__ UnitAt unit_at(const KParams& p, int unit) {
-    UnitAt u{unit, 0, 0, RS ? RS : p.nx};
-    if (!RS && p.nseg > 1) {
+    UnitAt u{unit, 0, 0, RS && MODE == kExactRow ? RS : p.nx};
+    if (MODE == kSegment) {
         u.row = unit / p.nseg;
         u.seg = unit - u.row * p.nseg;
         u.x0 = u.seg * p.seglen;
@@ -239,7 +238,7 @@ __device__ __forceinline__ UnitAt unit_at(const KParams& p, int unit) {
 // PULL: the rows (y - e_ay, z - e_az), read at x - e_ax; else the gather rows
 // (y + e_ay, z + e_az), read at x + e_ax.  The slots of the directions with one
 // (e_y, e_z) are consecutive: one copy per neighbouring row.
-template <class L, int RS, bool PULL, class T>
+template <class L, int RS, int MODE, bool PULL, class T>
 __device__ __forceinline__ void stage_rows(T* rows, const T* __restrict__ F, const UnitAt& u, uint64_t* bar,
                                            const KParams& p) {
     const int y = u.row % p.ny, z = u.row / p.ny;
@@ -253,7 +252,7 @@ __device__ __forceinline__ void stage_rows(T* rows, const T* __restrict__ F, con
         const int ey = PULL ? k / 3 - 1 : 1 - k / 3, ez = PULL ? k % 3 - 1 : 1 - k % 3, s0 = key_first<L>(k);
         const int ys = ey > 0 ? ym : (ey < 0 ? yp : y);
         const int zs = ez > 0 ? zm : (ez < 0 ? zp : z);
-        const int su = RS ? zs * p.ny + ys : (zs * p.ny + ys) * p.nseg + u.seg;
+        const int su = MODE != kSegment ? zs * p.ny + ys : (zs * p.ny + ys) * p.nseg + u.seg;
         bulk_load(rows + s0 * rs, F + ((int64_t)su * L::Q + s0) * rs,
                   (uint32_t)(key_count<L>(k) * rs) * (uint32_t)sizeof(T), bar);
     }

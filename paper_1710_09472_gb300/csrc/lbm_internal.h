@@ -276,6 +276,15 @@ template <class L, class S>
 __host__ __device__ constexpr bool whole_row(int nx) {
     return 3 * L::Q * nx * S::kBytes <= kRowSmem;
 }
+// What a staged kernel is compiled for: rows of exactly the compile-time stride,
+// rows, or segments.
+enum UnitMode { kExactRow, kWholeRow, kSegment };
+// The usual segment, for which the kernels have compile-time strides.
+__host__ __device__ constexpr int usual_segment(int Q) { return Q <= 9 ? 512 : 256; }
+template <class L>
+__host__ __device__ constexpr int segment_columns() {
+    return usual_segment(L::Q);
+}
 
 struct KParams {
     int nx, ny, nz;
@@ -412,6 +421,8 @@ int launch_reduce_partials(const double* partials, int64_t n_partials, double* o
 int launch_populations(int vel, int storage, const void* pop, const uint32_t* nbr, float* f, bool deviation,
                        const KParams& p, cudaStream_t s);
 int64_t moments_partial_count(const KParams& p);
+// SMs of the current device, asked once per device (1 where it cannot be told).
+int sm_count();
 
 // Adjoint (lbm_adjoint.cu).
 int64_t adjoint_slot_count(const KParams& p);

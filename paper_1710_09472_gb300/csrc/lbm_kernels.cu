@@ -14,6 +14,7 @@
 // rowG[u] .. rowG[u+1] (u a row, or a segment of a long row).  The collision stores f*_b(x) there, and the next
 // step reads it back as f_bbar(x).
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 
 #include <cub/device/device_scan.cuh>
@@ -267,21 +268,21 @@ __global__ void __launch_bounds__(kBlock) k_moments(const typename S::T* __restr
 // and cell order; no outputs to stage, so one barrier per unit and twice the
 // blocks per SM).  The general kernel spends 370 instructions a cell on
 // addresses and links: 0.24 ms on 256^3 porous D3V19 FP16, 0.135 of it floor.
-template <class L, class S, bool TOTALS>
+template <class L, class S, bool TOTALS, int MODE>
 __global__ void __launch_bounds__(256) k_moments_rows(const typename S::T* __restrict__ P, float* __restrict__ rho_out,
                                                       float* __restrict__ j_out, double* __restrict__ partials,
                                                       int gcap, int dcap, KParams p) {
     using T = typename S::T;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int rs = p.seglen, U = p.ny * p.nz * p.nseg, G = gridDim.x;
-    const bool halo = p.nseg > 1;
+    constexpr bool halo = MODE == kSegment;
     const stepk::StageLayout<L, S> lay{rs, p.lorder, gcap, dcap, dev::halo_bytes(L::Q, p.nseg, S::kBytes)};
     const int sbytes = lay.bytes();
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t gstart[2], dstart[2];
     const bool issuer = (int)threadIdx.x == (int)blockDim.x - 32;
     auto stage = [&](int k, int unit) {
-        stepk::stage_unit<L, S, 0>(smem_raw + k * sbytes, lay, &bar[k], P, unit, __ldg(p.rowG + unit),
+        stepk::stage_unit<L, S, 0, MODE>(smem_raw + k * sbytes, lay, &bar[k], P, unit, __ldg(p.rowG + unit),
                                    __ldg(p.rowG + unit + 1), &gstart[k], &dstart[k], p);
     };
     if (threadIdx.x == 0) {
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(256) k_moments_rows(const typename S::T* __res
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (halo && dev::halo_thread<L>())
-        dev::halo_put<L, true>(lay.halo(smem_raw), dev::halo_fetch<L, true>(P, dev::unit_at<0>(p, blockIdx.x), p));
+        dev::halo_put<L, true>(lay.halo(smem_raw), dev::halo_fetch<L, true>(P, dev::unit_at<0, MODE>(p, blockIdx.x), p));
     __syncthreads();
     if (issuer && (int)blockIdx.x < U) stage(0, blockIdx.x);
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(256) k_moments_rows(const typename S::T* __res
             dev::pause_cycles(1ll << 22);  // let this block's copies in flight land
         }
         T* buf = lay.rows(st);
-        dev::patch_links<true, true>(buf, rs, lay.halo(st), L::Q, lay.links(st), gstart[cs], g0, g1, lay.descs(st),
+        dev::patch_links<true, halo>(buf, rs, lay.halo(st), L::Q, lay.links(st), gstart[cs], g0, g1, lay.descs(st),
                                      dstart[cs]);
         dev::fence_proxy_async();  // this stage is overwritten by copies after the next barrier
         // bounced values in place; every thread is past its reads of the other stage
@@ -314,10 +315,10 @@ __global__ void __launch_bounds__(256) k_moments_rows(const typename S::T* __res
         if (issuer && ok && un < U) stage(cs ^ 1, un);
         const bool fetch = halo && un < U && dev::halo_thread<L>();
         T hv{};
-        if (fetch) hv = dev::halo_fetch<L, true>(P, dev::unit_at<0>(p, un), p);
+        if (fetch) hv = dev::halo_fetch<L, true>(P, dev::unit_at<0, MODE>(p, un), p);
         const uint16_t* ord = lay.order(st);
         const int nf = ord[0];
-        const dev::UnitAt at = dev::unit_at<0>(p, u);
+        const dev::UnitAt at = dev::unit_at<0, MODE>(p, u);
         const int64_t first = (int64_t)at.row * p.nx + at.x0;
         for (int i = threadIdx.x; i < at.len; i += blockDim.x) {
             const int x = (int)ord[8 + i];
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(256) k_moments_rows(const typename S::T* __res
 #pragma unroll
                 for (int a = 0; a < L::Q; ++a) {
                     const int ex = L::c(a, 0), s = pop_slot<L>(a);
-                    h[a] = S::cvt(ex > 0 ? bm[s * rm] : (ex < 0 ? bp[s * rp] : buf[s * rs + x]));
+                    h[a] = S::cvt(ex > 0 ? bm[s * (halo ? rm : rs)] : (ex < 0 ? bp[s * (halo ? rp : rs)] : buf[s * rs + x]));
                 }
                 cell_moments<L>(h, p, r, j);
                 if (TOTALS) {
@@ -388,7 +389,7 @@ int64_t launch_moments_rows(const void* pop, float* rho, float* j, double* parti
     const size_t smem = 2 * ((size_t)L::Q * p.seglen * S::kBytes + 2 * (size_t)p.lorder + gcap + dcap +
                              dev::halo_bytes(L::Q, p.nseg, S::kBytes));
     if (smem > stepk::kSmemBudget) return 0;
-    auto kern = k_moments_rows<L, S, TOTALS>;
+    auto kern = p.nseg > 1 ? k_moments_rows<L, S, TOTALS, kSegment> : k_moments_rows<L, S, TOTALS, kWholeRow>;
     const stepk::Shape sh = stepk::launch_shape(kern, p.seglen, smem);
     const int units = p.ny * p.nz * p.nseg;
     if (sh.blocks <= 0 || units < sh.sms) return 0;
@@ -486,6 +487,18 @@ int dispatch_storage(int storage, F&& f) {
 }
 
 }  // namespace
+
+int sm_count() {
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kDevices) sms = known[dev].load();
+    if (sms > 0) return sms;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(sms, 1);
+    if (dev >= 0 && dev < kDevices) known[dev].store(sms);
+    return sms;
+}
 
 int64_t moments_partial_count(const KParams& p) {
     Launch l = grid_of(p);
@@ -625,12 +638,7 @@ int launch_moments(int vel, int storage, const void* pop, const uint32_t* nbr, f
     const int chunks = (int)l.grid.y;
     const int64_t tiles = (int64_t)l.grid.x * chunks;
     int64_t blocks = tiles;
-    if (partials) {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        blocks = std::min<int64_t>(tiles, (int64_t)std::max(sms, 1) * kTotalsPerSm);
-    }
+    if (partials) blocks = std::min<int64_t>(tiles, (int64_t)sm_count() * kTotalsPerSm);
     return dispatch_lattice(vel, [&](auto lat) {
         using L = decltype(lat);
         return dispatch_storage(storage, [&](auto st) {

@@ -5,6 +5,7 @@
 #pragma once
 
 #include <mutex>
+#include <type_traits>
 
 #include "lbm_device.cuh"
 
@@ -526,7 +527,7 @@ struct StageLayout {
 // (dev::stage_rows), the cell order, the link window and the descriptor
 // window.  The window starts are written before the barrier is armed, so the
 // arrive releases them to the waiting threads.
-template <class L, class S, int RS>
+template <class L, class S, int RS, int MODE>
 __device__ __forceinline__ void stage_unit(unsigned char* st, const StageLayout<L, S>& lay, uint64_t* bar,
                                            const typename S::T* __restrict__ Pin, int unit, uint32_t g0, uint32_t g1,
                                            uint32_t* gstart, uint32_t* dstart, const KParams& p) {
@@ -537,7 +538,7 @@ __device__ __forceinline__ void stage_unit(unsigned char* st, const StageLayout<
     *dstart = (uint32_t)(db0 / 4);
     dev::mbar_expect_tx(bar, (uint32_t)lay.rows_bytes() + 2u * (uint32_t)lay.lorder + (uint32_t)(gb1 - gb0) +
                                  (uint32_t)(db1 - db0));
-    dev::stage_rows<L, RS, true>(lay.rows(st), Pin, dev::unit_at<RS>(p, unit), bar, p);
+    dev::stage_rows<L, RS, MODE, true>(lay.rows(st), Pin, dev::unit_at<RS, MODE>(p, unit), bar, p);
     dev::bulk_load(lay.order(st), p.rorder + (int64_t)unit * lay.lorder, 2u * (uint32_t)lay.lorder, bar);
     if (gb1 > gb0)
         dev::bulk_load(lay.links(st), reinterpret_cast<const unsigned char*>(Pin) + p.gofs + gb0,
@@ -555,28 +556,30 @@ __device__ __forceinline__ void stage_unit(unsigned char* st, const StageLayout<
 // thread has passed its link copies (the first barrier of the next unit).  For
 // FP16 the extra barrier and the 256-thread blocks cost more than the freed
 // memory gains (0.321 against 0.258 ms), so 16-bit storage keeps output rows.
-template <class S, int RS, bool LMU>
-constexpr bool kInPlaceOut = S::kBytes == 4 && RS == 256 && !LMU;
+template <class S, int RS, int MODE, bool LMU>
+constexpr bool kInPlaceOut = S::kBytes == 4 && RS == 256 && MODE == kExactRow && !LMU;
 
-template <class L, class S, int FORCE, bool EF, bool SR, int STAGES, int RS, bool LMU = false>
+template <class L, class S, int FORCE, bool EF, bool SR, int STAGES, int RS, int MODE, bool LMU = false>
 __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restrict__ Pin,
                                                    typename S::T* __restrict__ Pout, const float* __restrict__ Ef,
                                                    int gcap, int dcap, KParams p) {
     using T = typename S::T;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    // RS: whole rows of that many cells, a compile-time stride; 0: a run-time one, whole rows or segments
+    // RS: units of that many columns (a compile-time stride; 0: a run-time one).
+    // MODE: rows of exactly RS cells (kExactRow), rows (kWholeRow) or segments
+    constexpr bool kOne = MODE != kSegment, kExact = RS && MODE == kExactRow;
     const int rs = RS ? RS : p.seglen;
-    const bool halo = !RS && p.nseg > 1;
+    const bool halo = !kOne;
     // FP32 rows of 256 cells write their outputs over the row's own stage
     // (no output rows: four blocks per SM instead of three); see kInPlaceOut
-    constexpr bool kInPlace = kInPlaceOut<S, RS, LMU>;
-    const StageLayout<L, S> lay{rs, p.lorder, gcap, dcap, RS ? 0 : dev::halo_bytes(L::Q, p.nseg, S::kBytes)};
+    constexpr bool kInPlace = kInPlaceOut<S, RS, MODE, LMU>;
+    const StageLayout<L, S> lay{rs, p.lorder, gcap, dcap, kOne ? 0 : dev::halo_bytes(L::Q, p.nseg, S::kBytes)};
     const int sbytes = lay.bytes();
     T* outrow = reinterpret_cast<T*>(smem_raw + STAGES * sbytes);
     __shared__ __align__(8) uint64_t bar[STAGES];
     __shared__ uint32_t gstart[STAGES], dstart[STAGES];
     T* Gout = reinterpret_cast<T*>(reinterpret_cast<char*>(Pout) + p.gofs);
-    const int U = p.ny * p.nz * (RS ? 1 : p.nseg);
+    const int U = p.ny * p.nz * (kOne ? 1 : p.nseg);
     const int G = gridDim.x;
     const bool leader = threadIdx.x == 0;
     const bool issuer = (int)threadIdx.x == (int)blockDim.x - 32;  // lane 0 of the last warp
@@ -595,7 +598,7 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
     static_assert(STAGES == 2, "the halo values are fetched one unit ahead");
     if (halo && dev::halo_thread<L>())
         dev::halo_put<L, true>(lay.halo(smem_raw),
-                               dev::halo_fetch<L, true>(Pin, dev::unit_at<RS>(p, blockIdx.x), p));
+                               dev::halo_fetch<L, true>(Pin, dev::unit_at<RS, MODE>(p, blockIdx.x), p));
     __syncthreads();
     if (issuer) {
 #pragma unroll
@@ -604,7 +607,7 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
             if (uk < U) {
                 uint32_t g0, g1;
                 range(uk, g0, g1);
-                stage_unit<L, S, RS>(smem_raw + k * sbytes, lay, &bar[k], Pin, uk, g0, g1, &gstart[k], &dstart[k], p);
+                stage_unit<L, S, RS, MODE>(smem_raw + k * sbytes, lay, &bar[k], Pin, uk, g0, g1, &gstart[k], &dstart[k], p);
             }
         }
     }
@@ -627,7 +630,7 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
         const uint16_t* ord = lay.order(st);
         const uint32_t* desc = lay.descs(st);
         const uint32_t d0 = dstart[cs];
-        dev::patch_links<true, RS == 0>(buf, rs, lay.halo(st), L::Q, lay.links(st), gstart[cs], g0, g1, desc, d0);
+        dev::patch_links<true, !kOne>(buf, rs, lay.halo(st), L::Q, lay.links(st), gstart[cs], g0, g1, desc, d0);
         dev::bulk_wait_read();  // this thread's bulk stores of the previous unit have read the output rows
         // bounced values in place, output rows free; a timeout anywhere in
         // the block stops the copies
@@ -638,17 +641,17 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
             // its wait on that stage's barrier
             uint32_t n0, n1;
             range(un, n0, n1);
-            stage_unit<L, S, RS>(smem_raw + sn * sbytes, lay, &bar[sn], Pin, un, n0, n1, &gstart[sn], &dstart[sn], p);
+            stage_unit<L, S, RS, MODE>(smem_raw + sn * sbytes, lay, &bar[sn], Pin, un, n0, n1, &gstart[sn], &dstart[sn], p);
         }
         const bool fetch = halo && un < U && dev::halo_thread<L>();
         T hv{};
-        if (fetch) hv = dev::halo_fetch<L, true>(Pin, dev::unit_at<RS>(p, un), p);
+        if (fetch) hv = dev::halo_fetch<L, true>(Pin, dev::unit_at<RS, MODE>(p, un), p);
         const int nf = ord[0];
-        const dev::UnitAt at = dev::unit_at<RS>(p, u);
+        const dev::UnitAt at = dev::unit_at<RS, MODE>(p, u);
         const int nx = at.len;  // cells of the unit
-        const uint32_t rowbase = (uint32_t)at.row * (uint32_t)(RS ? RS : p.nx) + (uint32_t)at.x0;  // first cell
+        const uint32_t rowbase = (uint32_t)at.row * (uint32_t)(kExact ? RS : p.nx) + (uint32_t)at.x0;  // first cell
         if constexpr (kInPlace) {
-            // one cell per thread (the launcher sets blockDim.x = nx): every
+            // one cell per thread (the launcher sets blockDim.x = RS): every
             // pull first, then a barrier, then the outputs over the stage
             const int i = threadIdx.x;
             const int x = (int)ord[8 + i];
@@ -667,7 +670,7 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
             __syncthreads();  // no thread overwrites a slot another has still to pull
             if (fluid) {
                 float E[3];
-                load_E<L>(Ef, EF, p, (int64_t)at.row * (RS ? RS : p.nxp) + (at.x0 + x), E);
+                load_E<L>(Ef, EF, p, (int64_t)u * rs + x, E);
                 float out[L::Q];
                 collide_any<L, S, FORCE, LMU>(h, E, p, out);
                 typename S::T t[L::Q];
@@ -700,10 +703,10 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
 #pragma unroll
                 for (int a = 0; a < L::Q; ++a) {
                     const int ex = L::c(a, 0), s = pop_slot<L>(a);
-                    h[a] = S::cvt(ex > 0 ? bm[s * (RS ? RS : rm)] : (ex < 0 ? bp[s * (RS ? RS : rp)] : buf[s * rs + x]));
+                    h[a] = S::cvt(ex > 0 ? bm[s * (kOne ? rs : rm)] : (ex < 0 ? bp[s * (kOne ? rs : rp)] : buf[s * rs + x]));
                 }
                 float E[3];
-                load_E<L>(Ef, EF, p, (int64_t)at.row * (RS ? RS : p.nxp) + (at.x0 + x), E);
+                load_E<L>(Ef, EF, p, (int64_t)u * rs + x, E);
                 if (S::kBytes == 4) {
                     // FP32 storage: compensated collision
                     float out[L::Q];
@@ -815,22 +818,23 @@ Shape launch_shape(K kernel, int nx, size_t smem, int fixed_threads = 0) {
     return last;
 }
 
-template <class L, class S, int FORCE, bool EF, bool SR, int RS, bool LMU = false>
+template <class L, class S, int FORCE, bool EF, bool SR, int RS, int MODE, bool LMU = false>
 bool launch_rows(const S*, const void* fin, void* fout, const uint32_t* nbr, const float* Ef, const KParams& p,
                  cudaStream_t s) {
     using T = typename S::T;
-    if (!p.rorder || (RS && (RS != p.nx || p.nseg != 1))) return false;
+    if (!p.rorder || (RS && RS != p.seglen) || (MODE == kExactRow && RS != p.nx) || (MODE == kSegment) != (p.nseg > 1))
+        return false;
     const size_t srow = (size_t)p.seglen * S::kBytes;
     const int gcap = dev::window_cap(p.max_row_links, S::kBytes);
     const int dcap = dev::window_cap(p.max_row_links, 4);
     const size_t stage_bytes = (size_t)L::Q * srow + 2 * (size_t)p.lorder + gcap + dcap +
                                dev::halo_bytes(L::Q, p.nseg, S::kBytes);
-    constexpr bool kInPlace = kInPlaceOut<S, RS, LMU>;
+    constexpr bool kInPlace = kInPlaceOut<S, RS, MODE, LMU>;
     const size_t smem = (size_t)kStages * stage_bytes + (kInPlace ? 0 : (size_t)L::Q * srow);
     if (smem > kSmemBudget) return false;
-    auto kern = k_step_rows<L, S, FORCE, EF, SR, kStages, RS, LMU>;
-    // one cell per thread in place: exactly nx (= 256) threads
-    const Shape sh = launch_shape(kern, p.seglen, smem, kInPlace ? p.nx : 0);
+    auto kern = k_step_rows<L, S, FORCE, EF, SR, kStages, RS, MODE, LMU>;
+    // one cell per thread in place: exactly 256 threads
+    const Shape sh = launch_shape(kern, p.seglen, smem, kInPlace ? RS : 0);
     const int threads = sh.threads, blocks = sh.blocks;
     if (blocks <= 0) return false;
     const int units = p.ny * p.nz * p.nseg;
@@ -843,29 +847,68 @@ bool launch_rows(const S*, const void* fin, void* fout, const uint32_t* nbr, con
     return true;
 }
 
-// Row-staged kernel when the rows qualify, with the shared-memory row stride
-// (the row length) a compile-time constant for rows of 256 or 512 cells (the
-// indexing then folds into immediate offsets); otherwise the general kernel.
+// Row-staged kernel when the rows qualify, with the shared-memory row stride a
+// compile-time constant for the usual units (the indexing then folds into
+// immediate offsets); otherwise the general kernel.
 template <class L, class S, int FORCE, bool EF, bool SR>
 int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef, const KParams& p, cudaStream_t s) {
     using T = typename S::T;
     const S* tag = nullptr;
-    bool done;
-    // the compile-time strides for the benchmarked lattices (D2V9, D3V19, and 256
-    // for 16-bit D3V27); the others take the run-time stride (fewer
-    // instantiations to compile)
+    // Compile-time strides: rows of 256 and 512 cells of the benchmarked lattices
+    // (D2V9, D3V19), their usual segments, 256 for 16-bit D3V27, and for D3V19 rows
+    // padded to 256.  A run-time stride costs a fifth of the step (256^3 D3V27
+    // FP16, 10 steps and the fields: 4.33 against 3.63 ms); other widths take it, to
+    // keep the instantiations few.  Rows and segments are compiled apart: the
+    // halo of segments costs whole rows another tenth (250 x 128 x 128 D3V19 FP16,
+    // 20 steps and the fields: 1.52 against 1.40 ms).
+    auto rows = [&](auto rs, auto mode, auto lmu) {
+        return launch_rows<L, S, FORCE, EF, SR, decltype(rs)::value, decltype(mode)::value, decltype(lmu)::value>(
+            tag, fin, fout, nbr, Ef, p, s);
+    };
     constexpr bool kFixed = L::Q == 9 || L::Q == 19;
     constexpr bool kFixed256 = kFixed || (L::Q == 27 && whole_row<L, S>(256));
-    if (p.lmu_tab)  // the local-mu model (D2V9, D3V19 only)
-        done = kFixed && (p.nx == 256 && p.nseg == 1
-                              ? launch_rows<L, S, FORCE, EF, SR, kFixed ? 256 : 0, kFixed>(tag, fin, fout, nbr, Ef, p, s)
-                              : launch_rows<L, S, FORCE, EF, SR, 0, kFixed>(tag, fin, fout, nbr, Ef, p, s));
-    else if (kFixed256 && p.nx == 256 && p.nseg == 1)
-        done = launch_rows<L, S, FORCE, EF, SR, kFixed256 ? 256 : 0>(tag, fin, fout, nbr, Ef, p, s);
-    else if (kFixed && p.nx == 512 && p.nseg == 1)
-        done = launch_rows<L, S, FORCE, EF, SR, kFixed && whole_row<L, S>(512) ? 512 : 0>(tag, fin, fout, nbr, Ef, p, s);
-    else
-        done = launch_rows<L, S, FORCE, EF, SR, 0>(tag, fin, fout, nbr, Ef, p, s);
+    constexpr bool kFixed512 = kFixed && whole_row<L, S>(512);
+    constexpr int kSeg = segment_columns<L>();
+    using R0 = std::integral_constant<int, 0>;
+    using R256 = std::integral_constant<int, 256>;
+    using R512 = std::integral_constant<int, 512>;
+    using RSeg = std::integral_constant<int, kSeg>;
+    using Exact = std::integral_constant<int, kExactRow>;
+    using Whole = std::integral_constant<int, kWholeRow>;
+    using Segment = std::integral_constant<int, kSegment>;
+    const std::true_type local{};
+    const std::false_type plain{};
+    bool done = false, tried = false;
+    if constexpr (kFixed) {
+        if (p.lmu_tab) {  // the local-mu model (D2V9, D3V19 only)
+            tried = true;
+            done = p.nseg > 1     ? rows(R0{}, Segment{}, local)
+                   : p.nx == 256 ? rows(R256{}, Exact{}, local)
+                                 : rows(R0{}, Whole{}, local);
+        } else if (p.nseg > 1 && p.seglen == kSeg) {
+            tried = true;
+            done = rows(RSeg{}, Segment{}, plain);
+        }
+    }
+    if constexpr (kFixed256) {
+        if (!tried && p.nx == 256 && p.nseg == 1) {
+            tried = true;
+            done = rows(R256{}, Exact{}, plain);
+        }
+    }
+    if constexpr (kFixed512) {
+        if (!tried && p.nx == 512 && p.nseg == 1) {
+            tried = true;
+            done = rows(R512{}, Exact{}, plain);
+        }
+    }
+    if constexpr (L::Q == 19) {
+        if (!tried && p.seglen == 256 && p.nseg == 1) {
+            tried = true;
+            done = rows(R256{}, Whole{}, plain);
+        }
+    }
+    if (!tried) done = p.nseg > 1 ? rows(R0{}, Segment{}, plain) : rows(R0{}, Whole{}, plain);
     if (done) return 1;
     const int bx = p.nx >= kBlock ? kBlock : ((p.nx + 31) / 32) * 32;
     const dim3 grid((unsigned)(p.ny * p.nz), (unsigned)((p.nx + bx - 1) / bx));

@@ -725,13 +725,6 @@ bool is_dev(const void* ptr) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-int sm_count() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return std::max(sms, 1);
-}
-
 unsigned tgrid(int64_t nx) { return (unsigned)((nx + kTBlock - 1) / kTBlock); }
 
 }  // namespace
@@ -896,7 +889,7 @@ lbm_status lbm_thermal_init(lbm_thermal* t, const float* rho, const float* u, co
 lbm_status lbm_thermal_step(lbm_thermal* t, int64_t n) {
     if (!t || n < 0) return LBM_ERR_INVALID_ARG;
     if (!t->has_state) return tfail(t, LBM_ERR_STATE, "lbm_thermal_step before lbm_thermal_init");
-    const int sms = sm_count();
+    const int sms = lbm::sm_count();
     for (int64_t s = 0; s < n; ++s) {
         const TParams p = tparams(t);
         const bool sr = t->stochastic;
@@ -930,7 +923,7 @@ lbm_status lbm_thermal_moments(lbm_thermal* t, float* rho, float* j, float* ener
     const TParams p = tparams(t);
     unsigned blocks = tgrid(t->nx);
     if (totals) {
-        blocks = std::min(blocks, (unsigned)sm_count() * 8u);
+        blocks = std::min(blocks, (unsigned)lbm::sm_count() * 8u);
     }
     t->launches += by_storage_q(t->storage, t->Q, [&](auto st, auto q) {
         using S = decltype(st);
