@@ -176,9 +176,9 @@ lbm_status lbm_set_params(lbm_ctx* ctx, double tau, const double E[3], const dou
  * range the end value is used), built on the device when the model is
  * enabled (FD weight; with the MB weight thetabar does not depend on mu and
  * the model equals the default one).  Its steps run on the row-staged
- * kernel (an instantiation with a run-time row stride) where the rows
- * qualify, else on the general kernel.  lbm_init_equilibrium keeps the
- * default EDF; the local thetabar enters from the first collision.
+ * kernel where the rows qualify, else on the general kernel.
+ * lbm_init_equilibrium keeps the default EDF; the local thetabar enters from
+ * the first collision.
  * lbm_adjoint differentiates the model too: its reverse step adds the
  * density derivative of the local terms (thetabar'(rho) from the same table).
  * Errors: INVALID_ARG (D3V27, D1V3 or the BE weight: not built), OOM, CUDA. */
@@ -295,9 +295,9 @@ lbm_status lbm_adjoint(lbm_ctx* ctx, const float* w_rho, const float* w_j, int64
  * Host only; needs no device.  Errors: INVALID_ARG. */
 lbm_status lbm_weight_integrals(int D, int stat, double theta, double mu, double I[5]);
 
-/* Serialise / restore the state (raw stored populations, in the library's
- * internal layout, plus a header with lattice, dims, storage, step count and a
- * checksum) to / from host memory.
+/* Serialise / restore the state (the stored populations row by row, the
+ * directions of a row in the library's slot order, plus a header with lattice,
+ * dims, storage, step count and a checksum) to / from host memory.
  * lbm_save_state with host_buf == NULL only reports the size in *used.
  * lbm_load_state checks the header against the context.
  * Errors: INVALID_ARG (short buffer, header mismatch, bad checksum), CUDA. */

@@ -299,8 +299,8 @@ void ws_release(lbm_ctx* c) {
 // (usual_segment) where they fit and pad the row by no more than an eighth,
 // what a compile-time stride gains; else equal ones of that many columns at
 // most.  As whole rows, D2V9 FP32 rows of 1024 cells kept one block of eight
-// warps per SM: 27.6 us per step at 1024^2, and no reverse step but the general
-// one (95 us).
+// warps per SM: 27.6 us per step at 1024^2 (20.9 in segments), and no reverse
+// step but the general one (95 us; 38).
 void set_units(lbm_ctx* c) {
     const int nx = (int)c->nx;
     c->nseg = 1;

@@ -96,10 +96,9 @@ __device__ __forceinline__ double warp_sum(double v) {
 // The two cases differ in the address only, which is selected: one load per
 // direction, all of them in flight together.  With a branch around each load
 // they were issued one after another, and the kernels that pull this way
-// waited on them (long scoreboard 17 of 21 stalled cycles per issue): a run of
-// the general step on 250 x 128 x 128 porous D3V19 FP16 took 4.21 ms (20 steps
-// and the moments) against 3.44 ms now, 4 steps and the moments of a staged
-// 512^3 box 11.31 against 9.62 ms.  A cell's link slots follow its outgoing directions in
+// waited on them (long scoreboard 17 of 21 stalled cycles per issue): 20 general
+// steps and the fields of 250 x 128 x 128 porous D3V19 FP16 took 4.21 ms
+// against 3.44 with the selection.  A cell's link slots follow its outgoing directions in
 // ascending order, so a running count replaces a popcount per direction.
 template <class L, class S>
 __device__ __forceinline__ void pull(const typename S::T* __restrict__ P, const KParams& p, uint32_t m, const Cell& c,

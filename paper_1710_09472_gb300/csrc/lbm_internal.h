@@ -402,19 +402,12 @@ int launch_step(int vel, int storage, int force, bool efield, bool sr, const voi
 // fout, or in fin where *in_fin says so; the other buffer is overwritten.
 int launch_multi(int vel, int storage, int force, bool sr, void* fin, void* fout, const uint32_t* nbr, const float* Ef,
                  int n, unsigned* count, bool* in_fin, const KParams& p, cudaStream_t s);
-int launch_step_f32(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
-                    const float* Ef, const KParams& p, cudaStream_t s);
-int launch_step_f16(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
-                    const float* Ef, const KParams& p, cudaStream_t s);
-int launch_step_bf16(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
-                     const float* Ef, const KParams& p, cudaStream_t s);
-// the same for D3V27 and D1V3 (translation units lbm_step_*_x.cu)
-int launch_step_f32_x(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
-                      const float* Ef, const KParams& p, cudaStream_t s);
-int launch_step_f16_x(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
-                      const float* Ef, const KParams& p, cudaStream_t s);
-int launch_step_bf16_x(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
-                       const float* Ef, const KParams& p, cudaStream_t s);
+// one per storage, lattice group (_x: D3V27 and D1V3) and rounding (_n: nearest
+// rounding of the 16-bit storages); translation units lbm_step_*.cu
+using StepLauncher = int(int vel, int force, bool efield, const void* fin, void* fout, const uint32_t* nbr,
+                         const float* Ef, const KParams& p, cudaStream_t s);
+StepLauncher launch_step_f32, launch_step_f32_x, launch_step_f16, launch_step_f16_n, launch_step_f16_x,
+    launch_step_f16_x_n, launch_step_bf16, launch_step_bf16_n, launch_step_bf16_x, launch_step_bf16_x_n;
 int launch_moments(int vel, int storage, const void* pop, const uint32_t* nbr, float* rho, float* j,
                    double* partials, int64_t* n_partials, const KParams& p, cudaStream_t s);
 int launch_reduce_partials(const double* partials, int64_t n_partials, double* out4, cudaStream_t s);

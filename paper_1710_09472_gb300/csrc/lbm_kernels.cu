@@ -267,7 +267,8 @@ __global__ void __launch_bounds__(kBlock) k_moments(const typename S::T* __restr
 // The same over units staged in shared memory (the step kernel's stages, links
 // and cell order; no outputs to stage, so one barrier per unit and twice the
 // blocks per SM).  The general kernel spends 370 instructions a cell on
-// addresses and links: 0.24 ms on 256^3 porous D3V19 FP16, 0.135 of it floor.
+// addresses and links: 0.24 ms on 256^3 porous D3V19 FP16 (0.135 the floor),
+// against 0.15 staged.
 template <class L, class S, bool TOTALS, int MODE>
 __global__ void __launch_bounds__(256) k_moments_rows(const typename S::T* __restrict__ P, float* __restrict__ rho_out,
                                                       float* __restrict__ j_out, double* __restrict__ partials,
@@ -599,14 +600,15 @@ int launch_init(int vel, int storage, void* pop, const uint32_t* nbr, const floa
 
 int launch_step(int vel, int storage, int force, bool efield, bool sr, const void* fin, void* fout,
                 const uint32_t* nbr, const float* Ef, const KParams& p, cudaStream_t s) {
-    if (vel == LBM_D3V27 || vel == LBM_D1V3) {
-        if (storage == LBM_F16_DEV) return launch_step_f16_x(vel, force, efield, sr, fin, fout, nbr, Ef, p, s);
-        if (storage == LBM_BF16_DEV) return launch_step_bf16_x(vel, force, efield, sr, fin, fout, nbr, Ef, p, s);
-        return launch_step_f32_x(vel, force, efield, false, fin, fout, nbr, Ef, p, s);
-    }
-    if (storage == LBM_F16_DEV) return launch_step_f16(vel, force, efield, sr, fin, fout, nbr, Ef, p, s);
-    if (storage == LBM_BF16_DEV) return launch_step_bf16(vel, force, efield, sr, fin, fout, nbr, Ef, p, s);
-    return launch_step_f32(vel, force, efield, false, fin, fout, nbr, Ef, p, s);
+    const bool x = vel == LBM_D3V27 || vel == LBM_D1V3;
+    StepLauncher* f;
+    if (storage == LBM_F16_DEV)
+        f = sr ? (x ? launch_step_f16_x : launch_step_f16) : (x ? launch_step_f16_x_n : launch_step_f16_n);
+    else if (storage == LBM_BF16_DEV)
+        f = sr ? (x ? launch_step_bf16_x : launch_step_bf16) : (x ? launch_step_bf16_x_n : launch_step_bf16_n);
+    else
+        f = x ? launch_step_f32_x : launch_step_f32;
+    return f(vel, force, efield, fin, fout, nbr, Ef, p, s);
 }
 
 // With totals the blocks stride over the tiles, kTotalsPerSm of them per SM,

@@ -274,6 +274,14 @@ Plan plan_of(const KParams& p) {
     return {blocks, (int)cpc, smem};
 }
 
+// 1 for a launch that went out; the error of one that did not is cleared, since
+// the steps are then launched one by one.
+inline int launched(cudaError_t e) {
+    if (e == cudaSuccess) return 1;
+    cudaGetLastError();
+    return 0;
+}
+
 // Launches n steps, or returns 0: a box that does not fit, or a device on which
 // the cluster cannot be placed.
 template <class L, class S, int FORCE, bool SR>
@@ -314,7 +322,7 @@ int launch_cluster(const void* fin, void* fout, const uint32_t* nbr, const float
         }
         if (!fits) return 0;
     }
-    return cudaLaunchKernelEx(&cfg, kern, (const T*)fin, (T*)fout, nbr, Ef, n, plan.cpc, p) == cudaSuccess ? 1 : 0;
+    return launched(cudaLaunchKernelEx(&cfg, kern, (const T*)fin, (T*)fout, nbr, Ef, n, plan.cpc, p));
 }
 
 // The same for the cooperative grid; the result is in fin when n is even.
@@ -351,15 +359,13 @@ int launch_grid(void* fin, void* fout, const uint32_t* nbr, const float* Ef, int
         }
         if (!fits) return 0;
     }
-    if (cudaMemsetAsync(count, 0, sizeof(unsigned), s) != cudaSuccess) return 0;
+    if (!launched(cudaMemsetAsync(count, 0, sizeof(unsigned), s))) return 0;
     T *A = (T*)fin, *B = (T*)fout;
     KParams q = p;
     void* args[] = {&A, &B, &nbr, &Ef, &n, &count, &q};
     const unsigned blocks = (unsigned)((p.N + threads - 1) / threads);
-    return cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3((unsigned)threads), args,
-                                       (size_t)(L::Q - 1) * threads * 4, s) == cudaSuccess
-               ? 1
-               : 0;
+    return launched(cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3((unsigned)threads), args,
+                                                (size_t)(L::Q - 1) * threads * 4, s));
 }
 
 template <class L, class S, int FORCE, bool SR>

@@ -858,7 +858,8 @@ int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef
     // (D2V9, D3V19), their usual segments, 256 for 16-bit D3V27, and for D3V19 rows
     // padded to 256.  A run-time stride costs a fifth of the step (256^3 D3V27
     // FP16, 10 steps and the fields: 4.33 against 3.63 ms); other widths take it, to
-    // keep the instantiations few.  Rows and segments are compiled apart: the
+    // keep the instantiations few (the nearest rounding of 16-bit storage too, but
+    // for the exact rows).  Rows and segments are compiled apart: the
     // halo of segments costs whole rows another tenth (250 x 128 x 128 D3V19 FP16,
     // 20 steps and the fields: 1.52 against 1.40 ms).
     auto rows = [&](auto rs, auto mode, auto lmu) {
@@ -866,7 +867,7 @@ int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef
             tag, fin, fout, nbr, Ef, p, s);
     };
     constexpr bool kFixed = L::Q == 9 || L::Q == 19;
-    constexpr bool kFixed256 = kFixed || (L::Q == 27 && whole_row<L, S>(256));
+    constexpr bool kFixed256 = kFixed || (L::Q == 27 && SR && whole_row<L, S>(256));
     constexpr bool kFixed512 = kFixed && whole_row<L, S>(512);
     constexpr int kSeg = segment_columns<L>();
     using R0 = std::integral_constant<int, 0>;
@@ -902,7 +903,7 @@ int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef
             done = rows(R512{}, Exact{}, plain);
         }
     }
-    if constexpr (L::Q == 19) {
+    if constexpr (L::Q == 19 && (SR || S::kBytes == 4)) {
         if (!tried && p.seglen == 256 && p.nseg == 1) {
             tried = true;
             done = rows(R256{}, Whole{}, plain);
@@ -926,25 +927,18 @@ int launch_lat(int force, bool efield, const void* fin, void* fout, const uint32
                   : launch_one<L, S, 1, false, SR>(fin, fout, nbr, Ef, p, s);
 }
 
-// GROUP 0: D2V9 and D3V19; GROUP 1: D3V27 and D1V3 (compiled in translation
-// units of their own, so that the build runs them in parallel)
-template <class S, bool HAS_SR, int GROUP>
-int launch_storage(int vel, int force, bool efield, bool sr, const void* fin, void* fout, const uint32_t* nbr,
-                   const float* Ef, const KParams& p, cudaStream_t s) {
+// GROUP 0: D2V9 and D3V19; GROUP 1: D3V27 and D1V3.  These, and stochastic and
+// nearest rounding, are compiled in translation units of their own, so that the
+// build runs them in parallel.
+template <class S, bool SR, int GROUP>
+int launch_storage(int vel, int force, bool efield, const void* fin, void* fout, const uint32_t* nbr, const float* Ef,
+                   const KParams& p, cudaStream_t s) {
     if constexpr (GROUP == 0) {
-        if (HAS_SR && sr) {
-            if (vel == LBM_D2V9) return launch_lat<LatD2V9, S, HAS_SR>(force, efield, fin, fout, nbr, Ef, p, s);
-            return launch_lat<LatD3V19, S, HAS_SR>(force, efield, fin, fout, nbr, Ef, p, s);
-        }
-        if (vel == LBM_D2V9) return launch_lat<LatD2V9, S, false>(force, efield, fin, fout, nbr, Ef, p, s);
-        return launch_lat<LatD3V19, S, false>(force, efield, fin, fout, nbr, Ef, p, s);
+        if (vel == LBM_D2V9) return launch_lat<LatD2V9, S, SR>(force, efield, fin, fout, nbr, Ef, p, s);
+        return launch_lat<LatD3V19, S, SR>(force, efield, fin, fout, nbr, Ef, p, s);
     } else {
-        if (HAS_SR && sr) {
-            if (vel == LBM_D1V3) return launch_lat<LatD1V3, S, HAS_SR>(force, efield, fin, fout, nbr, Ef, p, s);
-            return launch_lat<LatD3V27, S, HAS_SR>(force, efield, fin, fout, nbr, Ef, p, s);
-        }
-        if (vel == LBM_D1V3) return launch_lat<LatD1V3, S, false>(force, efield, fin, fout, nbr, Ef, p, s);
-        return launch_lat<LatD3V27, S, false>(force, efield, fin, fout, nbr, Ef, p, s);
+        if (vel == LBM_D1V3) return launch_lat<LatD1V3, S, SR>(force, efield, fin, fout, nbr, Ef, p, s);
+        return launch_lat<LatD3V27, S, SR>(force, efield, fin, fout, nbr, Ef, p, s);
     }
 }
 

@@ -1,0 +1,9 @@
+// Step kernels instantiated for StoreBF16 storage, D2V9 and D3V19, nearest rounding (see lbm_step.cuh).
+#include "lbm_step.cuh"
+
+namespace lbm {
+int launch_step_bf16_n(int vel, int force, bool efield, const void* fin, void* fout, const uint32_t* nbr, const float* Ef,
+    const KParams& p, cudaStream_t s) {
+    return stepk::launch_storage<StoreBF16, false, 0>(vel, force, efield, fin, fout, nbr, Ef, p, s);
+}
+}  // namespace lbm
