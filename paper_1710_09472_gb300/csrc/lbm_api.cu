@@ -294,8 +294,9 @@ void ws_release(lbm_ctx* c) {
 }
 
 // Units (see pop_slot).  A row stays whole while its rows of all directions,
-// twice staged and once as outputs, fit kRowSmem: three or more blocks then
-// share an SM.  A longer row is cut into segments: the usual ones
+// twice staged and once as outputs, fit kRowSmem: two or more blocks then
+// share an SM (cut at 64 KB, the D3V27 FP32 rows of 256 cells were slower: 0.746
+// against 0.675 ms per 256^3 step).  A longer row is cut into segments: the usual ones
 // (usual_segment) where they fit and pad the row by no more than an eighth,
 // what a compile-time stride gains; else equal ones of that many columns at
 // most.  As whole rows, D2V9 FP32 rows of 1024 cells kept one block of eight

@@ -271,7 +271,7 @@ struct StoreBF16 {
 constexpr int kPitch = 8, kMinStagedRow = 32;
 // A row is one unit of the staged kernels while three copies of it (all
 // directions) fit kRowSmem bytes; a longer row is cut (set_units, lbm_api.cu).
-constexpr int kRowSmem = 64 * 1024;
+constexpr int kRowSmem = 96 * 1024;
 template <class L, class S>
 __host__ __device__ constexpr bool whole_row(int nx) {
     return 3 * L::Q * nx * S::kBytes <= kRowSmem;
