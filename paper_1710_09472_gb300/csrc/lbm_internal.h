@@ -398,8 +398,9 @@ int launch_step(int vel, int storage, int force, bool efield, bool sr, const voi
                 const uint32_t* nbr, const float* Ef, const KParams& p, cudaStream_t s);
 // n steps in one launch where the box is small enough (lbm_multi.cuh); 0 where it
 // is not.  p.step is the first step's index; Ef is null for a uniform field;
-// count is a word of device memory for the launch's barrier.  The result is in
-// fout, or in fin where *in_fin says so; the other buffer is overwritten.
+// count is a word of device memory for the launch's barrier.  The result is where
+// n single steps leave it (fin for even n, which *in_fin says), so that a
+// captured call can be replayed; the other buffer may be overwritten.
 int launch_multi(int vel, int storage, int force, bool sr, void* fin, void* fout, const uint32_t* nbr, const float* Ef,
                  int n, unsigned* count, bool* in_fin, const KParams& p, cudaStream_t s);
 // one per storage, lattice group (_x: D3V27 and D1V3) and rounding (_n: nearest

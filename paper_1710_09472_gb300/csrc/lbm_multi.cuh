@@ -81,9 +81,10 @@ __device__ __forceinline__ void cluster_barrier() {
 // memory: two states h~_a at [a * cpc + i], and the destination of each value
 // as a cluster address into the second state (direction 0: the cell's place in
 // the padded field, or kNoCell for a solid cell).  Ef: the per-cell field, or null.
+// Pin and Pout may be the same buffer: every block has pulled its cells from it
+// before the first barrier, and none writes to it before the last step (n > 1).
 template <class L, class S, int FORCE, bool SR>
-__global__ void __launch_bounds__(kThreads<L>) k_step_multi(const typename S::T* __restrict__ Pin,
-                                                            typename S::T* __restrict__ Pout,
+__global__ void __launch_bounds__(kThreads<L>) k_step_multi(const typename S::T* Pin, typename S::T* Pout,
                                                             const uint32_t* __restrict__ nbr,
                                                             const float* __restrict__ Ef, int n, int cpc, KParams p) {
     using T = typename S::T;
@@ -283,9 +284,9 @@ inline int launched(cudaError_t e) {
 }
 
 // Launches n steps, or returns 0: a box that does not fit, or a device on which
-// the cluster cannot be placed.
+// the cluster cannot be placed.  The result is in fin when n is even.
 template <class L, class S, int FORCE, bool SR>
-int launch_cluster(const void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n, const KParams& p,
+int launch_cluster(void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n, const KParams& p,
                cudaStream_t s) {
     using T = typename S::T;
     const Plan plan = plan_of<L, S>(p);
@@ -322,10 +323,10 @@ int launch_cluster(const void* fin, void* fout, const uint32_t* nbr, const float
         }
         if (!fits) return 0;
     }
-    return launched(cudaLaunchKernelEx(&cfg, kern, (const T*)fin, (T*)fout, nbr, Ef, n, plan.cpc, p));
+    return launched(cudaLaunchKernelEx(&cfg, kern, (const T*)fin, (T*)(n % 2 ? fout : fin), nbr, Ef, n, plan.cpc, p));
 }
 
-// The same for the cooperative grid; the result is in fin when n is even.
+// The same for the cooperative grid.
 template <class L, class S, int FORCE, bool SR>
 int launch_grid(void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n, unsigned* count, const KParams& p,
                 cudaStream_t s) {
@@ -371,10 +372,10 @@ int launch_grid(void* fin, void* fout, const uint32_t* nbr, const float* Ef, int
 template <class L, class S, int FORCE, bool SR>
 int launch_one(void* fin, void* fout, const uint32_t* nbr, const float* Ef, int n, unsigned* count, bool* in_fin,
                const KParams& p, cudaStream_t s) {
-    *in_fin = false;
+    // as after n single steps, which a captured call is replayed as
+    *in_fin = n % 2 == 0;
     if (int k = launch_cluster<L, S, FORCE, SR>(fin, fout, nbr, Ef, n, p, s)) return k;
     if (p.N * L::Q <= kClusterWork) return 0;
-    *in_fin = n % 2 == 0;
     return launch_grid<L, S, FORCE, SR>(fin, fout, nbr, Ef, n, count, p, s);
 }
 
