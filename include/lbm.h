@@ -244,6 +244,18 @@ lbm_status lbm_adjoint_stats(const lbm_ctx* ctx, int64_t out[5]);
  * timeout is returned first. */
 lbm_status lbm_selftest_wait_timeout(lbm_ctx* ctx, int64_t clocks);
 
+/* The same for the kernels themselves: until it is called again with units < 0,
+ * the row-staged kernels of this context (steps, fields, reverse steps) copy only
+ * the first `units` units (rows, or segments of long rows) that their blocks
+ * begin with into shared memory, their waits for the others run out after
+ * `clocks` SM cycles (1 <= clocks <= 2^31), and so does the grid barrier of many
+ * steps in one launch where units are withheld.  A block whose wait ran out does
+ * no work on its remaining units' cells; the kernel ends, and the next
+ * synchronising call returns LBM_ERR_TIMEOUT.  The state is then invalid
+ * (lbm_init_equilibrium or lbm_load_state set a new one).
+ * The paper has no counterpart.  Errors: INVALID_ARG. */
+lbm_status lbm_selftest_withhold(lbm_ctx* ctx, int64_t units, int64_t clocks);
+
 /* Reverse-mode gradient of a linear functional of the trajectory that starts
  * at the current state f_0 (this is an addition to the paper's method: a
  * hand-written adjoint of the Sec. 9.1 step, with the Sec. 7 forcing):

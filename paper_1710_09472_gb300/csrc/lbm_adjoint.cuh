@@ -644,7 +644,7 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
 #pragma unroll
         for (int k = 0; k < STAGES - 1; ++k) {
             const int uk = blockIdx.x + k * G;
-            if (uk < U) {
+            if (uk < p.staged) {
                 uint32_t g0, g1;
                 range(uk, g0, g1);
                 unsigned char* st = smem_raw + k * sbytes;
@@ -662,17 +662,13 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_rows(const typename S::T* __
         const int sn = (it + STAGES - 1) % STAGES;  // ... into the stage of the previous unit
         uint32_t g0, g1;
         range(u, g0, g1);
-        if (ok && !dev::mbar_wait(&bar[cs], (uint32_t)(it / STAGES) & 1u)) {
-            ok = false;
-            if (p.status) atomicExch(p.status, 2);
-            dev::pause_cycles(1ll << 22);  // let this block's copies in flight land
-        }
         unsigned char* st = smem_raw + cs * sbytes;
+        uint16_t* ord = reinterpret_cast<uint16_t*>(lay.order(st));
+        ok = dev::stage_wait(&bar[cs], (uint32_t)(it / STAGES) & 1u, ok, 2, g0, g1, ord, p);
         T* prow = reinterpret_cast<T*>(lay.prows(st));
         float* ge_s = reinterpret_cast<float*>(lay.gerows(st));
         const float* ef_s = reinterpret_cast<const float*>(lay.efrows(st));
         float* lrow = reinterpret_cast<float*>(lay.lrows(st));
-        const uint16_t* ord = reinterpret_cast<const uint16_t*>(lay.order(st));
         const uint32_t* desc = reinterpret_cast<const uint32_t*>(lay.descs(st));
         const uint32_t d0 = wstart[cs][1];
         T* phal = reinterpret_cast<T*>(lay.phalo(st));

@@ -215,6 +215,9 @@ lbm::KParams lbm::make_params(const lbm_ctx* c) {
     p.lorder = c->lorder;
     p.lgofs = 0;
     p.status = c->status_dev;
+    p.wait_clocks = (uint32_t)c->wait_clocks;
+    const int64_t units = c->ny * c->nz * c->nseg;
+    p.staged = (int)(c->withhold < 0 ? units : std::min(units, c->withhold));
     p.seed = c->rseed;
     if (c->lmu_tab) {
         // table coordinate (rho / rho0 - 1) / dr + k1 from the scaled deviation drho~
@@ -1013,10 +1016,19 @@ lbm_status lbm_selftest_wait_timeout(lbm_ctx* c, int64_t clocks) {
         lbm_status _ds = device_status(c);  // an earlier timeout is reported first
         if (_ds != LBM_OK) return _ds;
     }
-    c->launches += lbm::launch_wait_probe(c->status_dev, (long long)clocks, c->stream);
+    c->launches += lbm::launch_wait_probe(c->status_dev, (uint32_t)clocks, c->stream);
     LBM_CUDA(c, cudaGetLastError());
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
     return device_status(c);
+}
+
+lbm_status lbm_selftest_withhold(lbm_ctx* c, int64_t units, int64_t clocks) {
+    if (!c) return LBM_ERR_INVALID_ARG;
+    if (units >= 0 && (clocks < 1 || clocks > lbm::kWaitClocks))
+        return fail(c, LBM_ERR_INVALID_ARG, "lbm_selftest_withhold: need 1 <= clocks <= 2^31");
+    c->withhold = units < 0 ? -1 : units;
+    c->wait_clocks = units < 0 ? lbm::kWaitClocks : clocks;
+    return LBM_OK;
 }
 
 lbm_status lbm_adjoint(lbm_ctx* c, const float* w_rho, const float* w_j, int64_t t_begin, int64_t t_end,

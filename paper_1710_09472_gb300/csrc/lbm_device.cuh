@@ -179,12 +179,13 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 // Waits for the phase of the given parity to complete; gives up and returns
-// false after `limit` SM clock cycles (default 2^31, about one second).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit = 1ll << 31) {
+// false after `limit` SM clock cycles (32 bits of the clock: a 64-bit count took
+// the FP32 step on D3V19 segments from 64 to 74 registers).
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit) {
     if (mbar_try(bar, parity)) return true;
-    const long long t0 = clock64();
+    const uint32_t t0 = (uint32_t)clock();
     while (!mbar_try(bar, parity))
-        if (clock64() - t0 > limit) return false;
+        if ((uint32_t)clock() - t0 > limit) return false;
     return true;
 }
 // Sleeps about n SM clock cycles.  After a wait has run out, a block pauses
@@ -192,6 +193,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
 __device__ __forceinline__ void pause_cycles(long long n) {
     const long long t0 = clock64();
     while (clock64() - t0 < n) __nanosleep(1000);
+}
+// Waits for a unit's stage; true when it has arrived.  When the wait runs out
+// (or ran out in an earlier unit: ok is false), code goes to the status word and
+// nothing of the stage may be taken for an address, so this thread empties its
+// link range (its passes over the descriptors do nothing) and its part of the
+// unit's cell order (no fluid cells, every column the unit's first).  All threads
+// do that, or the stage had arrived after all, before the next block barrier, so
+// the unit's passes stay inside their buffers; what they write is invalid.
+// The passes themselves have no test for it: one around the link pass took the
+// FP16 step of 256^3 D3V19 from 240.8 to 242.9 us, leaving the loop after the
+// barrier to 250.5.
+__device__ __forceinline__ bool stage_wait(uint64_t* bar, uint32_t parity, bool ok, int code, uint32_t g0,
+                                           uint32_t& g1, uint16_t* order, const KParams& p) {
+    if (ok && mbar_wait(bar, parity, p.wait_clocks)) return true;
+    if (ok) {
+        if (p.status) atomicExch(p.status, code);
+        pause_cycles(1ll << 22);  // let this block's copies in flight land
+    }
+    g1 = g0;
+    for (int k = threadIdx.x; k < p.lorder; k += blockDim.x) order[k] = 0;
+    return false;
 }
 
 // global -> shared, completing `bytes` on the mbarrier

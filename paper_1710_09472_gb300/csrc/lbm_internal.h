@@ -276,6 +276,8 @@ template <class L, class S>
 __host__ __device__ constexpr bool whole_row(int nx) {
     return 3 * L::Q * nx * S::kBytes <= kRowSmem;
 }
+// Limit of a bounded wait on the device: about one second.
+constexpr int64_t kWaitClocks = 1ll << 31;
 // What a staged kernel is compiled for: rows of exactly the compile-time stride,
 // rows, or segments.
 enum UnitMode { kExactRow, kWholeRow, kSegment };
@@ -327,6 +329,11 @@ struct KParams {
     // host-mapped status word: a kernel whose bounded wait ran out writes a
     // nonzero code here (read by the next synchronising API call)
     int* status;
+    // Bounded waits of the staged kernels and of the grid barrier give up after
+    // this many SM clock cycles.  Units from `staged` on are not staged (all are,
+    // but for lbm_selftest_withhold).
+    uint32_t wait_clocks;
+    int staged;
     // Local chemical-potential model (lbm_set_local_mu; null table: off):
     // dth(r) = thetabar(r) - thetabar_w at r = rho / rho0 as a cubic Hermite
     // table of (dth, dth' dr) pairs on lmu_n uniform nodes; drho~ lmu_a is
@@ -382,7 +389,7 @@ int launch_build_neighbors(int vel, const uint8_t* mask, uint32_t* nbr, unsigned
 // Link buffer layout: lbase[cell] (exclusive prefix of outgoing-link counts),
 // rowG[0..ny*nz*nseg]; needs a temporary of *temp_bytes (queried with temp == NULL).
 // Bounded-wait probe (writes code 3 into *status when its wait runs out).
-int launch_wait_probe(int* status, long long limit, cudaStream_t s);
+int launch_wait_probe(int* status, uint32_t limit, cudaStream_t s);
 // FP32 field in the populations' slot layout -> direction-major out[a * N + cell].
 int launch_unslot(int vel, const float* in, float* out, const KParams& p, cudaStream_t s);
 // Per-unit cell order (fluid cells first) for the row-staged kernels.
@@ -516,6 +523,8 @@ struct lbm_ctx {
     float2* lmu_tab = nullptr;     // local-mu model table (null: off)
     int* status_host = nullptr;    // mapped pinned word written by kernels on a wait timeout
     int* status_dev = nullptr;     // its device address
+    int64_t withhold = -1;         // lbm_selftest_withhold: units that are staged (-1: all)
+    int64_t wait_clocks = lbm::kWaitClocks;
     float* stage = nullptr;  // device staging for host-pointer arguments
     size_t stage_bytes = 0;
     bool geometry_counted = false;

@@ -294,19 +294,16 @@ __global__ void __launch_bounds__(256) k_moments_rows(const typename S::T* __res
     if (halo && dev::halo_thread<L>())
         dev::halo_put<L, true>(lay.halo(smem_raw), dev::halo_fetch<L, true>(P, dev::unit_at<0, MODE>(p, blockIdx.x), p));
     __syncthreads();
-    if (issuer && (int)blockIdx.x < U) stage(0, blockIdx.x);
+    if (issuer && (int)blockIdx.x < p.staged) stage(0, blockIdx.x);
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     bool ok = true;
     int it = 0;
     for (int u = blockIdx.x; u < U; u += G, ++it) {
         const int cs = it & 1, un = u + G;
         unsigned char* st = smem_raw + cs * sbytes;
-        const uint32_t g0 = __ldg(p.rowG + u), g1 = __ldg(p.rowG + u + 1);
-        if (ok && !dev::mbar_wait(&bar[cs], (uint32_t)(it >> 1) & 1u)) {
-            ok = false;
-            if (p.status) atomicExch(p.status, 5);
-            dev::pause_cycles(1ll << 22);  // let this block's copies in flight land
-        }
+        const uint32_t g0 = __ldg(p.rowG + u);
+        uint32_t g1 = __ldg(p.rowG + u + 1);
+        ok = dev::stage_wait(&bar[cs], (uint32_t)(it >> 1) & 1u, ok, 5, g0, g1, lay.order(st), p);
         T* buf = lay.rows(st);
         dev::patch_links<true, halo>(buf, rs, lay.halo(st), L::Q, lay.links(st), gstart[cs], g0, g1, lay.descs(st),
                                      dstart[cs]);
@@ -543,7 +540,7 @@ int launch_build_links(int vel, const uint32_t* nbr, uint32_t* lbase, uint32_t* 
 // Failure-path probe: one block waits, with the staged kernels' bounded
 // wait, on an mbarrier that nothing completes; the wait runs out after
 // `limit` clocks and the block writes code 3 into the status word.
-__global__ void k_wait_probe(int* status, long long limit) {
+__global__ void k_wait_probe(int* status, uint32_t limit) {
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) {
         dev::mbar_init(&bar, 1);
@@ -554,7 +551,7 @@ __global__ void k_wait_probe(int* status, long long limit) {
     if (!done && threadIdx.x == 0 && status) atomicExch(status, 3);
 }
 
-int launch_wait_probe(int* status, long long limit, cudaStream_t s) {
+int launch_wait_probe(int* status, uint32_t limit, cudaStream_t s) {
     k_wait_probe<<<1, 32, 0, s>>>(status, limit);
     return 1;
 }

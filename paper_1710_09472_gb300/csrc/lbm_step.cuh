@@ -486,8 +486,8 @@ __global__ void __launch_bounds__(kBlock) k_step(const typename S::T* __restrict
 // Two block barriers per unit; a stage is refilled after the first barrier of
 // the unit that follows its own.  Every wait on an mbarrier is bounded; one
 // that runs out writes a code to p.status, the block stops issuing copies, and
-// the kernel carries on (its results are then invalid, but it ends and no
-// access leaves its buffers).
+// its remaining units have no links and no fluid cells (stage_wait): the results
+// are invalid, but the kernel ends and no access leaves its buffers.
 //
 // Rows whose length is not a whole number of 16-byte chunks are staged with
 // their padding (kPitch): on the general kernel such a box took 2.7 times as
@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
 #pragma unroll
         for (int k = 0; k < STAGES - 1; ++k) {
             const int uk = blockIdx.x + k * G;
-            if (uk < U) {
+            if (uk < p.staged) {
                 uint32_t g0, g1;
                 range(uk, g0, g1);
                 stage_unit<L, S, RS, MODE>(smem_raw + k * sbytes, lay, &bar[k], Pin, uk, g0, g1, &gstart[k], &dstart[k], p);
@@ -619,12 +619,8 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
         const int sn = (it + STAGES - 1) % STAGES;  // ... into the stage of the previous unit
         uint32_t g0, g1;  // this unit's links
         range(u, g0, g1);
-        if (ok && !dev::mbar_wait(&bar[cs], (uint32_t)(it / STAGES) & 1u)) {
-            ok = false;
-            if (p.status) atomicExch(p.status, 1);
-            dev::pause_cycles(1ll << 22);  // let this block's copies in flight land
-        }
         unsigned char* st = smem_raw + cs * sbytes;
+        ok = dev::stage_wait(&bar[cs], (uint32_t)(it / STAGES) & 1u, ok, 1, g0, g1, lay.order(st), p);
         T* buf = lay.rows(st);
         T* orow = kInPlace ? buf : outrow;  // where this unit's outputs go
         const uint16_t* ord = lay.order(st);

@@ -218,6 +218,12 @@ class LBM:
         raw status; LBM_ERR_TIMEOUT is the expected answer."""
         return int(_lib.load().lbm_selftest_wait_timeout(self._h, int(clocks)))
 
+    def selftest_withhold(self, units: int = -1, clocks: int = 1 << 20):
+        """Make the waits of this context's kernels run out: only the first `units` units are staged
+        (lbm_selftest_withhold); units < 0 ends it."""
+        _lib.check(_lib.load().lbm_selftest_withhold(self._h, int(units), int(clocks)), self._h,
+                   "lbm_selftest_withhold")
+
     def moment_totals_static(self, out):
         """FP64 totals into `out` (a float64 device tensor of 4) without any
         device allocation (lbm_moment_totals_static)."""
