@@ -28,8 +28,6 @@
 // block owns (deterministic for a fixed launch shape).
 #pragma once
 
-#include <mutex>
-
 #include "lbm_device.cuh"
 
 namespace lbm {
@@ -840,27 +838,8 @@ bool launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const ui
     if (smem_ref > kAdjSmemBudget) return false;
     const int threads = p.seglen >= kAdjThreads ? kAdjThreads : ((p.seglen + 31) / 32) * 32;
     auto kern = k_adjoint_rows<L, S, FORCE, EF, WIN, kAdjStages, RS, MODE, LMU>;
-    // persistent grid: co-resident blocks per SM (occupancy API) x SMs,
-    // cached per instantiation and shared-memory size
-    static std::mutex mu;
-    static size_t last_smem = 0;
-    static int last_threads = 0, last_blocks = 0;
-    int blocks;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (smem_ref != last_smem || threads != last_threads) {
-            int dev = 0, sms = 0, per_sm = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (smem_ref > 48 * 1024)
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ref);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem_ref);
-            last_smem = smem_ref;
-            last_threads = threads;
-            last_blocks = per_sm > 0 ? per_sm * sms : 0;
-        }
-        blocks = last_blocks;
-    }
+    // persistent grid: co-resident blocks per SM x SMs
+    int blocks = staged_shape((const void*)kern, p.seglen, smem_ref, kAdjSmemBudget, threads).blocks;
     const int units = p.ny * p.nz * p.nseg;
     if (blocks > units) blocks = units;
     if (blocks <= 0 || blocks > slot_blocks) return false;

@@ -425,6 +425,26 @@ int64_t moments_partial_count(const KParams& p);
 // SMs of the current device, asked once per device (1 where it cannot be told).
 int sm_count();
 
+// What the runtime says about launching a kernel: block size, co-resident blocks
+// on the device (0: it cannot run) and SMs.  It is asked once per kernel, device,
+// size n and dynamic shared memory: known_shape gives an answer that keep_shape
+// was given (kLaunchShapes of them at most, for all contexts and threads).
+struct Shape {
+    int threads, blocks, sms;
+};
+constexpr size_t kLaunchShapes = 1024;
+bool known_shape(const void* kernel, int n, size_t smem, Shape* s);
+void keep_shape(const void* kernel, int n, size_t smem, const Shape& s);
+// Raises the kernel's dynamic shared memory on the current device to `budget`, the
+// same for every launch of it: a limit of one launch's own size could be lowered
+// by another thread's smaller box before the launch went out.
+bool allow_smem(const void* kernel, size_t budget);
+// Shape of a staged kernel: any multiple of 32 threads up to the row length works;
+// the choice is the one with the most co-resident blocks per SM, the larger block
+// on a tie.  fixed_threads != 0 takes that block size.
+constexpr int kRowThreads = 256;
+Shape staged_shape(const void* kernel, int columns, size_t smem, size_t budget, int fixed_threads = 0);
+
 // Adjoint (lbm_adjoint.cu).
 int64_t adjoint_slot_count(const KParams& p);
 int launch_adjoint_seed(int vel, int storage, const void* P, const uint32_t* nbr, const float* w_rho,

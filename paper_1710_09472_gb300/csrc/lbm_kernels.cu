@@ -16,6 +16,10 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdio>
+#include <map>
+#include <mutex>
+#include <new>
+#include <tuple>
 
 #include <cub/device/device_scan.cuh>
 
@@ -388,7 +392,7 @@ int64_t launch_moments_rows(const void* pop, float* rho, float* j, double* parti
                              dev::halo_bytes(L::Q, p.nseg, S::kBytes));
     if (smem > stepk::kSmemBudget) return 0;
     auto kern = p.nseg > 1 ? k_moments_rows<L, S, TOTALS, kSegment> : k_moments_rows<L, S, TOTALS, kWholeRow>;
-    const stepk::Shape sh = stepk::launch_shape(kern, p.seglen, smem);
+    const Shape sh = staged_shape((const void*)kern, p.seglen, smem, stepk::kSmemBudget);
     const int units = p.ny * p.nz * p.nseg;
     if (sh.blocks <= 0 || units < sh.sms) return 0;
     const int64_t blocks = std::min<int64_t>(std::min(sh.blocks, units), most);
@@ -492,10 +496,68 @@ int sm_count() {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kDevices) sms = known[dev].load();
     if (sms > 0) return sms;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    sms = std::max(sms, 1);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 1;
     if (dev >= 0 && dev < kDevices) known[dev].store(sms);
     return sms;
+}
+
+namespace {
+using ShapeKey = std::tuple<const void*, int, int, size_t>;
+std::mutex g_shapes_mutex;
+std::map<ShapeKey, Shape> g_shapes;
+ShapeKey shape_key(const void* kernel, int n, size_t smem) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return ShapeKey(kernel, dev, n, smem);
+}
+}  // namespace
+
+bool known_shape(const void* kernel, int n, size_t smem, Shape* s) {
+    const ShapeKey key = shape_key(kernel, n, smem);
+    std::lock_guard<std::mutex> lock(g_shapes_mutex);
+    const auto it = g_shapes.find(key);
+    if (it == g_shapes.end()) return false;
+    *s = it->second;
+    return true;
+}
+
+void keep_shape(const void* kernel, int n, size_t smem, const Shape& s) {
+    const ShapeKey key = shape_key(kernel, n, smem);
+    std::lock_guard<std::mutex> lock(g_shapes_mutex);
+    if (g_shapes.size() >= kLaunchShapes) g_shapes.clear();
+    try {
+        g_shapes[key] = s;
+    } catch (const std::bad_alloc&) {  // then it is asked again
+    }
+}
+
+bool allow_smem(const void* kernel, size_t budget) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget) == cudaSuccess)
+        return true;
+    cudaGetLastError();
+    return false;
+}
+
+Shape staged_shape(const void* kernel, int columns, size_t smem, size_t budget, int fixed_threads) {
+    Shape best;
+    if (known_shape(kernel, columns, smem, &best)) return best;
+    const int tmax = fixed_threads ? fixed_threads
+                                   : (columns >= kRowThreads ? kRowThreads : ((columns + 31) / 32) * 32);
+    const int tmin = fixed_threads ? fixed_threads : tmax / 2;
+    best = Shape{tmax, 0, sm_count()};
+    if (allow_smem(kernel, budget)) {
+        for (int t = tmax; t >= 32 && t >= tmin; t -= 32) {
+            int per_sm = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, t, smem) != cudaSuccess)
+                cudaGetLastError();
+            if (per_sm * best.sms > best.blocks) {
+                best.blocks = per_sm * best.sms;
+                best.threads = t;
+            }
+        }
+    }
+    keep_shape(kernel, columns, smem, best);
+    return best;
 }
 
 int64_t moments_partial_count(const KParams& p) {

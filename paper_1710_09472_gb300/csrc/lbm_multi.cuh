@@ -28,8 +28,6 @@
 // results have the same bits.
 #pragma once
 
-#include <mutex>
-
 #include "lbm_step.cuh"
 
 namespace lbm {
@@ -305,26 +303,19 @@ int launch_cluster(void* fin, void* fout, const uint32_t* nbr, const float* Ef, 
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    {
-        // whether the device can place this cluster; asked once per shape
-        static std::mutex mu;
-        static int last_blocks = 0, last_threads = 0;
-        static size_t last_smem = 0;
-        static bool fits = false;
-        std::lock_guard<std::mutex> lock(mu);
-        if (last_blocks != plan.blocks || last_smem != plan.smem || last_threads != threads) {
-            int clusters = 0;
-            fits = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) ==
-                       cudaSuccess &&
-                   cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0;
-            if (!fits) cudaGetLastError();
-            last_blocks = plan.blocks;
-            last_smem = plan.smem;
-            last_threads = threads;
-        }
-        if (!fits) return 0;
+    // whether the device can place this cluster
+    const int n_shape = plan.blocks * 4096 + threads;
+    Shape sh;
+    if (!known_shape((const void*)kern, n_shape, plan.smem, &sh)) {
+        int clusters = 0;
+        if (!allow_smem((const void*)kern, kSmemMax) ||
+            cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess)
+            cudaGetLastError();
+        sh = Shape{threads, clusters * plan.blocks, 0};
+        keep_shape((const void*)kern, n_shape, plan.smem, sh);
     }
+    if (sh.blocks <= 0) return 0;
     return launched(cudaLaunchKernelEx(&cfg, kern, (const T*)fin, (T*)(n % 2 ? fout : fin), nbr, Ef, n, plan.cpc, p));
 }
 
@@ -334,41 +325,29 @@ int launch_grid(void* fin, void* fout, const uint32_t* nbr, const float* Ef, int
                 cudaStream_t s) {
     using T = typename S::T;
     auto kern = k_step_grid<L, S, FORCE, SR>;
-    static std::mutex mu;
-    static int sms = 0;  // SMs, 0 where the device has no cooperative launch
-    static int asked_threads = 0;
-    static bool fits = false;
-    int threads;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (sms == 0) {
-            int dev = 0, coop = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-            if (coop) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (sms < 1) return 0;
-        }
-        const int64_t per = ((p.N + sms - 1) / sms + 31) / 32 * 32;
-        if (per > kGridThreads<L>) return 0;
-        threads = (int)per;
-        if (asked_threads != threads) {
-            int blocks = 0;
-            const size_t smem = (size_t)(L::Q - 1) * threads * 4;
-            fits = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
-                   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, threads, smem) == cudaSuccess &&
-                   blocks > 0;
-            if (!fits) cudaGetLastError();
-            asked_threads = threads;
-        }
-        if (!fits) return 0;
+    const int sms = sm_count();
+    const int64_t per = ((p.N + sms - 1) / sms + 31) / 32 * 32;
+    if (per > kGridThreads<L>) return 0;
+    const int threads = (int)per;
+    const size_t smem = (size_t)(L::Q - 1) * threads * 4;
+    Shape sh;
+    if (!known_shape((const void*)kern, threads, smem, &sh)) {
+        int dev = 0, coop = 0, per_sm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        if (!coop || !allow_smem((const void*)kern, (size_t)(L::Q - 1) * kGridThreads<L> * 4) ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess)
+            cudaGetLastError();
+        sh = Shape{threads, per_sm * sms, sms};
+        keep_shape((const void*)kern, threads, smem, sh);
     }
+    const unsigned blocks = (unsigned)((p.N + threads - 1) / threads);
+    if ((int64_t)blocks > sh.blocks) return 0;
     if (!launched(cudaMemsetAsync(count, 0, sizeof(unsigned), s))) return 0;
     T *A = (T*)fin, *B = (T*)fout;
     KParams q = p;
     void* args[] = {&A, &B, &nbr, &Ef, &n, &count, &q};
-    const unsigned blocks = (unsigned)((p.N + threads - 1) / threads);
-    return launched(cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3((unsigned)threads), args,
-                                                (size_t)(L::Q - 1) * threads * 4, s));
+    return launched(cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3((unsigned)threads), args, smem, s));
 }
 
 template <class L, class S, int FORCE, bool SR>

@@ -4,7 +4,6 @@
 // Included by one translation unit per storage type.
 #pragma once
 
-#include <mutex>
 #include <type_traits>
 
 #include "lbm_device.cuh"
@@ -766,54 +765,13 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
 // capped by the number of units.
 // ---------------------------------------------------------------------------
 constexpr int kStages = 2;
-constexpr int kRowThreads = 256;
 constexpr size_t kSmemBudget = 160 * 1024;
 
-// Block size and persistent grid of the row-staged kernel.  A block walks
-// whole rows, so any multiple of 32 threads up to the row length works; the
-// choice is the one with the most co-resident blocks per SM (occupancy API),
-// the larger block on a tie: more rows in flight per SM hide the per-row
-// copy latency.  256-cell FP16 rows: 192 threads (six blocks per SM) take
-// 0.258 ms per 256^3 step, against 0.268 at 160, 0.277 at 224 and 0.278 at
-// 256 threads.  fixed_threads != 0 takes that block size (the in-place FP32
-// rows need one thread per cell).
-struct Shape {
-    int threads, blocks, sms;
-};
-template <class K>
-Shape launch_shape(K kernel, int nx, size_t smem, int fixed_threads = 0) {
-    static std::mutex mu;
-    static const void* last_k = nullptr;
-    static size_t last_smem = 0;
-    static int last_nx = 0;
-    static Shape last{0, 0, 0};
-    std::lock_guard<std::mutex> lock(mu);
-    if ((const void*)kernel != last_k || smem != last_smem || nx != last_nx) {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        const int tmax = fixed_threads ? fixed_threads : (nx >= kRowThreads ? kRowThreads : ((nx + 31) / 32) * 32);
-        const int tmin = fixed_threads ? fixed_threads : tmax / 2;
-        Shape best{tmax, 0, sms};
-        int best_per_sm = -1;
-        for (int t = tmax; t >= 32 && t >= tmin; t -= 32) {
-            int per_sm = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, t, smem);
-            if (per_sm > best_per_sm) {
-                best_per_sm = per_sm;
-                best.threads = t;
-            }
-        }
-        best.blocks = best_per_sm > 0 ? best_per_sm * sms : 0;
-        last_k = (const void*)kernel;
-        last_smem = smem;
-        last_nx = nx;
-        last = best;
-    }
-    return last;
-}
-
+// Block size and persistent grid of the row-staged kernel (staged_shape): more
+// rows in flight per SM hide the per-row copy latency.  256-cell FP16 rows: 192
+// threads (six blocks per SM) take 0.258 ms per 256^3 step, against 0.268 at 160,
+// 0.277 at 224 and 0.278 at 256 threads.  The in-place FP32 rows need one thread
+// per cell.
 template <class L, class S, int FORCE, bool EF, bool SR, int RS, int MODE, bool LMU = false>
 bool launch_rows(const S*, const void* fin, void* fout, const uint32_t* nbr, const float* Ef, const KParams& p,
                  cudaStream_t s) {
@@ -830,7 +788,7 @@ bool launch_rows(const S*, const void* fin, void* fout, const uint32_t* nbr, con
     if (smem > kSmemBudget) return false;
     auto kern = k_step_rows<L, S, FORCE, EF, SR, kStages, RS, MODE, LMU>;
     // one cell per thread in place: exactly 256 threads
-    const Shape sh = launch_shape(kern, p.seglen, smem, kInPlace ? RS : 0);
+    const Shape sh = staged_shape((const void*)kern, p.seglen, smem, kSmemBudget, kInPlace ? RS : 0);
     const int threads = sh.threads, blocks = sh.blocks;
     if (blocks <= 0) return false;
     const int units = p.ny * p.nz * p.nseg;
