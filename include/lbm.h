@@ -447,6 +447,15 @@ const char* lbm_status_string(lbm_status s);
 /* Number of kernels this context has launched so far (host-side counter). */
 int64_t lbm_launch_count(const lbm_ctx* ctx);
 
+/* The kernel that the context's last launch of an operation (0: a step, 1: the
+ * fields or totals, 2: a reverse step) ran, for tests and benchmarks that mean a
+ * certain one: out = {kind, units, columns} with kind 0 none yet, 1 general (a
+ * thread per cell), 2 row-staged, 3 many steps on a cluster, 4 many steps on a
+ * cooperative grid; for a row-staged one units 0 rows of exactly `columns`
+ * cells, 1 rows, 2 segments of rows, and columns its compile-time stride or 0.
+ * The paper has no counterpart.  Errors: INVALID_ARG. */
+lbm_status lbm_last_kernel(const lbm_ctx* ctx, int operation, int out[3]);
+
 #ifdef __cplusplus
 }
 #endif

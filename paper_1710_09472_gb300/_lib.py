@@ -63,6 +63,7 @@ SIGNATURES = {
     "lbm_moment_totals_static": (_i, [_vp, _vp]),
     "lbm_last_error": (ctypes.c_char_p, [_vp]),
     "lbm_status_string": (ctypes.c_char_p, [_i]),
+    "lbm_last_kernel": (_i, [_vp, _i, _vp]),
     "lbm_launch_count": (_i64, [_vp]),
     "lbm_selftest_withhold": (_i, [_vp, _i64, _i64]),
     "lbm_selftest_wait_timeout": (_i, [_vp, _i64]),

@@ -817,11 +817,11 @@ constexpr int kAdjThreads = 256;
 constexpr size_t kAdjSmemBudget = 200 * 1024;
 
 template <class L, class S, int FORCE, bool EF, bool WIN, int RS, int MODE, bool LMU = false>
-bool launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
+int launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
                  const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
                  const KParams& p, cudaStream_t s) {
     if (!p.rorder || (RS && RS != p.seglen) || (MODE == kExactRow && RS != p.nx) || (MODE == kSegment) != (p.nseg > 1))
-        return false;
+        return 0;
     const int gcapP = dev::window_cap(p.max_row_links, S::kBytes);
     const int gcapL = dev::window_cap(p.max_row_links, 4);
     const int rs = p.seglen, hP = dev::halo_bytes(L::Q, p.nseg, S::kBytes), hL = dev::halo_bytes(L::Q, p.nseg, 4);
@@ -835,22 +835,22 @@ bool launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const ui
     // dL/dE rows, whether or not this call has them, so that the blocks (and
     // with them the order of the FP64 gradient sums) are the same either way
     const size_t smem_ref = smem_for(gerow);
-    if (smem_ref > kAdjSmemBudget) return false;
+    if (smem_ref > kAdjSmemBudget) return 0;
     const int threads = p.seglen >= kAdjThreads ? kAdjThreads : ((p.seglen + 31) / 32) * 32;
     auto kern = k_adjoint_rows<L, S, FORCE, EF, WIN, kAdjStages, RS, MODE, LMU>;
     // persistent grid: co-resident blocks per SM x SMs
     int blocks = staged_shape((const void*)kern, p.seglen, smem_ref, kAdjSmemBudget, threads).blocks;
     const int units = p.ny * p.nz * p.nseg;
     if (blocks > units) blocks = units;
-    if (blocks <= 0 || blocks > slot_blocks) return false;
+    if (blocks <= 0 || blocks > slot_blocks) return 0;
     kern<<<blocks, threads, smem, s>>>((const typename S::T*)P, lam_in, lam_out, Ef, w_rho, w_j, gE, slots,
                                        gcapP, gcapL, p);
-    return true;
+    return route(kStaged, MODE, RS);
 }
 
 // Rows or segments at a run-time stride.
 template <class L, class S, int FORCE, bool EF, bool WIN, bool LMU = false>
-bool launch_rows_any(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
+int launch_rows_any(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
                      const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
                      const KParams& p, cudaStream_t s) {
     return p.nseg > 1 ? launch_rows_rs<L, S, FORCE, EF, WIN, 0, kSegment, LMU>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j,
@@ -862,7 +862,7 @@ bool launch_rows_any(const void* P, const float* lam_in, float* lam_out, const u
 // The shared-memory row stride is a compile-time constant for the usual units,
 // as in the step kernel.
 template <class L, class S, int FORCE, bool EF, bool WIN>
-bool launch_rows(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
+int launch_rows(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
                  const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
                  const KParams& p, cudaStream_t s) {
     // the compile-time strides only for the benchmarked lattices (D2V9, D3V19)
@@ -908,18 +908,21 @@ int step_storage(int vel, int force, bool efield, bool in_window, const void* P,
     return dispatch_lattice<GROUP>(vel, [&](auto lat) {
         using L = decltype(lat);
         const auto* Pt = (const typename S::T*)P;
+        int done = route(kGeneral);
 // GROUP 2: the local-mu model (D2V9, D3V19), whose staged reverse kernel is
 // an instantiation of its own with the run-time row stride
 #define LBM_ADJ(F, EFV, W)                                                                                    \
     do {                                                                                                      \
-        bool staged;                                                                                          \
+        int staged;                                                                                           \
         if constexpr (GROUP == 2)                                                                             \
             staged = launch_rows_any<L, S, F, EFV, W, true>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,      \
                                                             slots, slot_blocks, p, s);                        \
         else                                                                                                  \
             staged = launch_rows<L, S, F, EFV, W>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots,         \
                                                   slot_blocks, p, s);                                         \
-        if (!staged)                                                                                          \
+        if (staged)                                                                                           \
+            done = staged;                                                                                    \
+        else                                                                                                  \
             k_adjoint_step<L, S, F, EFV, W>                                                                   \
                 <<<(unsigned)slot_blocks, l.block, 0, s>>>(Pt, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,      \
                                                            slots, (int)l.grid.y, p);                          \
@@ -938,7 +941,7 @@ int step_storage(int vel, int force, bool efield, bool in_window, const void* P,
             }
         }
 #undef LBM_ADJ
-        return 1;
+        return done;
     });
 }
 

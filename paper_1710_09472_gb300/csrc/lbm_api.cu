@@ -387,7 +387,7 @@ void advance(lbm_ctx* c, KParams& p, int64_t n) {
         if (!k)
             k = lbm::launch_step(c->lat.vel, c->storage, c->lat.force, c->use_Efield, c->stochastic, c->pop[c->cur],
                                  c->pop[c->cur ^ 1], c->nbr, c->Efield, p, c->stream);
-        c->launches += k;
+        lbm::note(c, lbm::kOpStep, k);
         if (!(done > 1 && in_place)) c->cur ^= 1;
         c->steps += done;
         t += done;
@@ -479,6 +479,15 @@ lbm_status lbm_weight_integrals(int D, int stat, double theta, double mu, double
 const char* lbm_last_error(const lbm_ctx* c) { return c ? c->err.c_str() : "null context"; }
 
 int64_t lbm_launch_count(const lbm_ctx* c) { return c ? c->launches : 0; }
+
+lbm_status lbm_last_kernel(const lbm_ctx* c, int operation, int out[3]) {
+    if (!c || !out || operation < lbm::kOpStep || operation > lbm::kOpReverse) return LBM_ERR_INVALID_ARG;
+    const int r = c->route[operation];
+    out[0] = (r >> 4) & 15;
+    out[1] = (r >> 8) & 15;
+    out[2] = r >> 12;
+    return LBM_OK;
+}
 
 lbm_status lbm_create(lbm_ctx** out, const lbm_lattice* lat, const int64_t dims[3], double tau, const double E[3],
                       const double B[3], int storage, void* cuda_stream) {
@@ -822,8 +831,9 @@ lbm_status lbm_moments(lbm_ctx* c, float* rho, float* j, double* total_rho, doub
     const bool want_totals = total_rho || total_j;
     KParams p = make_params(c);
     int64_t np = 0;
-    lbm_status st = after_launch(c, lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, rho_d, j_d,
-                                                         want_totals ? c->partials : nullptr, &np, p, c->stream));
+    lbm::note(c, lbm::kOpMoments, lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, rho_d, j_d,
+                                                      want_totals ? c->partials : nullptr, &np, p, c->stream));
+    lbm_status st = after_launch(c, 0);
     if (st != LBM_OK) return st;
     if (want_totals) {
         st = after_launch(c, lbm::launch_reduce_partials(c->partials, np, c->totals_dev, c->stream));
@@ -958,20 +968,21 @@ lbm_status lbm_window_totals(lbm_ctx* c, int64_t t_begin, int64_t t_end, double 
     LBM_CUDA(c, cudaMemsetAsync(c->totals_dev, 0, sizeof(double) * 4, c->stream));
     int64_t np = 0;
     if (t_begin < 0) {  // the start state itself is in the window
-        c->launches += lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, nullptr, nullptr,
-                                           c->partials, &np, p, c->stream);
+        lbm::note(c, lbm::kOpMoments, lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, nullptr,
+                                                          nullptr, c->partials, &np, p, c->stream));
         c->launches += lbm::launch_accumulate_totals(c->partials, np, c->totals_dev, c->stream);
     }
     const int64_t before = std::max<int64_t>(t_begin, 0);  // steps whose states are not in the window
     advance(c, p, before);
     for (int64_t t = before + 1; t <= t_end; ++t) {
         p.step = (uint32_t)(c->steps);
-        c->launches += lbm::launch_step(c->lat.vel, c->storage, c->lat.force, c->use_Efield, c->stochastic,
-                                        c->pop[c->cur], c->pop[c->cur ^ 1], c->nbr, c->Efield, p, c->stream);
+        lbm::note(c, lbm::kOpStep, lbm::launch_step(c->lat.vel, c->storage, c->lat.force, c->use_Efield, c->stochastic,
+                                                    c->pop[c->cur], c->pop[c->cur ^ 1], c->nbr, c->Efield, p,
+                                                    c->stream));
         c->cur ^= 1;
         c->steps += 1;
-        c->launches += lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, nullptr, nullptr,
-                                           c->partials, &np, p, c->stream);
+        lbm::note(c, lbm::kOpMoments, lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, nullptr,
+                                                          nullptr, c->partials, &np, p, c->stream));
         c->launches += lbm::launch_accumulate_totals(c->partials, np, c->totals_dev, c->stream);
     }
     LBM_CUDA(c, cudaGetLastError());
@@ -1196,14 +1207,15 @@ lbm_status lbm_adjoint(lbm_ctx* c, const float* w_rho, const float* w_j, int64_t
     // one forward step of global index step0 + t, in -> out
     auto fstep = [&](int64_t t, const void* in, void* out) {
         p.step = (uint32_t)(step0 + t);
-        c->launches += lbm::launch_step(vel, sto, force, ef, sr, in, out, c->nbr, c->Efield, p, c->stream);
+        lbm::note(c, lbm::kOpStep, lbm::launch_step(vel, sto, force, ef, sr, in, out, c->nbr, c->Efield, p, c->stream));
         ++fwd_steps;
     };
     // one reverse step at t from the state at t: lam_{t+1} -> lam_t
     auto rstep = [&](int64_t t, const void* state) {
         const bool win = t > t_begin && t <= t_end;
-        c->launches += lbm::launch_adjoint_step(vel, sto, force, ef, win, state, lam[li], lam[li ^ 1], c->nbr,
-                                                c->Efield, wr_d, wj_d, gpart, slots, p, c->stream);
+        lbm::note(c, lbm::kOpReverse, lbm::launch_adjoint_step(vel, sto, force, ef, win, state, lam[li], lam[li ^ 1],
+                                                               c->nbr, c->Efield, wr_d, wj_d, gpart, slots, p,
+                                                               c->stream));
         li ^= 1;
         if (gpart && ++rsteps % kFoldEvery == 0)
             c->launches += lbm::launch_fold_partials(gpart, dL_dE, c->D, p, c->stream);

@@ -383,7 +383,14 @@ struct Launch {
     dim3 grid, block;
 };
 
-// Launchers (lbm_kernels.cu).  Each returns the number of kernels launched.
+// What the launcher of a step, of the fields or of a reverse step returns: one
+// kernel, its kind, and for a staged one its unit mode (UnitMode) and compile-time
+// columns (0: a run-time stride).  0: nothing was launched.
+enum KernelKind { kGeneral = 1, kStaged, kCluster, kGrid };
+constexpr int route(int kind, int mode = 0, int columns = 0) { return 1 | kind << 4 | mode << 8 | columns << 12; }
+
+// Launchers (lbm_kernels.cu).  Each returns the number of kernels launched, or
+// the route of the one.
 int launch_build_neighbors(int vel, const uint8_t* mask, uint32_t* nbr, unsigned long long* fluid_count,
                            const KParams& p, cudaStream_t s);
 // Link buffer layout: lbase[cell] (exclusive prefix of outgoing-link counts),
@@ -474,7 +481,6 @@ namespace lbm {
 KParams make_params(const lbm_ctx* c);
 }  // namespace lbm
 
-// The context (opaque to C callers).
 // Device buffers of lbm_adjoint, kept by the context between calls so that
 // repeated calls allocate once (released by lbm_release_workspace,
 // lbm_set_geometry and lbm_destroy).
@@ -496,6 +502,7 @@ struct AdjWorkspace {
     }
 };
 
+// The context (opaque to C callers).
 struct lbm_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -551,5 +558,15 @@ struct lbm_ctx {
     bool has_state = false;
     int64_t steps = 0;
     int64_t launches = 0;
+    int route[3] = {0, 0, 0};  // of the last step, fields and reverse step (lbm_last_kernel)
     std::string err;
 };
+
+namespace lbm {
+enum Operation { kOpStep, kOpMoments, kOpReverse };
+// Counts a launch by its route.
+inline void note(lbm_ctx* c, Operation op, int r) {
+    c->launches += r & 15;
+    if (r) c->route[op] = r;
+}
+}  // namespace lbm

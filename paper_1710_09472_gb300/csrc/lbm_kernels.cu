@@ -709,12 +709,12 @@ int launch_moments(int vel, int storage, const void* pop, const uint32_t* nbr, f
             const int64_t staged = partials ? launch_moments_rows<L, S, true>(pop, rho, j, partials, tiles, p, s)
                                             : launch_moments_rows<L, S, false>(pop, rho, j, nullptr, tiles, p, s);
             if (n_partials) *n_partials = staged ? staged : blocks;
-            if (staged) return 1;
+            if (staged) return route(kStaged, p.nseg > 1 ? kSegment : kWholeRow);
             if (partials)
                 k_moments<L, S, true><<<(unsigned)blocks, l.block, 0, s>>>((const T*)pop, nbr, rho, j, partials, chunks, p);
             else
                 k_moments<L, S, false><<<(unsigned)blocks, l.block, 0, s>>>((const T*)pop, nbr, rho, j, nullptr, chunks, p);
-            return 1;
+            return route(kGeneral);
         });
     });
 }

@@ -316,7 +316,9 @@ int launch_cluster(void* fin, void* fout, const uint32_t* nbr, const float* Ef, 
         keep_shape((const void*)kern, n_shape, plan.smem, sh);
     }
     if (sh.blocks <= 0) return 0;
-    return launched(cudaLaunchKernelEx(&cfg, kern, (const T*)fin, (T*)(n % 2 ? fout : fin), nbr, Ef, n, plan.cpc, p));
+    return launched(cudaLaunchKernelEx(&cfg, kern, (const T*)fin, (T*)(n % 2 ? fout : fin), nbr, Ef, n, plan.cpc, p))
+               ? route(kCluster)
+               : 0;
 }
 
 // The same for the cooperative grid.
@@ -347,7 +349,9 @@ int launch_grid(void* fin, void* fout, const uint32_t* nbr, const float* Ef, int
     T *A = (T*)fin, *B = (T*)fout;
     KParams q = p;
     void* args[] = {&A, &B, &nbr, &Ef, &n, &count, &q};
-    return launched(cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3((unsigned)threads), args, smem, s));
+    return launched(cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3((unsigned)threads), args, smem, s))
+               ? route(kGrid)
+               : 0;
 }
 
 template <class L, class S, int FORCE, bool SR>

@@ -69,8 +69,8 @@ extern "C" lbm_status lbm_moment_totals_static(lbm_ctx* c, double* totals) {
         scratch = g_addr[dev];
     }
     int64_t np = 0;
-    c->launches += lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, nullptr, nullptr, scratch,
-                                       &np, p, c->stream);
+    lbm::note(c, lbm::kOpMoments, lbm::launch_moments(c->lat.vel, c->storage, c->pop[c->cur], c->nbr, nullptr, nullptr,
+                                                      scratch, &np, p, c->stream));
     c->launches += lbm::launch_reduce_partials(scratch, np, totals, c->stream);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {

@@ -773,11 +773,11 @@ constexpr size_t kSmemBudget = 160 * 1024;
 // 0.277 at 224 and 0.278 at 256 threads.  The in-place FP32 rows need one thread
 // per cell.
 template <class L, class S, int FORCE, bool EF, bool SR, int RS, int MODE, bool LMU = false>
-bool launch_rows(const S*, const void* fin, void* fout, const uint32_t* nbr, const float* Ef, const KParams& p,
+int launch_rows(const S*, const void* fin, void* fout, const uint32_t* nbr, const float* Ef, const KParams& p,
                  cudaStream_t s) {
     using T = typename S::T;
     if (!p.rorder || (RS && RS != p.seglen) || (MODE == kExactRow && RS != p.nx) || (MODE == kSegment) != (p.nseg > 1))
-        return false;
+        return 0;
     const size_t srow = (size_t)p.seglen * S::kBytes;
     const int gcap = dev::window_cap(p.max_row_links, S::kBytes);
     const int dcap = dev::window_cap(p.max_row_links, 4);
@@ -785,20 +785,20 @@ bool launch_rows(const S*, const void* fin, void* fout, const uint32_t* nbr, con
                                dev::halo_bytes(L::Q, p.nseg, S::kBytes);
     constexpr bool kInPlace = kInPlaceOut<S, RS, MODE, LMU>;
     const size_t smem = (size_t)kStages * stage_bytes + (kInPlace ? 0 : (size_t)L::Q * srow);
-    if (smem > kSmemBudget) return false;
+    if (smem > kSmemBudget) return 0;
     auto kern = k_step_rows<L, S, FORCE, EF, SR, kStages, RS, MODE, LMU>;
     // one cell per thread in place: exactly 256 threads
     const Shape sh = staged_shape((const void*)kern, p.seglen, smem, kSmemBudget, kInPlace ? RS : 0);
     const int threads = sh.threads, blocks = sh.blocks;
-    if (blocks <= 0) return false;
+    if (blocks <= 0) return 0;
     const int units = p.ny * p.nz * p.nseg;
     // Fewer units than SMs: most of the chip would idle while each block runs its
     // chain of copy, wait and two barriers once; the general kernel spreads the
     // cells over more blocks (4096 x 8 cells of D2V9 BF16, 128 units: 6.2 us a
     // step staged, below the 4.1 us that a launch takes the host otherwise).
-    if (units < sh.sms) return false;
+    if (units < sh.sms) return 0;
     kern<<<blocks < units ? blocks : units, threads, smem, s>>>((const T*)fin, (T*)fout, Ef, gcap, dcap, p);
-    return true;
+    return route(kStaged, MODE, RS);
 }
 
 // Row-staged kernel when the rows qualify, with the shared-memory row stride a
@@ -833,7 +833,8 @@ int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef
     using Segment = std::integral_constant<int, kSegment>;
     const std::true_type local{};
     const std::false_type plain{};
-    bool done = false, tried = false;
+    int done = 0;
+    bool tried = false;
     if constexpr (kFixed) {
         if (p.lmu_tab) {  // the local-mu model (D2V9, D3V19 only)
             tried = true;
@@ -864,11 +865,11 @@ int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef
         }
     }
     if (!tried) done = p.nseg > 1 ? rows(R0{}, Segment{}, plain) : rows(R0{}, Whole{}, plain);
-    if (done) return 1;
+    if (done) return done;
     const int bx = p.nx >= kBlock ? kBlock : ((p.nx + 31) / 32) * 32;
     const dim3 grid((unsigned)(p.ny * p.nz), (unsigned)((p.nx + bx - 1) / bx));
     k_step<L, S, FORCE, EF, SR><<<grid, bx, 0, s>>>((const T*)fin, (T*)fout, nbr, Ef, p);
-    return 1;
+    return route(kGeneral);
 }
 
 template <class L, class S, bool SR>

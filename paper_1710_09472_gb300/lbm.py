@@ -151,6 +151,15 @@ class LBM:
     def launch_count(self) -> int:
         return int(_lib.load().lbm_launch_count(self._h))
 
+    def last_kernel(self, operation: str):
+        """The kernel of the last "step", "moments" or "reverse" launch: (kind, units, columns)
+        (lbm_last_kernel); units is None for a kind without units."""
+        out = (ctypes.c_int * 3)()
+        op = {"step": 0, "moments": 1, "reverse": 2}[operation]
+        _lib.check(_lib.load().lbm_last_kernel(self._h, op, out), self._h, "lbm_last_kernel")
+        kind = ["none", "general", "staged", "cluster", "grid"][out[0]]
+        return kind, (["exact", "rows", "segments"][out[1]] if kind == "staged" else None), int(out[2])
+
     # -- set-up -------------------------------------------------------------------
     def set_geometry(self, mask):
         _lib.check(_lib.load().lbm_set_geometry(self._h, _ptr(mask, np.uint8, self.N, "mask")), self._h,
