@@ -630,7 +630,9 @@ __global__ void __launch_bounds__(256) k_step_rows(const typename S::T* __restri
         // bounced values in place, output rows free; a timeout anywhere in
         // the block stops the copies
         ok = __syncthreads_and(ok) != 0;
-        if (issuer && ok && un < U) {
+        // (the local-mu kernel spills four bytes with U here: 269.7 us against 263.2
+        // per 256^3 D3V19 FP16 step; the others are the same or slower with p.staged)
+        if (issuer && ok && un < (LMU ? p.staged : U)) {
             // refill the stage of the previous unit: every thread is past its
             // last reads of it (the link pass that follows the output) and
             // its wait on that stage's barrier
