@@ -66,7 +66,7 @@ int launch_fold_partials(float* part, double* acc, int D, const KParams& p, cuda
 }
 
 int64_t adjoint_slot_count(const KParams& p) {
-    return adjk::strided_blocks(p) * adjk::kSlots;
+    return adjk::slot_blocks(p) * adjk::kSlots;
 }
 
 int launch_adjoint_seed(int vel, int storage, const void* P, const uint32_t* nbr, const float* w_rho,

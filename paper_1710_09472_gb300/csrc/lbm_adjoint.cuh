@@ -28,6 +28,8 @@
 // block owns (deterministic for a fixed launch shape).
 #pragma once
 
+#include <algorithm>
+
 #include "lbm_device.cuh"
 
 namespace lbm {
@@ -786,12 +788,24 @@ inline Launch grid_of(const KParams& p) {
     return l;
 }
 
-// Blocks of the general reverse kernels, and with them the gradient slots.
+// Blocks of the general reverse kernels.
 constexpr int kAdjPerSm = 8;
 inline int64_t strided_blocks(const KParams& p) {
     const Launch l = grid_of(p);
     const int64_t tiles = (int64_t)l.grid.x * l.grid.y, cap = (int64_t)sm_count() * kAdjPerSm;
     return tiles < cap ? tiles : cap;
+}
+// Gradient slots, and with them the most blocks of a reverse kernel.  Narrow rows
+// have 12 to 21 staged blocks resident per SM.  Boxes of many units take up to 16
+// (us per forward and reverse step: D2V9 FP32 64 x 16384 77.5, with eight 82.3, on
+// the general kernel 97.5; D3V19 FP16 32 x 128 x 128 74.4, 88.9, 110.7); boxes whose
+// blocks come round a few times only take eight (64 x 2048 27.7, with 16 30.2;
+// 64 x 4096 35.7 and 36.8).  The line lies between the measured 4096 and 16384 units.
+inline int64_t slot_blocks(const KParams& p) {
+    const Launch l = grid_of(p);
+    const int64_t units = (int64_t)p.ny * p.nz * p.nseg;
+    const int64_t most = std::max<int64_t>((int64_t)l.grid.x * l.grid.y, units);
+    return std::min<int64_t>(most, (int64_t)sm_count() * (units > 8192 ? 2 * kAdjPerSm : kAdjPerSm));
 }
 
 // GROUP 0: D2V9 and D3V19; GROUP 1: D3V27 and D1V3 (separate translation units)
@@ -818,8 +832,7 @@ constexpr size_t kAdjSmemBudget = 200 * 1024;
 
 template <class L, class S, int FORCE, bool EF, bool WIN, int RS, int MODE, bool LMU = false>
 int launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
-                 const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
-                 const KParams& p, cudaStream_t s) {
+                 const float* w_rho, const float* w_j, float* gE, double* slots, const KParams& p, cudaStream_t s) {
     if (!p.rorder || (RS && RS != p.seglen) || (MODE == kExactRow && RS != p.nx) || (MODE == kSegment) != (p.nseg > 1))
         return 0;
     const int gcapP = dev::window_cap(p.max_row_links, S::kBytes);
@@ -841,8 +854,8 @@ int launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const uin
     // persistent grid: co-resident blocks per SM x SMs
     int blocks = staged_shape((const void*)kern, p.seglen, smem_ref, kAdjSmemBudget, threads).blocks;
     const int units = p.ny * p.nz * p.nseg;
-    if (blocks > units) blocks = units;
-    if (blocks <= 0 || blocks > slot_blocks) return 0;
+    blocks = (int)std::min<int64_t>(blocks, std::min<int64_t>(units, slot_blocks(p)));
+    if (blocks <= 0) return 0;
     kern<<<blocks, threads, smem, s>>>((const typename S::T*)P, lam_in, lam_out, Ef, w_rho, w_j, gE, slots,
                                        gcapP, gcapL, p);
     return route(kStaged, MODE, RS);
@@ -851,38 +864,37 @@ int launch_rows_rs(const void* P, const float* lam_in, float* lam_out, const uin
 // Rows or segments at a run-time stride.
 template <class L, class S, int FORCE, bool EF, bool WIN, bool LMU = false>
 int launch_rows_any(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
-                     const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
-                     const KParams& p, cudaStream_t s) {
+                     const float* w_rho, const float* w_j, float* gE, double* slots, const KParams& p,
+                     cudaStream_t s) {
     return p.nseg > 1 ? launch_rows_rs<L, S, FORCE, EF, WIN, 0, kSegment, LMU>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j,
-                                                                               gE, slots, slot_blocks, p, s)
+                                                                               gE, slots, p, s)
                       : launch_rows_rs<L, S, FORCE, EF, WIN, 0, kWholeRow, LMU>(P, lam_in, lam_out, nbr, Ef, w_rho,
-                                                                                w_j, gE, slots, slot_blocks, p, s);
+                                                                                w_j, gE, slots, p, s);
 }
 
 // The shared-memory row stride is a compile-time constant for the usual units,
 // as in the step kernel.
 template <class L, class S, int FORCE, bool EF, bool WIN>
 int launch_rows(const void* P, const float* lam_in, float* lam_out, const uint32_t* nbr, const float* Ef,
-                 const float* w_rho, const float* w_j, float* gE, double* slots, int64_t slot_blocks,
-                 const KParams& p, cudaStream_t s) {
+                 const float* w_rho, const float* w_j, float* gE, double* slots, const KParams& p,
+                 cudaStream_t s) {
     // the compile-time strides only for the benchmarked lattices (D2V9, D3V19)
     constexpr bool kFixed = L::Q == 9 || L::Q == 19;
     if constexpr (kFixed) {
         constexpr int kSeg = segment_columns<L>();
         if (p.nseg > 1 && p.seglen == kSeg)
             return launch_rows_rs<L, S, FORCE, EF, WIN, kSeg, kSegment>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,
-                                                                        slots, slot_blocks, p, s);
+                                                                        slots, p, s);
         if (p.nseg == 1 && p.nx == 256)
             return launch_rows_rs<L, S, FORCE, EF, WIN, 256, kExactRow>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,
-                                                                        slots, slot_blocks, p, s);
+                                                                        slots, p, s);
         if constexpr (whole_row<L, S>(512)) {
             if (p.nseg == 1 && p.nx == 512)
                 return launch_rows_rs<L, S, FORCE, EF, WIN, 512, kExactRow>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j,
-                                                                            gE, slots, slot_blocks, p, s);
+                                                                            gE, slots, p, s);
         }
     }
-    return launch_rows_any<L, S, FORCE, EF, WIN>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots, slot_blocks, p,
-                                                 s);
+    return launch_rows_any<L, S, FORCE, EF, WIN>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots, p, s);
 }
 
 // Launchers for one storage type (instantiated in one translation unit per
@@ -904,7 +916,7 @@ int step_storage(int vel, int force, bool efield, bool in_window, const void* P,
                  float* lam_out, const uint32_t* nbr, const float* Ef, const float* w_rho, const float* w_j,
                  float* gE, double* slots, const KParams& p, cudaStream_t s) {
     Launch l = grid_of(p);
-    const int64_t slot_blocks = strided_blocks(p);
+    const unsigned blocks = (unsigned)strided_blocks(p);
     return dispatch_lattice<GROUP>(vel, [&](auto lat) {
         using L = decltype(lat);
         const auto* Pt = (const typename S::T*)P;
@@ -916,16 +928,15 @@ int step_storage(int vel, int force, bool efield, bool in_window, const void* P,
         int staged;                                                                                           \
         if constexpr (GROUP == 2)                                                                             \
             staged = launch_rows_any<L, S, F, EFV, W, true>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,      \
-                                                            slots, slot_blocks, p, s);                        \
+                                                            slots, p, s);                                     \
         else                                                                                                  \
-            staged = launch_rows<L, S, F, EFV, W>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots,         \
-                                                  slot_blocks, p, s);                                         \
+            staged = launch_rows<L, S, F, EFV, W>(P, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots, p, s);  \
         if (staged)                                                                                           \
             done = staged;                                                                                    \
         else                                                                                                  \
             k_adjoint_step<L, S, F, EFV, W>                                                                   \
-                <<<(unsigned)slot_blocks, l.block, 0, s>>>(Pt, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE,      \
-                                                           slots, (int)l.grid.y, p);                          \
+                <<<blocks, l.block, 0, s>>>(Pt, lam_in, lam_out, nbr, Ef, w_rho, w_j, gE, slots,              \
+                                            (int)l.grid.y, p);                                                \
     } while (0)
         if (force == LBM_FORCE_SHIFT) {
             if (efield) {

@@ -179,6 +179,9 @@ REVERSE = [("D3V19", (2, 3, 256), ("staged", "exact", 256)), ("D3V19", (2, 3, 25
            ("D3V19", (2, 3, 512), ("staged", "segments", 256)), ("D2V9", (3, 256), ("staged", "exact", 256)),
            ("D2V9", (3, 512), ("staged", "exact", 512)), ("D2V9", (2, 1500), ("staged", "segments", 512)),
            ("D3V27", (2, 3, 256), ("staged", "rows", 0)), ("D3V27", (2, 3, 305), ("staged", "segments", 0)),
+           # narrow rows in numbers: more than eight blocks are resident per SM
+           ("D2V9", (2048, 64), ("staged", "rows", 0)), ("D3V19", (64, 64, 32), ("staged", "rows", 0)),
+           ("D2V9", (8200, 40), ("staged", "rows", 0)),
            ("D3V19", (4, 5, 31), ("general", None, 0)), ("D3V27", (4, 5, 30), ("general", None, 0)),
            ("D1V3", (31,), ("general", None, 0)), ("D2V9", (9, 31), ("general", None, 0))]
 
