@@ -13,16 +13,17 @@ The start state waits for backward() in device memory (LBM.snapshot).  Through
 host memory (LBM.save_state: a copy each way and a checksum byte by byte) it
 cost more than both sweeps: of 97 ms for 100 steps of 1024^2 D2V9 FP32 cells
 and their gradient, about 85.  Where the device has no room, for the copy or
-for the adjoint's buffers beside it, the host keeps it as before.
+for what backward() and lbm_adjoint allocate beside it, the host keeps it as
+before.
 
 Two effects of backward() that a caller should know:
   - the incoming FP64 gradient is passed to lbm_adjoint as FP32 per-cell loss
     weights (w_rho, w_j), so it is rounded to FP32 (relative 6e-8) before the
     reverse sweep; the sweep itself accumulates the parameter gradients in
     FP64;
-  - the simulation is left at the restored start state (the state before
-    forward() ran), not at step t_end: a caller that wants to step on from
-    t_end after backward() must save that state after forward() and load it.
+  - the sweep starts from the restored start state (the state before forward()
+    ran) and leaves the simulation at step t_end, as forward() did: a caller
+    that has stepped on in between must save that state and load it.
 """
 from __future__ import annotations
 
@@ -43,6 +44,17 @@ def _bring_back(sim, state):
         sim.load_state(state)
     else:
         sim.restore(state)
+
+
+def _reverse(ctx, g):
+    """lbm_adjoint from the restored start state: dL/dE(x) in FP32 and the other gradients."""
+    sim = ctx.sim
+    dev = torch.device("cuda", torch.cuda.current_device())
+    w_rho = torch.full((sim.N,), g[0], dtype=torch.float32, device=dev)
+    w_j = torch.tensor(g[1: 1 + sim.D], dtype=torch.float32, device=dev).repeat_interleave(sim.N)
+    dE = torch.empty(sim.D * sim.N, dtype=torch.float64, device=dev)
+    res = sim.adjoint(ctx.t[0], ctx.t[1], w_rho, w_j, ctx.t[2], dL_dE=dE)
+    return dE.view(ctx.shape).to(torch.float32), res
 
 
 class WindowCurrent(torch.autograd.Function):
@@ -66,24 +78,20 @@ class WindowCurrent(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, grad):
-        sim = ctx.sim
-        _bring_back(sim, ctx.state)
         g = grad.detach().double().cpu().tolist()
-        dev = torch.device("cuda", torch.cuda.current_device())
-        w_rho = torch.full((sim.N,), g[0], dtype=torch.float32, device=dev)
-        w_j = torch.tensor(g[1: 1 + sim.D], dtype=torch.float32, device=dev).repeat_interleave(sim.N)
-        dE = torch.empty(sim.D * sim.N, dtype=torch.float64, device=dev)
+        _bring_back(ctx.sim, ctx.state)
+        got = None
         try:
-            res = sim.adjoint(ctx.t[0], ctx.t[1], w_rho, w_j, ctx.t[2], dL_dE=dE)
-        except _lib.LBMError as e:
-            if e.status != _lib.LBM_ERR_OOM or isinstance(ctx.state, bytes):
+            got = _reverse(ctx, g)
+        except (torch.cuda.OutOfMemoryError, _lib.LBMError) as e:
+            if isinstance(ctx.state, bytes) or getattr(e, "status", _lib.LBM_ERR_OOM) != _lib.LBM_ERR_OOM:
                 raise
-            # once more with the start state on the host
-            _bring_back(sim, ctx.state)
-            ctx.state = sim.save_state()
+        if got is None:  # once more with the start state on the host (the failed try's tensors are gone here)
+            _bring_back(ctx.sim, ctx.state)
+            ctx.state = ctx.sim.save_state()
             torch.cuda.empty_cache()
-            res = sim.adjoint(ctx.t[0], ctx.t[1], w_rho, w_j, ctx.t[2], dL_dE=dE)
-        gE = dE.view(ctx.shape).to(torch.float32)
+            got = _reverse(ctx, g)
+        gE, res = got
         gB = torch.tensor(res["dL_dB"], dtype=ctx.B_dtype, device=ctx.B_dev)
         gtau = torch.tensor(res["dL_dtau"], dtype=torch.float64, device=ctx.tau_dev)
         return gE, gB, gtau, None, None, None, None
