@@ -399,6 +399,8 @@ int launch_build_neighbors(int vel, const uint8_t* mask, uint32_t* nbr, unsigned
 int launch_wait_probe(int* status, uint32_t limit, cudaStream_t s);
 // FP32 field in the populations' slot layout -> direction-major out[a * N + cell].
 int launch_unslot(int vel, const float* in, float* out, const KParams& p, cudaStream_t s);
+// A state's populations (units) to or from whole rows of nx columns, slot by slot.
+int launch_pack_rows(int storage, int Q, void* units, void* rows, bool pack, const KParams& p, cudaStream_t s);
 // Per-unit cell order (fluid cells first) for the row-staged kernels.
 int launch_build_row_order(const uint32_t* nbr, uint16_t* rorder, const KParams& p, cudaStream_t s);
 // Per-link descriptors (link_desc; needs lbase).
