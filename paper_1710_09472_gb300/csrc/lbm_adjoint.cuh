@@ -799,8 +799,8 @@ inline int64_t strided_blocks(const KParams& p) {
 // have 12 to 21 staged blocks resident per SM.  Boxes of many units take up to 16
 // (us per forward and reverse step: D2V9 FP32 64 x 16384 77.5, with eight 82.3, on
 // the general kernel 97.5; D3V19 FP16 32 x 128 x 128 74.4, 88.9, 110.7); boxes whose
-// blocks come round a few times only take eight (64 x 2048 27.7, with 16 30.2;
-// 64 x 4096 35.7 and 36.8).  The line lies between the measured 4096 and 16384 units.
+// blocks come round once or twice take eight (64 x 2048 27.7, with 16 30.2; at 64 x
+// 4096 both 36 to 37).  The line lies between the measured 4096 and 16384 units.
 inline int64_t slot_blocks(const KParams& p) {
     const Launch l = grid_of(p);
     const int64_t units = (int64_t)p.ny * p.nz * p.nseg;

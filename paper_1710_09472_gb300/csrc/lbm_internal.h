@@ -181,23 +181,6 @@ __host__ __device__ constexpr int key_count(int k) {
         return s;
     }
 }
-// slot(a) for a direction known only at run time: 5 bits per direction,
-// directions 12 k .. 12 k + 11 in word k
-template <class L>
-__host__ __device__ constexpr unsigned long long packed_slots(int word) {
-    unsigned long long v = 0;
-    for (int a = 12 * word; a < L::Q && a < 12 * (word + 1); ++a)
-        v |= (unsigned long long)pop_slot_calc<L>(a) << (5 * (a - 12 * word));
-    return v;
-}
-template <class L>
-__host__ __device__ __forceinline__ int slot_of(int a) {
-    constexpr unsigned long long w0 = packed_slots<L>(0), w1 = packed_slots<L>(1), w2 = packed_slots<L>(2);
-    if constexpr (L::Q <= 24)
-        return (int)((a < 12 ? (w0 >> (5 * a)) : (w1 >> (5 * (a - 12)))) & 31ull);
-    else
-        return (int)((a < 12 ? (w0 >> (5 * a)) : (a < 24 ? (w1 >> (5 * (a - 12))) : (w2 >> (5 * (a - 24))))) & 31ull);
-}
 
 // ---------------------------------------------------------------------------
 // Storage of the deviation h_a = f_a - rho0 w_a / I_0.  The kernels work in

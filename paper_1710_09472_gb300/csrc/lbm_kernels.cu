@@ -381,8 +381,9 @@ __global__ void __launch_bounds__(256) k_moments_rows(const typename S::T* __res
 }
 
 // Launches it where the context has units, two stages fit the step kernel's
-// budget and there are units for every SM; returns the blocks, 0 where it does
-// not run.
+// budget and there are units for every SM (staged / general, us: D2V9 BF16 4096 x
+// 8, 64 units, 2.69 / 2.02; D3V19 FP16 256 x 10 x 15, 150 units, 2.49 / 2.41);
+// returns the blocks, 0 where it does not run.
 template <class L, class S, bool TOTALS>
 int64_t launch_moments_rows(const void* pop, float* rho, float* j, double* partials, int64_t most, const KParams& p,
                             cudaStream_t s) {

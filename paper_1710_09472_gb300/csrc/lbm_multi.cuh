@@ -14,8 +14,8 @@
 //
 // What bounds it: the serial chain of a collision (about 0.6 us) plus the
 // barrier while a block has a warp or two per scheduler, the issue slots of 16
-// SMs beyond that: 0.9 us a step at 32 x 64 (D2V9 FP32), 4.0 us at 4096 x 8
-// (D2V9 BF16).
+// SMs beyond that: 0.9 us a step at 32 x 64 (D2V9 FP32); 4.0 us at 4096 x 8 (D2V9
+// BF16), measured without the limit that follows, which sends that box elsewhere.
 //
 // Beyond kClusterWork populations (where 16 SMs take as long as the other
 // kernel's barrier costs) a cooperative grid with a thread for every cell does
@@ -36,12 +36,13 @@ namespace multik {
 using dev::Cell;
 
 constexpr int kClusterMax = 16;  // the non-portable limit
-constexpr size_t kSmemMax = 220 * 1024;
+constexpr size_t kSmemMax = 128 * 1024;  // of a block of the cluster (see kClusterWork)
 constexpr uint32_t kNoCell = 0xFFFFFFFFu;
 
 // Populations up to which the cluster is the faster of the two.  Its step grows
-// with the box (0.87 us at 2048 cells of D2V9, 3.97 us at 32768), the grid's
-// hardly does (2.36 us at 32768): they meet near 16384 cells.
+// with the box (0.87 us at 2048 cells of D2V9; 3.97 us at 32768, without this
+// limit), the grid's hardly does (2.36 us at 32768): they meet near 16384 cells.
+// 16 blocks then need 120 KB of shared memory each at most.
 constexpr int64_t kClusterWork = 16384 * 9;
 // Threads per block: the FP32 collision of the larger lattices needs more than
 // 64 registers.  The grid has one block per SM.
@@ -271,7 +272,7 @@ Plan plan_of(const KParams& p) {
     while (blocks < kClusterMax && p.N > (int64_t)blocks * 128) blocks *= 2;
     const int64_t cpc = ((p.N + blocks - 1) / blocks + 31) / 32 * 32;
     const size_t smem = (size_t)L::Q * (size_t)cpc * (2 * S::kBytes + 4);
-    if (smem > kSmemMax || p.N * L::Q > kClusterWork) return {0, 0, 0};
+    if (p.N * L::Q > kClusterWork) return {0, 0, 0};
     return {blocks, (int)cpc, smem};
 }
 

@@ -796,8 +796,10 @@ int launch_rows(const S*, const void* fin, void* fout, const uint32_t* nbr, cons
     const int units = p.ny * p.nz * p.nseg;
     // Fewer units than SMs: most of the chip would idle while each block runs its
     // chain of copy, wait and two barriers once; the general kernel spreads the
-    // cells over more blocks (4096 x 8 cells of D2V9 BF16, 128 units: 6.2 us a
-    // step staged, below the 4.1 us that a launch takes the host otherwise).
+    // cells over more blocks.  Single steps from a graph, staged / general, us:
+    // D2V9 BF16 4096 x 8 (64 units) 3.76 / 2.65; D2V9 FP32 256 x 128 2.83 / 2.73,
+    // 1024 x 70 (140) 4.18 / 3.80; D3V19 FP16 256 x 8 x 8 3.53 / 3.00, 256 x 10 x 15
+    // (150) 3.55 / 3.48, 400 x 10 x 15 (150) 3.68 / 4.65.
     if (units < sh.sms) return 0;
     kern<<<blocks < units ? blocks : units, threads, smem, s>>>((const T*)fin, (T*)fout, Ef, gcap, dcap, p);
     return route(kStaged, MODE, RS);
@@ -811,11 +813,11 @@ int launch_one(const void* fin, void* fout, const uint32_t* nbr, const float* Ef
     using T = typename S::T;
     const S* tag = nullptr;
     // Compile-time strides: rows of 256 and 512 cells of the benchmarked lattices
-    // (D2V9, D3V19), their usual segments, 256 for 16-bit D3V27, and for D3V19 rows
-    // padded to 256.  A run-time stride costs a fifth of the step (256^3 D3V27
-    // FP16, 10 steps and the fields: 4.33 against 3.63 ms); other widths take it, to
-    // keep the instantiations few (the nearest rounding of 16-bit storage too, but
-    // for the exact rows).  Rows and segments are compiled apart: the
+    // (D2V9, D3V19), their usual segments, 256 for 16-bit D3V27 and for the local-mu
+    // model, and for D3V19 rows padded to 256.  A run-time stride costs a fifth of the
+    // step (256^3 D3V27 FP16, 10 steps and the fields: 4.33 against 3.63 ms); other
+    // widths take it, to keep the instantiations few (the nearest rounding of 16-bit
+    // storage too, but for the exact rows).  Rows and segments are compiled apart: the
     // halo of segments costs whole rows another tenth (250 x 128 x 128 D3V19 FP16,
     // 20 steps and the fields: 1.52 against 1.40 ms).
     auto rows = [&](auto rs, auto mode, auto lmu) {

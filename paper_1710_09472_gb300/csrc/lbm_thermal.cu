@@ -418,10 +418,12 @@ __global__ void __launch_bounds__(kTBlock) k_thermal_step(const typename S::T* _
     }
 }
 
-// The same for the start state, in plain expressions: their contraction is left
-// to the compiler, as it was when t_equilibrium was written so too, and start
-// states keep their bits (t_equilibrium's explicit order is the compiler's own
-// choice in the step kernel, which differs for orders 2 and 3).
+// The same for the start state, in plain expressions whose contraction is left to
+// the compiler, as t_equilibrium was before it was written for pairs of cells: so
+// start states kept their bits (compared on the GPU over 1 to 2^20 cells, orders 2
+// to 4, D1V5a and D1V7, the three storages).  Stepped states differ from the
+// earlier ones by roundings; their distance from 64 bits is the same to 1 %.
+// The two are one formula: a change to one is a change to the other.
 template <int Q, bool kLo>
 __device__ __forceinline__ void t_start_equilibrium(const TParams& p, float drho, float rho, float us, float dth,
                                                     float* heq) {
