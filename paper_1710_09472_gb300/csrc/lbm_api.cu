@@ -304,7 +304,10 @@ void ws_release(lbm_ctx* c) {
 // what a compile-time stride gains; else equal ones of that many columns at
 // most.  As whole rows, D2V9 FP32 rows of 1024 cells kept one block of eight
 // warps per SM: 27.6 us per step at 1024^2 (20.9 in segments), and no reverse
-// step but the general one (95 us; 38).
+// step but the general one (95 us; 38).  The rule looks at the forward stages only:
+// 16-bit D2V9 rows of about 1250 to 1816 cells stay whole and run the general
+// reverse step, whose FP32 adjoint rows do not fit (512 x 1816 FP16: 17 us a
+// forward step, 592 us for six steps and their gradient).
 void set_units(lbm_ctx* c) {
     const int nx = (int)c->nx;
     c->nseg = 1;
