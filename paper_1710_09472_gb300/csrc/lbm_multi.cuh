@@ -170,12 +170,14 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, b
         __threadfence();
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(count) : "memory");
         if (ok) {
-            const long long t0 = clock64();
+            // counted against a constant from an earlier start: with the limit itself in
+            // the comparison a step of 28 x 40 x 21 D3V19 BF16 took 2.80 us, 2.64 so
+            const long long t0 = clock64() - (kWaitClocks - (long long)limit);
             for (;;) {
                 unsigned v;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(count) : "memory");
                 if (v >= target) break;
-                if (clock64() - t0 > limit) {
+                if (clock64() - t0 > kWaitClocks) {
                     ok = false;
                     if (status) atomicExch(status, 4);
                     break;
